@@ -367,7 +367,9 @@ __device__ __forceinline__ void xpass_body(const LOC &loc, int64_t tiles, int st
       const int64_t m0 = T.m0;
       const int cg = T.cg;
       const int64_t row_end = p.row0 + p.rows;
-      const uint32_t tacc = tbase + ((uint32_t)(q * 32) << 16) + 2 * XN + h * half;
+      // a column region of its own for each warp whatever the tile's xn: in a
+      // grouped launch the other warp of the lane quarter may be a tile ahead
+      const uint32_t tacc = tbase + ((uint32_t)(q * 32) << 16) + 2 * XN + h * HALF;
       float acc[AREG];
 #pragma unroll
       for (int c = 0; c < AREG; ++c) acc[c] = 0.0f;
