@@ -197,8 +197,9 @@ int dgemm(bool transA, bool transB, int M, int N, int K, double alpha, const dou
 // In-place lower Cholesky of an n x n SPD matrix (upper part zeroed).
 int cholesky_lower(Ctx *ctx, double *A, int n, cudaStream_t s);
 // In-place X := L^{-1} X for L n x n lower, X n x ncol with leading dim ld.
+// With enough scratch (device memory, overwritten) on the tensor cores.
 int trsm_lower_left(Ctx *ctx, const double *L, int n, double *X, int64_t ncol, int64_t ld,
-                    cudaStream_t s);
+                    void *scratch, size_t scratch_bytes, cudaStream_t s);
 
 }  // namespace bqc
 

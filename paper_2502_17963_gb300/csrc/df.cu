@@ -19,6 +19,7 @@
 #include "bqc_internal.h"
 #include "df_internal.h"
 #include "gemm64.cuh"
+#include "oz.h"
 
 namespace bqc {
 
@@ -462,11 +463,136 @@ int group_jpass(Df *const *dfs, double *const *J, int n, cudaStream_t s) {
   return BQC_OK;
 }
 
+// FP64 X pass and K on the tensor cores (oz.cu), over chunks of pc aux
+// functions.  The handle's X buffer (Naux N nocc doubles) is the scratch: a
+// chunk's sliced B, its X (FP64), its sliced X, and the K partials.
+struct OzJkPlan {
+  int pc = 0;               // aux functions per chunk (0: does not fit)
+  int ns = 0;               // splits of the K contraction of a chunk
+  size_t cs, ce, bs, be, x, xs, xe, kp, total;  // offsets, and the bytes used
+};
+
+static OzJkPlan oz_jk_layout(int n, int no, int pc, int ns) {
+  OzJkPlan p;
+  p.pc = pc;
+  p.ns = oz_splits(pc * no, ns);
+  size_t o = 0;
+  auto take = [&o](size_t b) {
+    const size_t at = o;
+    o += oz_align(b);
+    return at;
+  };
+  p.kp = take((size_t)p.ns * n * n * 8);
+  p.cs = take(oz_slice_bytes(no, n));
+  p.ce = take(oz_exp_bytes(no, 1));
+  p.bs = take(oz_slice_bytes((int64_t)pc * n, n));
+  p.be = take(oz_exp_bytes((int64_t)pc * n, 1));
+  p.x = take((size_t)pc * n * no * 8);
+  p.xs = take(oz_slice_bytes(n, pc * no));
+  p.xe = take(oz_exp_bytes(n, p.ns));
+  p.total = o;
+  return p;
+}
+
+static OzJkPlan oz_jk_plan(int n, int naux, int no, size_t bytes) {
+  // K splits: the count whose tiles fill whole waves best, splits of at least 256
+  const int64_t tiles = oz_tiles(n, n, true);
+  const int nsm = sm_count();
+  OzJkPlan best;
+  for (int chunks = 1; chunks <= 64 && chunks <= naux; ++chunks) {
+    const int pc = (naux + chunks - 1) / chunks;
+    int ns = 1;
+    double eff = 0.0;
+    for (int c = 1; c <= 2 * nsm && (c == 1 || c * 256 <= pc * no); ++c) {
+      const int64_t items = tiles * c;
+      const double e = (double)items / ((double)((items + nsm - 1) / nsm) * nsm);
+      if (e > eff + 1e-3) {
+        eff = e;
+        ns = c;
+      }
+      if (items >= 2 * nsm) break;
+    }
+    OzJkPlan p = oz_jk_layout(n, no, pc, ns);
+    if (p.total <= bytes) return p;
+  }
+  return best;
+}
+
+static int jk_fp64_oz(Df *df, const OzJkPlan &p, const double *C, double *J, double *K,
+                      cudaStream_t s) {
+  const int n = df->basis->nbf, naux = df->naux_loc, no = df->basis->nocc;
+  char *scr = df->X64.as<char>();
+  double *X = reinterpret_cast<double *>(scr + p.x), *kp = reinterpret_cast<double *>(scr + p.kp);
+  auto ints = [scr](size_t at) { return reinterpret_cast<int *>(scr + at); };
+  df->mark(0, s);
+  df->mark(1, s);
+  OzSrc c;  // C^T: rows i, contraction nu
+  c.kind = kOzCols;
+  c.p = C;
+  c.rows = no;
+  c.K = n;
+  c.ld = no;
+  BQC_TRY(oz_slice(c, oz_kblocks(n), scr + p.cs, ints(p.ce), s));
+  OzOperand oc;
+  oc.slices = scr + p.cs;
+  oc.exps = ints(p.ce);
+  oc.rows = no;
+  oc.K = n;
+  const int ns = p.ns;
+  for (int P0 = 0; P0 < naux; P0 += p.pc) {
+    const int np = std::min(p.pc, naux - P0);
+    OzSrc b;  // rows (P, mu), contraction nu
+    b.kind = kOzSym;
+    b.p = df->B64.as<double>() + (int64_t)P0 * df->npair;
+    b.rows = (int64_t)np * n;
+    b.n2 = n;
+    b.sz = df->npair;
+    b.K = n;
+    BQC_TRY(oz_slice(b, oz_kblocks(n), scr + p.bs, ints(p.be), s));
+    OzOperand ob;
+    ob.slices = scr + p.bs;
+    ob.exps = ints(p.be);
+    ob.rows = b.rows;
+    ob.K = n;
+    BQC_TRY(oz_gemm(oc, ob, oz_kblocks(n), 1, 0, X, no, 0, 0, df->ctx->flag, s));
+    k_wdot<<<np, 256, 0, s>>>(X, C, (int64_t)n * no, df->w.as<double>() + P0);
+    BQC_LAUNCH_CHECK();
+    // K partials: rows mu, contraction (P, i); a short last chunk may have
+    // fewer splits than the others, and adds to the first ones
+    OzSrc x;
+    x.kind = kOzRows;
+    x.p = X;
+    x.rows = n;
+    x.K = np * no;
+    x.k2 = no;
+    x.s1 = (int64_t)n * no;
+    x.ld = no;
+    const int kb = oz_split_kb(x.K, ns);
+    BQC_TRY(oz_slice(x, kb, scr + p.xs, ints(p.xe), s));
+    OzOperand ox;
+    ox.slices = scr + p.xs;
+    ox.exps = ints(p.xe);
+    ox.rows = n;
+    ox.K = x.K;
+    BQC_TRY(oz_gemm(ox, ox, kb, 1, P0 > 0, kp, n, (int64_t)n * n, 1, df->ctx->flag, s));
+  }
+  df->mark(2, s);
+  BQC_TRY(jpass_fp64(df, J, s));
+  df->mark(3, s);
+  BQC_TRY(oz_sym_reduce(kp, ns, (int64_t)n * n, n, n, K, s));
+  df->mark(4, s);
+  return BQC_OK;
+}
+
 int jk_fp64_stored(Df *df, const double *C, double *J, double *K, cudaStream_t s) {
   const Basis *b = df->basis;
   const int n = b->nbf, naux = df->naux_loc, no = b->nocc;
   const int64_t npair = df->npair;
   double *X = df->X64.as<double>();
+  if (n >= 64) {
+    const OzJkPlan p = oz_jk_plan(n, naux, no, df->X64.n);
+    if (p.pc) return jk_fp64_oz(df, p, C, J, K, s);
+  }
   df->mark(0, s);
   df->mark(1, s);
   // X_P = Bsym_P C  (batched over P)
@@ -638,6 +764,8 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
   if ((st = df->w.alloc(ctx, (size_t)naux * 8)) != BQC_OK) return fail(st);
   if (mode == BQC_DF_STORED) {
     df->Vdiag.release();  // metric only needed for the screening plan
+    // the FP64 X buffer, first used as the metric solve's scratch
+    if ((st = df->X64.alloc(ctx, (size_t)df->naux_loc * n * no * 8)) != BQC_OK) return fail(st);
     if (!shard) {
       if ((st = df->B64.alloc(ctx, (size_t)naux * npair * 8)) != BQC_OK) return fail(st);
       if (cudaMemsetAsync(df->B64.p, 0, (size_t)naux * npair * 8, s) != cudaSuccess)
@@ -646,7 +774,7 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
           BQC_OK)
         return fail(st);
       if ((st = trsm_lower_left(ctx, df->L.as<double>(), naux, df->B64.as<double>(), npair,
-                                npair, s)) != BQC_OK)
+                                npair, df->X64.p, df->X64.n, s)) != BQC_OK)
         return fail(st);
     } else {
       // B_P for P in [P0, P1) depends on (Q|mu nu) for every Q <= P (the
@@ -662,8 +790,8 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
       if (cudaMemcpy2DAsync(Lb.p, (size_t)P1 * 8, df->L.p, (size_t)naux * 8, (size_t)P1 * 8, P1,
                             cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return fail(BQC_E_CUDA);
-      if ((st = trsm_lower_left(ctx, Lb.as<double>(), P1, raw.as<double>(), npair, npair, s)) !=
-          BQC_OK)
+      if ((st = trsm_lower_left(ctx, Lb.as<double>(), P1, raw.as<double>(), npair, npair,
+                                df->X64.p, df->X64.n, s)) != BQC_OK)
         return fail(st);
       if ((st = df->B64.alloc(ctx, (size_t)(P1 - P0) * npair * 8)) != BQC_OK) return fail(st);
       if (cudaMemcpyAsync(df->B64.p, raw.as<double>() + (size_t)P0 * npair,
@@ -673,7 +801,6 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
       if (cudaStreamSynchronize(s) != cudaSuccess) return fail(BQC_E_CUDA);
     }
     const int nl = df->naux_loc;
-    if ((st = df->X64.alloc(ctx, (size_t)nl * n * no * 8)) != BQC_OK) return fail(st);
     if ((st = df->Jp.alloc(ctx, (size_t)jpass_split(npair, nl) * npair * 8)) != BQC_OK)
       return fail(st);
     if (o.keep_fp32 != BQC_SHADOW_NONE)

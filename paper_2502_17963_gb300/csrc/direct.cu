@@ -113,10 +113,11 @@ int direct_setup(Df *df, cudaStream_t s) {
   df->aux_block = std::max(1, std::min(df->opts.aux_block, naux));
   // L^{-1} (FP64), once
   BQC_TRY(df->Linv.alloc(ctx, (size_t)naux * naux * 8));
+  BQC_TRY(df->raw.alloc(ctx, (size_t)df->aux_block * df->npair * 8));
   k_identity<<<nb((int64_t)naux * naux), 256, 0, s>>>(df->Linv.as<double>(), naux);
   BQC_LAUNCH_CHECK();
-  BQC_TRY(trsm_lower_left(ctx, df->L.as<double>(), naux, df->Linv.as<double>(), naux, naux, s));
-  BQC_TRY(df->raw.alloc(ctx, (size_t)df->aux_block * df->npair * 8));
+  BQC_TRY(trsm_lower_left(ctx, df->L.as<double>(), naux, df->Linv.as<double>(), naux, naux,
+                          df->raw.p, df->raw.n, s));
   BQC_TRY(df->gamma.alloc(ctx, (size_t)naux * 8 * 2));
   BQC_TRY(df->D2.alloc(ctx, (size_t)df->npair * 8));
   BQC_TRY(df->Jp.alloc(ctx, (size_t)df->npair * 8));
@@ -191,7 +192,7 @@ int jk_direct(Df *df, const double *C, int prec, double *J, double *K, cudaStrea
     BQC_TRY(direct_mixed_finish(df, split, K, s));
   } else {
     BQC_TRY(trsm_lower_left(ctx, df->L.as<double>(), naux, df->Xraw.as<double>(),
-                            (int64_t)n * no, (int64_t)n * no, s));
+                            (int64_t)n * no, (int64_t)n * no, df->raw.p, df->raw.n, s));
     Gemm64Args k;
     k.M = n;
     k.N = n;

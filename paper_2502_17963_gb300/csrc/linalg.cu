@@ -10,9 +10,11 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "bqc_internal.h"
 #include "gemm64.cuh"
+#include "oz.h"
 
 namespace bqc {
 
@@ -157,10 +159,146 @@ __global__ void __launch_bounds__(128) k_trsm_diag(const double *L, int n, int k
   }
 }
 
+// Explicit inverses of the kNB x kNB diagonal blocks of L, out[block][kNB][kNB]
+// row-major with zeros above the diagonal (and past the end of a ragged last
+// block).  One block per diagonal block, one thread per column; column j of
+// the inverse lives in row j of the same shared array, right of the diagonal.
+__global__ void __launch_bounds__(kNB) k_tri_inv(const double *L, int n, double *out) {
+  __shared__ double a[kNB][kNB + 1];
+  __shared__ double dinv[kNB];
+  const int k0 = blockIdx.x * kNB, nb = min(kNB, n - k0), j = threadIdx.x;
+  for (int r = 0; r < nb; ++r)
+    if (j <= r) a[r][j] = L[(int64_t)(k0 + r) * n + k0 + j];
+  __syncthreads();
+  if (j < nb) dinv[j] = 1.0 / a[j][j];
+  __syncthreads();
+  if (j < nb)
+    for (int r = j + 1; r < nb; ++r) {
+      double v = -a[r][j] * dinv[j];
+      for (int l = j + 1; l < r; ++l) v = fma(-a[r][l], a[j][l], v);
+      a[j][r] = v * dinv[r];
+    }
+  __syncthreads();
+  double *o = out + (int64_t)blockIdx.x * kNB * kNB;
+  for (int r = 0; r < kNB; ++r) {
+    double v = 0.0;
+    if (r < nb && j < nb) v = j < r ? a[j][r] : (j == r ? dinv[r] : 0.0);
+    o[r * kNB + j] = v;
+  }
+}
+
+// The metric solve as tensor-core products (oz.cu): recursive halving,
+//   X_1 := L_11^{-1} X_1;  X_2 -= L_21 X_1;  X_2 := L_22^{-1} X_2,
+// down to 64-row diagonal blocks, which are multiplied by their explicit
+// inverses.  Every product reads sliced copies, so all of them run in place.
+// L's slices are made once; X is solved in column panels whose slices (half
+// of X's rows at the top of the recursion) fit the scratch.
+struct OzTrsmOp {
+  int r0, nr, k0, nk;  // X[r0 .. r0 + nr) from X[k0 .. k0 + nk); r0 == k0: diagonal block
+  size_t slices, exps;  // offsets of L's operand in the scratch
+};
+
+static void oz_trsm_ops(int n, int b0, int b1, std::vector<OzTrsmOp> &ops) {
+  const int r0 = b0 * kNB;
+  if (b1 - b0 == 1) {
+    const int nb = std::min(kNB, n - r0);
+    ops.push_back({r0, nb, r0, nb, 0, 0});
+    return;
+  }
+  const int mid = (b0 + b1 + 1) / 2, rm = mid * kNB;
+  oz_trsm_ops(n, b0, mid, ops);
+  ops.push_back({rm, std::min(n, b1 * kNB) - rm, r0, rm - r0, 0, 0});
+  oz_trsm_ops(n, mid, b1, ops);
+}
+
+// Columns of X a panel can hold in the scratch (0: not worth it).
+static int64_t oz_trsm_plan(int n, int64_t ncol, size_t bytes, std::vector<OzTrsmOp> &ops,
+                            size_t *inv, size_t *panel) {
+  const int nblk = (n + kNB - 1) / kNB;
+  oz_trsm_ops(n, 0, nblk, ops);
+  size_t off = 0;
+  int kmax = 0;
+  for (auto &o : ops) {
+    o.slices = off;
+    off += oz_slice_bytes(o.nr, o.nk);
+    o.exps = off;
+    off += oz_exp_bytes(o.nr, 1);
+    kmax = std::max(kmax, o.nk);
+  }
+  *inv = off;
+  off += oz_align((size_t)nblk * kNB * kNB * 8);
+  *panel = off;
+  if (off >= bytes) return 0;
+  const size_t per_col = (size_t)oz_kblocks(kmax) * kOzSlices * kOzKb * 2 + sizeof(int);
+  int64_t cols = (int64_t)((bytes - off) / per_col) - 512;  // alignment of the two arrays
+  if (cols >= ncol) return ncol;
+  cols = cols / 128 * 128;
+  if (cols < 16384) return 0;
+  const int64_t np = (ncol + cols - 1) / cols;  // equal panels
+  return std::min(cols, ((ncol + np - 1) / np + 127) / 128 * 128);
+}
+
+static int oz_trsm(Ctx *ctx, const double *L, int n, double *X, int64_t ncol, int64_t ld,
+                   const std::vector<OzTrsmOp> &ops, int64_t cols, size_t inv, size_t panel,
+                   char *scr, cudaStream_t s) {
+  const int nblk = (n + kNB - 1) / kNB;
+  double *li = reinterpret_cast<double *>(scr + inv);
+  k_tri_inv<<<(unsigned)nblk, kNB, 0, s>>>(L, n, li);
+  BQC_LAUNCH_CHECK();
+  for (const auto &o : ops) {
+    OzSrc a;
+    a.kind = kOzRows;
+    a.rows = o.nr;
+    a.K = o.nk;
+    if (o.r0 == o.k0) {
+      a.p = li + (int64_t)(o.r0 / kNB) * kNB * kNB;
+      a.ld = kNB;
+    } else {
+      a.p = L + (int64_t)o.r0 * n + o.k0;
+      a.ld = n;
+    }
+    BQC_TRY(oz_slice(a, oz_kblocks(o.nk), scr + o.slices, reinterpret_cast<int *>(scr + o.exps), s));
+  }
+  for (int64_t c0 = 0; c0 < ncol; c0 += cols) {
+    const int64_t nc = std::min(cols, ncol - c0);
+    for (const auto &o : ops) {
+      OzSrc x;
+      x.kind = kOzCols;
+      x.p = X + (int64_t)o.k0 * ld + c0;
+      x.rows = nc;
+      x.K = o.nk;
+      x.ld = ld;
+      void *xs = scr + panel;
+      int *xe = reinterpret_cast<int *>(scr + panel + oz_slice_bytes(nc, o.nk));
+      BQC_TRY(oz_slice(x, oz_kblocks(o.nk), xs, xe, s));
+      OzOperand A, B;
+      A.slices = xs;
+      A.exps = xe;
+      A.rows = nc;
+      A.K = o.nk;
+      B.slices = scr + o.slices;
+      B.exps = reinterpret_cast<int *>(scr + o.exps);
+      B.rows = o.nr;
+      B.K = o.nk;
+      const bool diag = o.r0 == o.k0;
+      BQC_TRY(oz_gemm(A, B, oz_kblocks(o.nk), diag ? 1 : -1, diag ? 0 : 1,
+                      X + (int64_t)o.r0 * ld + c0, ld, 0, 0, ctx->flag, s));
+    }
+  }
+  return BQC_OK;
+}
+
 int trsm_lower_left(Ctx *ctx, const double *L, int n, double *X, int64_t ncol, int64_t ld,
-                    cudaStream_t s) {
-  (void)ctx;
+                    void *scratch, size_t scratch_bytes, cudaStream_t s) {
   if (ncol <= 0) return BQC_OK;
+  if (scratch && n > kNB) {
+    std::vector<OzTrsmOp> ops;
+    size_t inv = 0, panel = 0;
+    const int64_t cols = oz_trsm_plan(n, ncol, scratch_bytes, ops, &inv, &panel);
+    if (cols > 0)
+      return oz_trsm(ctx, L, n, X, ncol, ld, ops, cols, inv, panel, static_cast<char *>(scratch),
+                     s);
+  }
   for (int k0 = 0; k0 < n; k0 += kNB) {
     const int nb = std::min(kNB, n - k0);
     k_trsm_diag<<<(unsigned)((ncol + 127) / 128), 128, 0, s>>>(L, n, k0, X, ncol, ld);

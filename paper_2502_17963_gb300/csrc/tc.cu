@@ -51,7 +51,8 @@ static PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
 // fp32 tensor map, rank 2 or 3, 128-byte swizzle; dims/box innermost first;
 // strides in bytes for dims 1.. (rank-1 entries).
 static int make_tmap(CUtensorMap *map, CUtensorMapDataType dtype, const void *base, int rank,
-                     const uint64_t *dims, const uint64_t *strides_bytes, const uint32_t *box);
+                     const uint64_t *dims, const uint64_t *strides_bytes, const uint32_t *box,
+                     CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B);
 
 int make_tmap_f32(CUtensorMap *map, const void *base, int rank, const uint64_t *dims,
                   const uint64_t *strides_bytes, const uint32_t *box) {
@@ -64,8 +65,16 @@ static int make_tmap_f16(CUtensorMap *map, const void *base, int rank, const uin
   return make_tmap(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, base, rank, dims, strides_bytes, box);
 }
 
+// the same with boxes of 32 elements (64 bytes) in the 64-byte swizzle.
+int make_tmap_f16_sw64(CUtensorMap *map, const void *base, int rank, const uint64_t *dims,
+                       const uint64_t *strides_bytes, const uint32_t *box) {
+  return make_tmap(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, base, rank, dims, strides_bytes, box,
+                   CU_TENSOR_MAP_SWIZZLE_64B);
+}
+
 static int make_tmap(CUtensorMap *map, CUtensorMapDataType dtype, const void *base, int rank,
-                     const uint64_t *dims, const uint64_t *strides_bytes, const uint32_t *box) {
+                     const uint64_t *dims, const uint64_t *strides_bytes, const uint32_t *box,
+                     CUtensorMapSwizzle swizzle) {
   auto enc = get_encode();
   if (!enc) {
     set_error("cuTensorMapEncodeTiled unavailable", __FILE__, __LINE__);
@@ -84,7 +93,7 @@ static int make_tmap(CUtensorMap *map, CUtensorMapDataType dtype, const void *ba
   }
   for (int i = 0; i < rank - 1; ++i) s[i] = strides_bytes[i];
   CUresult r = enc(map, dtype, (cuuint32_t)rank, const_cast<void *>(base),
-                   d, s, b, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                   d, s, b, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("cuTensorMapEncodeTiled failed", __FILE__, __LINE__);
