@@ -19,6 +19,7 @@
 #include "bqc_internal.h"
 #include "df_internal.h"
 #include "gemm64.cuh"
+#include "oz.h"
 
 namespace bqc {
 
@@ -80,60 +81,154 @@ static int mp2_block(int nocc, int nvir) {
   return std::max(1, std::min({bi, 16, nocc}));
 }
 
-// prec FP64: every GEMM on the DFMA path; MIXED_F16X3: the MO transform in
-// FP64, the pair blocks as split-FP16 tensor-core GEMMs (FP32 accumulation in
-// short chains, float-float drains, FP64 blocks), the energy in FP64.
+// X_P = B_P C_occ (into the handle's FP64 X buffer) and B_P,ia = sum_nu
+// X_P[nu][i] C[nu][no + a] -> Bt[P][i][a] on the DFMA path.
+static int mp2_transform_dfma(Df *df, const double *C, int nmo, double *Bt, cudaStream_t s) {
+  const int n = df->basis->nbf, naux = df->basis->naux, no = df->basis->nocc, nv = nmo - no;
+  Gemm64Args g;
+  g.M = n;
+  g.N = no;
+  g.K1 = 1;
+  g.K2 = n;
+  g.A = df->B64.as<double>();
+  g.bsA = df->npair;
+  g.B = C;
+  g.ldb = nmo;
+  g.C = df->X64.as<double>();
+  g.ldc = no;
+  g.bsC = (int64_t)n * no;
+  g.batch = naux;
+  BQC_TRY(launch_gemm64(kASym, false, g, s));
+  Gemm64Args t;
+  t.M = no;
+  t.N = nv;
+  t.K1 = 1;
+  t.K2 = n;
+  t.A = df->X64.as<double>();
+  t.lda = no;
+  t.bsA = (int64_t)n * no;
+  t.B = C + no;
+  t.ldb = nmo;
+  t.C = Bt;
+  t.ldc = nv;
+  t.bsC = (int64_t)no * nv;
+  t.batch = naux;
+  return launch_gemm64(kAT, false, t, s);
+}
+
+// The same as sliced tensor-core products (oz.cu), chunks of pc aux functions.
+// Scratch: the sliced C_occ^T and C_vir^T, then a chunk's sliced B (rows
+// (P, mu)) or X (rows (P, i)).
+static int mp2_transform_pc(int n, int naux, int no, int nv, size_t bytes) {
+  const size_t fixed = oz_slice_bytes(no, n) + oz_exp_bytes(no, 1) + oz_slice_bytes(nv, n) +
+                       oz_exp_bytes(nv, 1) + 4096;
+  const size_t row = (size_t)oz_kblocks(n) * kOzSlices * kOzKb * 2 + sizeof(int);
+  if (bytes <= fixed) return 0;
+  return (int)std::min<size_t>((bytes - fixed) / (row * n), (size_t)naux);
+}
+
+static int mp2_transform_oz(Df *df, const double *C, int nmo, double *Bt, char *scr, int pc,
+                            cudaStream_t s) {
+  const int n = df->basis->nbf, naux = df->basis->naux, no = df->basis->nocc, nv = nmo - no;
+  const int kb = oz_kblocks(n);
+  int *flag = df->ctx->flag;
+  double *X = df->X64.as<double>();
+  OzOperand oc[2];
+  for (int k = 0; k < 2; ++k) {
+    OzSrc c;
+    c.kind = kOzCols;
+    c.p = C + (k ? no : 0);
+    c.rows = k ? nv : no;
+    c.K = n;
+    c.ld = nmo;
+    oc[k].slices = scr;
+    int *e = reinterpret_cast<int *>(scr + oz_slice_bytes(c.rows, n));
+    oc[k].exps = e;
+    oc[k].rows = c.rows;
+    oc[k].K = n;
+    BQC_TRY(oz_slice(c, kb, scr, e, s));
+    scr += oz_slice_bytes(c.rows, n) + oz_exp_bytes(c.rows, 1);
+  }
+  for (int P0 = 0; P0 < naux; P0 += pc) {
+    const int np = std::min(pc, naux - P0);
+    for (int k = 0; k < 2; ++k) {
+      OzSrc b;
+      b.K = n;
+      if (k == 0) {
+        b.kind = kOzSym;
+        b.p = df->B64.as<double>() + (int64_t)P0 * df->npair;
+        b.n2 = n;
+        b.sz = df->npair;
+      } else {
+        b.kind = kOzCols;
+        b.p = X + (int64_t)P0 * n * no;
+        b.n2 = no;
+        b.sz = (int64_t)n * no;
+        b.ld = no;
+      }
+      b.rows = (int64_t)np * b.n2;
+      OzOperand ob;
+      ob.slices = scr;
+      int *e = reinterpret_cast<int *>(scr + oz_slice_bytes(b.rows, n));
+      ob.exps = e;
+      ob.rows = b.rows;
+      ob.K = n;
+      BQC_TRY(oz_slice(b, kb, scr, e, s));
+      BQC_TRY(oz_gemm(oc[k], ob, kb, 1, 0,
+                      k == 0 ? X + (int64_t)P0 * n * no : Bt + (int64_t)P0 * no * nv,
+                      k == 0 ? no : nv, 0, 0, flag, s));
+    }
+  }
+  return BQC_OK;
+}
+
+// prec FP64: the transform and the pair blocks V = B_ia^T B_jb as sliced
+// FP64-accurate tensor-core products; MIXED_F16X3: the pair blocks as
+// split-FP16 tensor-core GEMMs (FP32 accumulation in short chains, float-float
+// drains, FP64 blocks); the energy in FP64.  Without memory for the slices,
+// or below 64 functions, where a tile would be mostly padding, the DFMA GEMM.
 static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec, double *e2,
                    cudaStream_t s) {
   const Basis *b = df->basis;
   const int n = b->nbf, naux = b->naux, no = b->nocc, nv = nmo - no;
   Ctx *ctx = df->ctx;
-  DBuf Bt, V, ep, out;
+  DBuf Bt, V, ep, out, Ts;
   BQC_TRY(ep.alloc(ctx, (size_t)no * no * 8));
   BQC_TRY(out.alloc(ctx, 8));
   BQC_CUDA_TRY(cudaMemsetAsync(ep.p, 0, ep.n, s));
   if (nv > 0) {
-    // X_P = B_P C_occ (N x nocc per P), into the handle's FP64 X buffer
-    Gemm64Args g;
-    g.M = n;
-    g.N = no;
-    g.K1 = 1;
-    g.K2 = n;
-    g.A = df->B64.as<double>();
-    g.bsA = df->npair;
-    g.B = C;
-    g.ldb = nmo;
-    g.C = df->X64.as<double>();
-    g.ldc = no;
-    g.bsC = (int64_t)n * no;
-    g.batch = naux;
-    BQC_TRY(launch_gemm64(kASym, false, g, s));
-    // B_P,ia = sum_nu X_P[nu][i] C[nu][no + a]  ->  Bt[P][i][a]
-    BQC_TRY(Bt.alloc(ctx, (size_t)naux * no * nv * 8));
-    Gemm64Args t;
-    t.M = no;
-    t.N = nv;
-    t.K1 = 1;
-    t.K2 = n;
-    t.A = df->X64.as<double>();
-    t.lda = no;
-    t.bsA = (int64_t)n * no;
-    t.B = C + no;
-    t.ldb = nmo;
-    t.C = Bt.as<double>();
-    t.ldc = nv;
-    t.bsC = (int64_t)no * nv;
-    t.batch = naux;
-    BQC_TRY(launch_gemm64(kAT, false, t, s));
+    const int64_t Q = (int64_t)no * nv;
+    BQC_TRY(Bt.alloc(ctx, (size_t)naux * Q * 8));
+    const int bi = mp2_block(no, nv);
+    int pc = 0;
+    if (n >= 64 && Ts.alloc(ctx, oz_slice_bytes(Q, naux) + oz_exp_bytes(Q, 1)) == BQC_OK)
+      pc = mp2_transform_pc(n, naux, no, nv, Ts.n);
+    const bool oz = prec == BQC_PREC_FP64 && Ts.p;
+    if (pc)
+      BQC_TRY(mp2_transform_oz(df, C, nmo, Bt.as<double>(), Ts.as<char>(), pc, s));
+    else
+      BQC_TRY(mp2_transform_dfma(df, C, nmo, Bt.as<double>(), s));
     std::unique_ptr<Mp2Tc, Mp2TcDeleter> tcs;
     if (prec == BQC_PREC_MIXED_F16X3) {
+      if (Ts.p) {
+        BQC_CUDA_TRY(cudaStreamSynchronize(s));
+        Ts.release();
+      }
       BQC_TRY(mp2_tc_setup(ctx, Bt.as<double>(), naux, no, nv, ctx->flag, tcs, s));
       BQC_CUDA_TRY(cudaStreamSynchronize(s));
       Bt.release();  // the split operand replaces it
     }
-    const int bi = mp2_block(no, nv);
+    int *te = oz ? reinterpret_cast<int *>(Ts.as<char>() + oz_slice_bytes(Q, naux)) : nullptr;
+    if (oz) {  // rows (i, a), contraction P
+      OzSrc q;
+      q.kind = kOzCols;
+      q.p = Bt.as<double>();
+      q.rows = Q;
+      q.K = naux;
+      q.ld = Q;
+      BQC_TRY(oz_slice(q, oz_kblocks(naux), Ts.p, te, s));
+    }
     BQC_TRY(V.alloc(ctx, (size_t)bi * nv * bi * nv * 8));
-    const int64_t ldt = (int64_t)no * nv;
     for (int i0 = 0; i0 < no; i0 += bi) {
       const int ni = std::min(bi, no - i0);
       for (int j0 = 0; j0 <= i0; j0 += bi) {
@@ -142,23 +237,32 @@ static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec
         if (tcs) {
           BQC_TRY(mp2_tc_block(tcs.get(), nv, i0, ni, j0, nj, V.as<double>(), (int64_t)nj * nv,
                                ctx->flag, s));
-          k_mp2_pairs<<<dim3((unsigned)ni, (unsigned)nj), 256, 0, s>>>(
-              V.as<double>(), (int64_t)nj * nv, i0, j0, nv, eps, no, ep.as<double>());
-          BQC_LAUNCH_CHECK();
-          continue;
+        } else if (oz) {
+          auto rows = [&](int o0, int cnt) {
+            OzOperand r;
+            r.slices = Ts.as<char>() + (int64_t)o0 * nv * kOzKb * 2;
+            r.exps = te + (int64_t)o0 * nv;
+            r.rows = (int64_t)cnt * nv;
+            r.K = naux;
+            r.stride = Q;
+            return r;
+          };
+          BQC_TRY(oz_gemm(rows(j0, nj), rows(i0, ni), oz_kblocks(naux), 1, 0, V.as<double>(),
+                          (int64_t)nj * nv, 0, 0, ctx->flag, s));
+        } else {
+          Gemm64Args v;
+          v.M = ni * nv;
+          v.N = nj * nv;
+          v.K1 = 1;
+          v.K2 = naux;
+          v.A = Bt.as<double>() + (int64_t)i0 * nv;
+          v.lda = Q;
+          v.B = Bt.as<double>() + (int64_t)j0 * nv;
+          v.ldb = Q;
+          v.C = V.as<double>();
+          v.ldc = (int64_t)nj * nv;
+          BQC_TRY(launch_gemm64(kAT, false, v, s));
         }
-        Gemm64Args v;
-        v.M = ni * nv;
-        v.N = nj * nv;
-        v.K1 = 1;
-        v.K2 = naux;
-        v.A = Bt.as<double>() + (int64_t)i0 * nv;
-        v.lda = ldt;
-        v.B = Bt.as<double>() + (int64_t)j0 * nv;
-        v.ldb = ldt;
-        v.C = V.as<double>();
-        v.ldc = (int64_t)nj * nv;
-        BQC_TRY(launch_gemm64(kAT, false, v, s));
         k_mp2_pairs<<<dim3((unsigned)ni, (unsigned)nj), 256, 0, s>>>(
             V.as<double>(), (int64_t)nj * nv, i0, j0, nv, eps, no, ep.as<double>());
         BQC_LAUNCH_CHECK();
