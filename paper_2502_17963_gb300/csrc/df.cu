@@ -23,17 +23,25 @@
 
 namespace bqc {
 
-// w[P] = sum_{mu,i} X[P][mu][i] C[mu][i]  (one block per P, FP64).
-__global__ void __launch_bounds__(256) k_wdot(const double *X, const double *C, int64_t nc,
-                                              double *w) {
+// w[P] = sum_{mu,i} X[P][mu][i] C[mu][i]  (one block of up to 1024 threads per
+// P, FP64).  Bound by the load latency of the few blocks a chunk of P gives:
+// four independent sums a thread keep four loads of each operand in flight.
+__global__ void __launch_bounds__(1024) k_wdot(const double *X, const double *C, int64_t nc,
+                                               double *w) {
   const int P = blockIdx.x;
   const double *x = X + (int64_t)P * nc;
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < nc; i += blockDim.x) s = fma(x[i], C[i], s);
-  __shared__ double red[256];
-  red[threadIdx.x] = s;
+  const int64_t st = blockDim.x;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  int64_t i = threadIdx.x;
+  for (; i + 3 * st < nc; i += 4 * st) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = fma(x[i + k * st], __ldg(C + i + k * st), s[k]);
+  }
+  for (; i < nc; i += st) s[0] = fma(x[i], __ldg(C + i), s[0]);
+  __shared__ double red[1024];
+  red[threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
+  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
     if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
     __syncthreads();
   }
@@ -231,6 +239,7 @@ __device__ __forceinline__ void unpack_jsum_one(const double *Jp, int nsplit, in
   const int64_t hi = r > c ? r : c, lo = r > c ? c : r;
   const int64_t q = hi * (hi + 1) / 2 + lo;
   double s = Jp[q];
+#pragma unroll 8
   for (int y = 1; y < nsplit; ++y) s += Jp[(int64_t)y * npair + q];
   J[i] = s;
 }
@@ -245,11 +254,13 @@ __global__ void k_unpack_jsum_grp(const __grid_constant__ JGroup g) {
                   (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// aux chunks of the J pass: enough blocks for four per SM, at least 64 P each
-int jpass_split(int64_t npair, int naux) {
+// aux chunks of the J pass: enough blocks for four per SM, at least min_aux P
+// each.  8: with the former 64 a small system ran on a few blocks, each a
+// serial stream ((H2O)_4 piece of 75 P: 10 blocks, 32 us).
+int jpass_split(int64_t npair, int naux, int min_aux) {
   const int64_t blocks = (npair / 2 + 256) / 256;
-  int sp = (int)std::min<int64_t>(16, (4 * (int64_t)sm_count() + blocks - 1) / blocks);
-  sp = std::max(1, std::min(sp, naux / 64));
+  int sp = (int)std::min<int64_t>(64, (4 * (int64_t)sm_count() + blocks - 1) / blocks);
+  sp = std::max(1, std::min(sp, naux / min_aux));
   return sp;
 }
 
@@ -463,6 +474,127 @@ int group_jpass(Df *const *dfs, double *const *J, int n, cudaStream_t s) {
   return BQC_OK;
 }
 
+// ------------------------------------------------ small molecules (FP64) --
+// Up to kSmallN functions a Fock build is a few microseconds of DFMA work, and
+// tiles of 64 or 128 would be mostly padding and too few to fill the chip.
+// One block per aux function does everything that needs B_P while it is in
+// shared memory: X_P = B_P C, w_P, and its contributions to K and J (packed
+// lower triangles, one slice per block, accumulated by their owner threads
+// over the block's aux functions); a second kernel sums the slices.
+constexpr int kSmallN = 112;
+
+__global__ void __launch_bounds__(256) k_jk64_small(const double *__restrict__ B,
+                                                    const double *__restrict__ C, int n, int no,
+                                                    int naux, double *__restrict__ w,
+                                                    double *__restrict__ part) {
+  extern __shared__ double sm[];
+  const int npair = n * (n + 1) / 2, ldb = n | 1, ldx = no | 1, t = threadIdx.x;
+  double *Bs = sm, *Cs = Bs + n * ldb, *Xs = Cs + n * no;
+  __shared__ double red[8];
+  double *pk = part + (int64_t)blockIdx.x * 2 * npair, *pj = pk + npair;
+  for (int e = t; e < n * no; e += 256) Cs[e] = C[e];
+  for (int P = blockIdx.x; P < naux; P += gridDim.x) {
+    const double *b = B + (int64_t)P * npair;
+    for (int q = t; q < npair; q += 256) {
+      int mu = (int)((sqrtf(8.0f * q + 1.0f) - 1.0f) * 0.5f);
+      while ((mu + 1) * (mu + 2) / 2 <= q) ++mu;
+      while (mu * (mu + 1) / 2 > q) --mu;
+      const int nu = q - mu * (mu + 1) / 2;
+      const double v = b[q];
+      Bs[mu * ldb + nu] = v;
+      Bs[nu * ldb + mu] = v;
+    }
+    __syncthreads();
+    double s = 0.0;
+    for (int e = t; e < n * no; e += 256) {
+      const int mu = e / no, i = e - mu * no;
+      double x0 = 0.0, x1 = 0.0;
+      int nu = 0;
+      for (; nu + 1 < n; nu += 2) {
+        x0 = fma(Bs[mu * ldb + nu], Cs[nu * no + i], x0);
+        x1 = fma(Bs[mu * ldb + nu + 1], Cs[(nu + 1) * no + i], x1);
+      }
+      if (nu < n) x0 = fma(Bs[mu * ldb + nu], Cs[nu * no + i], x0);
+      x0 += x1;
+      Xs[mu * ldx + i] = x0;
+      s = fma(x0, Cs[e], s);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((t & 31) == 0) red[t >> 5] = s;
+    __syncthreads();
+    double wp = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) wp += red[k];
+    if (t == 0) w[P] = wp;
+    const bool first = P == blockIdx.x;
+    for (int q = t; q < npair; q += 256) {
+      int mu = (int)((sqrtf(8.0f * q + 1.0f) - 1.0f) * 0.5f);
+      while ((mu + 1) * (mu + 2) / 2 <= q) ++mu;
+      while (mu * (mu + 1) / 2 > q) --mu;
+      const int nu = q - mu * (mu + 1) / 2;
+      double k0 = first ? 0.0 : pk[q];
+      for (int i = 0; i < no; ++i) k0 = fma(Xs[mu * ldx + i], Xs[nu * ldx + i], k0);
+      pk[q] = k0;
+      pj[q] = fma(wp, Bs[mu * ldb + nu], first ? 0.0 : pj[q]);
+    }
+    __syncthreads();
+  }
+}
+
+// K and J (full, symmetric) from the slices: 32 elements and 8 slice classes
+// per block, summed in a fixed order.
+__global__ void __launch_bounds__(256) k_jk64_small_sum(const double *__restrict__ part, int nslice,
+                                                        int n, double *__restrict__ K,
+                                                        double *__restrict__ J) {
+  __shared__ double t[8][33];
+  const int npair = n * (n + 1) / 2, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int q = blockIdx.x * 32 + tx;  // over K's pairs, then J's
+  double s = 0.0;
+  if (q < 2 * npair)
+    for (int k = ty; k < nslice; k += 8) s += part[(int64_t)k * 2 * npair + q];
+  t[ty][tx] = s;
+  __syncthreads();
+  if (ty || q >= 2 * npair) return;
+  s = 0.0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) s += t[k][tx];
+  const int p = q < npair ? q : q - npair;
+  int mu = (int)((sqrtf(8.0f * p + 1.0f) - 1.0f) * 0.5f);
+  while ((mu + 1) * (mu + 2) / 2 <= p) ++mu;
+  while (mu * (mu + 1) / 2 > p) --mu;
+  const int nu = p - mu * (mu + 1) / 2;
+  double *out = q < npair ? K : J;
+  out[mu * n + nu] = s;
+  out[nu * n + mu] = s;
+}
+
+static int jk64_small_slices(int naux) { return std::min(naux, 2 * sm_count()); }
+
+// Bytes of the FP64 X buffer: X, or the scratch of the small and the sliced
+// builds where that is more (at most 32 MiB more).
+static size_t x64_bytes(int n, int naux, int no);
+
+static int jk_fp64_small(Df *df, const double *C, double *J, double *K, cudaStream_t s) {
+  const int n = df->basis->nbf, naux = df->naux_loc, no = df->basis->nocc;
+  const int npair = n * (n + 1) / 2, nsl = jk64_small_slices(naux);
+  const size_t smem = ((size_t)n * (n | 1) + (size_t)n * no + (size_t)n * (no | 1)) * 8;
+  BQC_CUDA_TRY(cudaFuncSetAttribute(k_jk64_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem));
+  df->mark(0, s);
+  df->mark(1, s);
+  k_jk64_small<<<(unsigned)nsl, 256, smem, s>>>(df->B64.as<double>(), C, n, no, naux,
+                                                df->w.as<double>(), df->X64.as<double>());
+  BQC_LAUNCH_CHECK();
+  df->mark(2, s);
+  df->mark(3, s);
+  k_jk64_small_sum<<<(unsigned)((2 * npair + 31) / 32), 256, 0, s>>>(df->X64.as<double>(), nsl, n,
+                                                                     K, J);
+  BQC_LAUNCH_CHECK();
+  df->mark(4, s);
+  return BQC_OK;
+}
+
 // FP64 X pass and K on the tensor cores (oz.cu), over chunks of pc aux
 // functions.  The handle's X buffer (Naux N nocc doubles) is the scratch: a
 // chunk's sliced B, its X (FP64), its sliced X, and the K partials.
@@ -495,7 +627,8 @@ static OzJkPlan oz_jk_layout(int n, int no, int pc, int ns) {
 }
 
 static OzJkPlan oz_jk_plan(int n, int naux, int no, size_t bytes) {
-  // K splits: the count whose tiles fill whole waves best, splits of at least 256
+  // K splits: the count whose tiles fill whole waves best, splits of at
+  // least one accumulation chain (128)
   const int64_t tiles = oz_tiles(n, n, true);
   const int nsm = sm_count();
   OzJkPlan best;
@@ -503,7 +636,7 @@ static OzJkPlan oz_jk_plan(int n, int naux, int no, size_t bytes) {
     const int pc = (naux + chunks - 1) / chunks;
     int ns = 1;
     double eff = 0.0;
-    for (int c = 1; c <= 2 * nsm && (c == 1 || c * 256 <= pc * no); ++c) {
+    for (int c = 1; c <= 2 * nsm && (c == 1 || c * 128 <= pc * no); ++c) {
       const int64_t items = tiles * c;
       const double e = (double)items / ((double)((items + nsm - 1) / nsm) * nsm);
       if (e > eff + 1e-3) {
@@ -516,6 +649,13 @@ static OzJkPlan oz_jk_plan(int n, int naux, int no, size_t bytes) {
     if (p.total <= bytes) return p;
   }
   return best;
+}
+
+static size_t x64_bytes(int n, int naux, int no) {
+  const size_t x = (size_t)naux * n * no * 8;
+  const size_t more = n <= kSmallN ? (size_t)jk64_small_slices(naux) * n * (n + 1) * 8
+                                   : oz_jk_plan(n, naux, no, SIZE_MAX).total;
+  return std::max(x, std::min<size_t>(more, (size_t)32 << 20));
 }
 
 static int jk_fp64_oz(Df *df, const OzJkPlan &p, const double *C, double *J, double *K,
@@ -555,7 +695,7 @@ static int jk_fp64_oz(Df *df, const OzJkPlan &p, const double *C, double *J, dou
     ob.rows = b.rows;
     ob.K = n;
     BQC_TRY(oz_gemm(oc, ob, oz_kblocks(n), 1, 0, X, no, 0, 0, df->ctx->flag, s));
-    k_wdot<<<np, 256, 0, s>>>(X, C, (int64_t)n * no, df->w.as<double>() + P0);
+    k_wdot<<<np, 1024, 0, s>>>(X, C, (int64_t)n * no, df->w.as<double>() + P0);
     BQC_LAUNCH_CHECK();
     // K partials: rows mu, contraction (P, i); a short last chunk may have
     // fewer splits than the others, and adds to the first ones
@@ -589,7 +729,8 @@ int jk_fp64_stored(Df *df, const double *C, double *J, double *K, cudaStream_t s
   const int n = b->nbf, naux = df->naux_loc, no = b->nocc;
   const int64_t npair = df->npair;
   double *X = df->X64.as<double>();
-  if (n >= 64) {
+  if (n <= kSmallN && df->X64.n >= x64_bytes(n, naux, no)) return jk_fp64_small(df, C, J, K, s);
+  if (n > kSmallN) {
     const OzJkPlan p = oz_jk_plan(n, naux, no, df->X64.n);
     if (p.pc) return jk_fp64_oz(df, p, C, J, K, s);
   }
@@ -641,15 +782,19 @@ size_t df_stored_bytes(int n, int naux, int nocc, int shadow) {
   const size_t npair = (size_t)n * (n + 1) / 2;
   size_t b = (size_t)naux * naux * 8 + (size_t)naux * npair * 8;  // L, B64
   b += (size_t)naux * n * nocc * 8;                                // X64
-  b += (size_t)jpass_split((int64_t)npair, naux) * npair * 8 + (size_t)naux * 8 * 2;
+  // (J partials of systems that fill the GPU; the few MB that smaller ones
+  // hold beyond this, and X's scratch, are among the caller's small buffers)
+  b += (size_t)std::min(16, jpass_split((int64_t)npair, naux, 64)) * npair * 8 + (size_t)naux * 8 * 2;
   if (shadow == BQC_SHADOW_TF32 || shadow == BQC_SHADOW_F16)
     b += mixed_workspace_bytes(n, naux, nocc, shadow);
   if (shadow == BQC_SHADOW_F16) {  // float-pair B and w of the J pass, the pieces' J partials
     b += (size_t)naux * npair * 8 + (size_t)naux * 8;
     const int np = std::min(kJPieces, std::max(naux, 1));
     for (int k = 0; k < np; ++k)
-      b += (size_t)jpass_split((int64_t)npair, (int)((int64_t)naux * (k + 1) / np) -
-                                                   (int)((int64_t)naux * k / np)) *
+      b += (size_t)std::min(16, jpass_split((int64_t)npair,
+                                            (int)((int64_t)naux * (k + 1) / np) -
+                                                (int)((int64_t)naux * k / np),
+                                            64)) *
            npair * 8;
   }
   return b;
@@ -750,6 +895,13 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
     *out = df;
     return BQC_OK;
   }
+  // the FP64 X buffer (stored) or the raw block (direct), first used as the
+  // scratch of the factorisation and of the metric solve
+  DBuf &scr = mode == BQC_DF_STORED ? df->X64 : df->raw;
+  df->aux_block = std::max(1, std::min(o.aux_block, naux));
+  if ((st = scr.alloc(ctx, mode == BQC_DF_STORED ? x64_bytes(n, df->naux_loc, no)
+                                                 : (size_t)df->aux_block * npair * 8)) != BQC_OK)
+    return fail(st);
   // metric and its Cholesky factor
   if ((st = df->L.alloc(ctx, (size_t)naux * naux * 8)) != BQC_OK) return fail(st);
   if ((st = launch_int2c(basis, df->L.as<double>(), s)) != BQC_OK) return fail(st);
@@ -757,15 +909,13 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
   if (cudaMemcpyAsync(df->Vdiag.p, df->L.p, (size_t)naux * naux * 8, cudaMemcpyDeviceToDevice,
                       s) != cudaSuccess)
     return fail(BQC_E_CUDA);
-  if ((st = cholesky_lower(ctx, df->L.as<double>(), naux, s)) != BQC_OK) return fail(st);
+  if ((st = cholesky_lower(ctx, df->L.as<double>(), naux, scr.p, scr.n, s)) != BQC_OK) return fail(st);
   if ((st = ctx->check_flag(s)) != BQC_OK) return fail(st);
   if ((st = eri3c_plan(basis, o.schwarz, df->Vdiag.as<double>(), s, &df->plan)) != BQC_OK)
     return fail(st);
   if ((st = df->w.alloc(ctx, (size_t)naux * 8)) != BQC_OK) return fail(st);
   if (mode == BQC_DF_STORED) {
     df->Vdiag.release();  // metric only needed for the screening plan
-    // the FP64 X buffer, first used as the metric solve's scratch
-    if ((st = df->X64.alloc(ctx, (size_t)df->naux_loc * n * no * 8)) != BQC_OK) return fail(st);
     if (!shard) {
       if ((st = df->B64.alloc(ctx, (size_t)naux * npair * 8)) != BQC_OK) return fail(st);
       if (cudaMemsetAsync(df->B64.p, 0, (size_t)naux * npair * 8, s) != cudaSuccess)

@@ -110,10 +110,8 @@ int direct_setup(Df *df, cudaStream_t s) {
   Ctx *ctx = df->ctx;
   const Basis *b = df->basis;
   const int n = b->nbf, naux = b->naux, no = b->nocc;
-  df->aux_block = std::max(1, std::min(df->opts.aux_block, naux));
   // L^{-1} (FP64), once
   BQC_TRY(df->Linv.alloc(ctx, (size_t)naux * naux * 8));
-  BQC_TRY(df->raw.alloc(ctx, (size_t)df->aux_block * df->npair * 8));
   k_identity<<<nb((int64_t)naux * naux), 256, 0, s>>>(df->Linv.as<double>(), naux);
   BQC_LAUNCH_CHECK();
   BQC_TRY(trsm_lower_left(ctx, df->L.as<double>(), naux, df->Linv.as<double>(), naux, naux,

@@ -42,78 +42,141 @@ int dgemm(bool tA, bool tB, int M, int N, int K, double alpha, const double *A, 
 
 constexpr int kNB = 64;
 
-// Unblocked Cholesky of the kNB x kNB diagonal block at (k0, k0), in shared
-// memory; writes L (lower) and zeros above.  flag <- 1 when not positive.
+// Cholesky of the kNB x kNB diagonal block at (k0, k0) in shared memory, by
+// 16-column steps: one warp factors the 16 x 16 block in registers (lane =
+// row, no block-wide barrier per column), a thread per row solves the panel
+// below it, all threads update the rest.  Writes L (lower) and zeros above;
+// flag <- 1 when not positive.  One SM's FP64 pipe: 87000 DFMAs, 23 us at its
+// rate; a barrier-per-column version took 100 us.
+constexpr int kPB = 16;
 __global__ void __launch_bounds__(256) k_potrf_diag(double *A, int n, int k0, int *flag) {
   __shared__ double a[kNB][kNB + 1];
-  const int nb = min(kNB, n - k0);
-  for (int i = threadIdx.x; i < kNB * kNB; i += blockDim.x) {
+  __shared__ double dinv[kPB];
+  const int nb = min(kNB, n - k0), t = threadIdx.x;
+  for (int i = t; i < kNB * kNB; i += 256) {
     const int r = i / kNB, c = i % kNB;
-    a[r][c] = (r < nb && c < nb) ? A[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
+    // a ragged block is padded with the identity
+    a[r][c] = (r < nb && c < nb) ? A[(int64_t)(k0 + r) * n + k0 + c] : (r == c ? 1.0 : 0.0);
   }
   __syncthreads();
-  for (int j = 0; j < nb; ++j) {
-    if (threadIdx.x == 0) {
-      const double d = a[j][j];
-      if (!(d > 0.0)) {
-        atomicExch(flag, 1);
-        a[j][j] = 1.0;
-      } else {
-        a[j][j] = sqrt(d);
+  for (int j0 = 0; j0 < nb; j0 += kPB) {
+    if (t < 32) {
+      const int r = j0 + (t & (kPB - 1));
+      double x[kPB], di = 1.0;
+#pragma unroll
+      for (int c = 0; c < kPB; ++c) x[c] = a[r][j0 + c];
+#pragma unroll
+      for (int c = 0; c < kPB; ++c) {
+        double d = __shfl_sync(0xffffffffu, x[c], c);
+        if (!(d > 0.0)) {
+          if (t == 0) atomicExch(flag, 1);
+          d = 1.0;
+        }
+        const double sd = sqrt(d), iv = 1.0 / sd;
+        x[c] = (t & (kPB - 1)) == c ? sd : x[c] * iv;
+        if ((t & (kPB - 1)) == c) di = iv;
+#pragma unroll
+        for (int q = c + 1; q < kPB; ++q)
+          x[q] = fma(-x[c], __shfl_sync(0xffffffffu, x[c], q), x[q]);
+      }
+      if (t < kPB) {
+#pragma unroll
+        for (int c = 0; c < kPB; ++c) a[r][j0 + c] = c <= t ? x[c] : 0.0;
+        dinv[t] = di;
       }
     }
     __syncthreads();
-    const double djj = a[j][j];
-    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) a[i][j] /= djj;
-    __syncthreads();
-    const int m = nb - j - 1;
-    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-      const int r = j + 1 + t / m, c = j + 1 + t % m;
-      if (c <= r) a[r][c] -= a[r][j] * a[c][j];
+    const int r1 = j0 + kPB;
+    if (r1 + t < kNB) {
+      double x[kPB];
+#pragma unroll
+      for (int c = 0; c < kPB; ++c) {
+        double v = a[r1 + t][j0 + c];
+#pragma unroll
+        for (int l = 0; l < c; ++l) v = fma(-x[l], a[j0 + c][j0 + l], v);
+        x[c] = v * dinv[c];
+      }
+#pragma unroll
+      for (int c = 0; c < kPB; ++c) a[r1 + t][j0 + c] = x[c];
     }
     __syncthreads();
+    // a 16 x 16 grid of threads over the remaining square's lower part
+    const int tx = t & 15, ty = t >> 4;
+    for (int r = r1 + ty; r < kNB; r += 16)
+      for (int c = r1 + tx; c <= r; c += 16) {
+        double v = a[r][c];
+#pragma unroll
+        for (int l = 0; l < kPB; ++l) v = fma(-a[r][j0 + l], a[c][j0 + l], v);
+        a[r][c] = v;
+      }
+    __syncthreads();
   }
-  for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) {
+  for (int i = t; i < nb * nb; i += 256) {
     const int r = i / nb, c = i % nb;
     A[(int64_t)(k0 + r) * n + k0 + c] = (c <= r) ? a[r][c] : 0.0;
   }
 }
 
 // Rows below the diagonal block: A_rk := A_rk L_kk^{-T} (forward substitution
-// per row, one thread per row); also zeroes the block above the diagonal.
-__global__ void __launch_bounds__(128) k_chol_panel(double *A, int n, int k0) {
+// per row, one thread per row, the row in registers: the block is whole when
+// rows follow it); also zeroes the block above the diagonal.  A warp a block,
+// since a warp's 2080 DFMAs take 17 us of an SM's FP64 pipe.
+__global__ void __launch_bounds__(32) k_chol_panel(double *A, int n, int k0) {
   __shared__ double L[kNB][kNB + 1];
-  const int nb = min(kNB, n - k0);
-  for (int i = threadIdx.x; i < kNB * kNB; i += blockDim.x) {
-    const int r = i / kNB, c = i % kNB;
-    L[r][c] = (r < nb && c < nb) ? A[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
+  __shared__ double dinv[kNB];
+  for (int i = threadIdx.x; i < kNB * kNB; i += 32)
+    L[i / kNB][i % kNB] = A[(int64_t)(k0 + i / kNB) * n + k0 + i % kNB];
+  __syncwarp();
+  for (int i = threadIdx.x; i < kNB; i += 32) dinv[i] = 1.0 / L[i][i];
+  __syncwarp();
+  const int row = k0 + kNB + blockIdx.x * 32 + threadIdx.x;
+  if (row >= n) return;
+  double x[kNB];
+  double *ar = A + (int64_t)row * n + k0;
+#pragma unroll
+  for (int j = 0; j < kNB; ++j) x[j] = ar[j];
+#pragma unroll
+  for (int j = 0; j < kNB; ++j) {
+    x[j] *= dinv[j];
+#pragma unroll
+    for (int l = j + 1; l < kNB; ++l) x[l] = fma(-x[j], L[l][j], x[l]);
   }
-  __syncthreads();
-  const int row = k0 + nb + blockIdx.x * blockDim.x + threadIdx.x;
-  if (row < n) {
-    double x[kNB];
-    double *ar = A + (int64_t)row * n + k0;
-    for (int j = 0; j < nb; ++j) {
-      double v = ar[j];
-      for (int l = 0; l < j; ++l) v -= x[l] * L[j][l];
-      x[j] = v / L[j][j];
-    }
-    for (int j = 0; j < nb; ++j) ar[j] = x[j];
-    // upper block (row k0 + j, column `row`) = 0
-    for (int j = 0; j < nb; ++j) A[(int64_t)(k0 + j) * n + row] = 0.0;
-  }
+#pragma unroll
+  for (int j = 0; j < kNB; ++j) ar[j] = x[j];
+  // upper block (row k0 + j, column `row`) = 0
+  for (int j = 0; j < kNB; ++j) A[(int64_t)(k0 + j) * n + row] = 0.0;
 }
 
-int cholesky_lower(Ctx *ctx, double *A, int n, cudaStream_t s) {
+int cholesky_lower(Ctx *ctx, double *A, int n, void *scratch, size_t scratch_bytes,
+                   cudaStream_t s) {
   for (int k0 = 0; k0 < n; k0 += kNB) {
     const int nb = std::min(kNB, n - k0);
     k_potrf_diag<<<1, 256, 0, s>>>(A, n, k0, ctx->flag);
     BQC_LAUNCH_CHECK();
     const int rem = n - k0 - nb;
     if (rem <= 0) break;
-    k_chol_panel<<<(rem + 127) / 128, 128, 0, s>>>(A, n, k0);
+    k_chol_panel<<<(rem + 31) / 32, 32, 0, s>>>(A, n, k0);
     BQC_LAUNCH_CHECK();
     // trailing update, lower triangle only: A22 -= L21 L21^T
+    const double *L21 = A + (int64_t)(k0 + nb) * n + k0;
+    double *A22 = A + (int64_t)(k0 + nb) * n + k0 + nb;
+    if (oz_slice_bytes(rem, nb) + oz_exp_bytes(rem, 1) <= scratch_bytes) {
+      OzSrc x;
+      x.kind = kOzRows;
+      x.p = L21;
+      x.rows = rem;
+      x.K = nb;
+      x.ld = n;
+      OzOperand o;
+      o.slices = scratch;
+      int *e = reinterpret_cast<int *>(static_cast<char *>(scratch) + oz_slice_bytes(rem, nb));
+      o.exps = e;
+      o.rows = rem;
+      o.K = nb;
+      BQC_TRY(oz_slice(x, oz_kblocks(nb), scratch, e, s));
+      BQC_TRY(oz_gemm(o, o, oz_kblocks(nb), -1, 1, A22, n, 0, kOzUpper, ctx->flag, s));
+      continue;
+    }
     Gemm64Args g;
     g.M = rem;
     g.N = rem;
@@ -121,13 +184,13 @@ int cholesky_lower(Ctx *ctx, double *A, int n, cudaStream_t s) {
     g.K2 = nb;
     g.alpha = -1.0;
     g.beta = 1.0;
-    g.A = A + (int64_t)(k0 + nb) * n + k0;
+    g.A = L21;
     g.lda = n;
     g.sA1 = 0;
     g.B = g.A;
     g.ldb = n;
     g.sB1 = 0;
-    g.C = A + (int64_t)(k0 + nb) * n + k0 + nb;
+    g.C = A22;
     g.ldc = n;
     g.lower_only = 1;
     BQC_TRY(launch_gemm64(kAN, true, g, s));
@@ -160,30 +223,29 @@ __global__ void __launch_bounds__(128) k_trsm_diag(const double *L, int n, int k
 }
 
 // Explicit inverses of the kNB x kNB diagonal blocks of L, out[block][kNB][kNB]
-// row-major with zeros above the diagonal (and past the end of a ragged last
-// block).  One block per diagonal block, one thread per column; column j of
-// the inverse lives in row j of the same shared array, right of the diagonal.
+// row-major with zeros above the diagonal (and the identity past the end of a
+// ragged last block).  One block per diagonal block, one thread per column:
+// forward substitution of a unit vector held in registers.
 __global__ void __launch_bounds__(kNB) k_tri_inv(const double *L, int n, double *out) {
   __shared__ double a[kNB][kNB + 1];
   __shared__ double dinv[kNB];
   const int k0 = blockIdx.x * kNB, nb = min(kNB, n - k0), j = threadIdx.x;
-  for (int r = 0; r < nb; ++r)
-    if (j <= r) a[r][j] = L[(int64_t)(k0 + r) * n + k0 + j];
+  for (int r = 0; r < kNB; ++r)
+    a[r][j] = (r < nb && j < nb) ? (j <= r ? L[(int64_t)(k0 + r) * n + k0 + j] : 0.0)
+                                 : (r == j ? 1.0 : 0.0);
   __syncthreads();
-  if (j < nb) dinv[j] = 1.0 / a[j][j];
+  dinv[j] = 1.0 / a[j][j];
   __syncthreads();
-  if (j < nb)
-    for (int r = j + 1; r < nb; ++r) {
-      double v = -a[r][j] * dinv[j];
-      for (int l = j + 1; l < r; ++l) v = fma(-a[r][l], a[j][l], v);
-      a[j][r] = v * dinv[r];
-    }
-  __syncthreads();
-  double *o = out + (int64_t)blockIdx.x * kNB * kNB;
+  double x[kNB];
+#pragma unroll
+  for (int r = 0; r < kNB; ++r) x[r] = r == j ? 1.0 : 0.0;
+  double *o = out + (int64_t)blockIdx.x * kNB * kNB + j;
+#pragma unroll
   for (int r = 0; r < kNB; ++r) {
-    double v = 0.0;
-    if (r < nb && j < nb) v = j < r ? a[j][r] : (j == r ? dinv[r] : 0.0);
-    o[r * kNB + j] = v;
+    x[r] *= dinv[r];
+#pragma unroll
+    for (int l = r + 1; l < kNB; ++l) x[l] = fma(-x[r], a[l][r], x[l]);
+    o[r * kNB] = x[r];
   }
 }
 

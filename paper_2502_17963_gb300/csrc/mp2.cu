@@ -186,7 +186,7 @@ static int mp2_transform_oz(Df *df, const double *C, int nmo, double *Bt, char *
 // FP64-accurate tensor-core products; MIXED_F16X3: the pair blocks as
 // split-FP16 tensor-core GEMMs (FP32 accumulation in short chains, float-float
 // drains, FP64 blocks); the energy in FP64.  Without memory for the slices,
-// or below 64 functions, where a tile would be mostly padding, the DFMA GEMM.
+// or up to 64 functions, where a tile would be mostly padding, the DFMA GEMM.
 static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec, double *e2,
                    cudaStream_t s) {
   const Basis *b = df->basis;
@@ -201,7 +201,7 @@ static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec
     BQC_TRY(Bt.alloc(ctx, (size_t)naux * Q * 8));
     const int bi = mp2_block(no, nv);
     int pc = 0;
-    if (n >= 64 && Ts.alloc(ctx, oz_slice_bytes(Q, naux) + oz_exp_bytes(Q, 1)) == BQC_OK)
+    if (n > 64 && Ts.alloc(ctx, oz_slice_bytes(Q, naux) + oz_exp_bytes(Q, 1)) == BQC_OK)
       pc = mp2_transform_pc(n, naux, no, nv, Ts.n);
     const bool oz = prec == BQC_PREC_FP64 && Ts.p;
     if (pc)

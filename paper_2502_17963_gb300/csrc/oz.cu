@@ -196,7 +196,7 @@ struct OzParams {
   int N, mt, nt;
   int nkb, split_kb, ns;
   int tiles;  // tiles of one split
-  int lower;
+  int tri;
   const int *eA, *eB;
   double *out;
   int64_t ldo, split_stride;
@@ -212,12 +212,16 @@ __device__ __forceinline__ OzItem oz_item(const OzParams &p, int64_t it) {
   OzItem x;
   x.split = (int)(it / p.tiles);
   const int t = (int)(it - (int64_t)x.split * p.tiles);
-  if (p.lower) {  // row tile tm has column tiles 0 .. 2 tm + 1
+  if (p.tri) {  // row tile tm has column tiles 0 .. 2 tm + 1 (upper: counted from the end)
     int tm = (int)((sqrtf(4.0f * t + 1.0f) - 1.0f) * 0.5f);
     while ((tm + 1) * (tm + 2) <= t) ++tm;
     while (tm * (tm + 1) > t) --tm;
     x.tm = tm;
     x.tn = t - tm * (tm + 1);
+    if (p.tri == kOzUpper) {  // an odd column count leaves tile nt empty
+      x.tm = p.mt - 1 - x.tm;
+      x.tn = 2 * p.mt - 1 - x.tn;
+    }
   } else {
     x.tm = t / p.nt;
     x.tn = t - x.tm * p.nt;
@@ -412,9 +416,9 @@ static int oz_map(CUtensorMap *map, const OzOperand &o, int box_rows) {
 }
 
 int oz_gemm(const OzOperand &A, const OzOperand &B, int split_kb, int alpha, int beta, double *out,
-            int64_t ldo, int64_t split_stride, int lower, int *flag, cudaStream_t s) {
+            int64_t ldo, int64_t split_stride, int tri, int *flag, cudaStream_t s) {
   if (A.rows <= 0 || B.rows <= 0 || A.K <= 0 || A.K != B.K || split_kb <= 0 ||
-      A.rows > 0x7fffff00 || B.rows > 0x7fffff00 || (lower && A.rows != B.rows))
+      A.rows > 0x7fffff00 || B.rows > 0x7fffff00 || (tri && A.rows != B.rows))
     return BQC_E_INVALID;
   CUtensorMap ma, mb;
   BQC_TRY(oz_map(&ma, A, kOzM));
@@ -427,9 +431,9 @@ int oz_gemm(const OzOperand &A, const OzOperand &B, int split_kb, int alpha, int
   p.nkb = oz_kblocks(A.K);
   p.split_kb = split_kb;
   p.ns = (p.nkb + split_kb - 1) / split_kb;
-  p.lower = lower;
-  const int64_t tiles =
-      lower ? (int64_t)p.mt * (p.mt - 1) + std::min(p.nt, 2 * p.mt) : (int64_t)p.mt * p.nt;
+  p.tri = tri;
+  const int64_t tiles = tri == kOzUpper ? (int64_t)p.mt * (p.mt + 1)
+                                        : oz_tiles(A.rows, B.rows, tri == kOzLower);
   if (tiles > (1 << 30)) return BQC_E_INVALID;
   p.tiles = (int)tiles;
   p.eA = A.exps;

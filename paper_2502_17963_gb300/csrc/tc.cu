@@ -1137,12 +1137,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // K = sum over chunks of the FP64 partial tiles, symmetric.  One block per
-// (lower tile, 32-row strip): sums into shared memory, writes the strip and
-// its mirror image coalesced.
-__device__ __forceinline__ void syrk_reduce_strip(const double *part, int nchunk, int ntri, int n,
-                                                  double *K, int t, int sr) {
-  __shared__ double strip[32][kBM + 1];
-  int tm = 0;
+// (lower tile, 8 x 32 sub-tile), one element a thread: small systems have one
+// tile and over a hundred chunks, so the blocks have to come from the tile and
+// the loads of 16 chunks be in flight ((H2O)_4: 387 -> 12 us).  The mirror
+// image is written through shared memory.
+constexpr int kRedSub = (kBM / 8) * (kBM / 32);
+__device__ __forceinline__ void syrk_reduce_sub(const double *part, int nchunk, int ntri, int n,
+                                                double *K, int t, int sub) {
+  __shared__ double sm[8][33];
+  int tm = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
   while ((tm + 1) * (tm + 2) / 2 <= t) ++tm;
   const int tn = t - tm * (tm + 1) / 2;
   for (int e = threadIdx.x; e < 32 * kBM; e += blockDim.x) {
@@ -1167,7 +1170,7 @@ __device__ __forceinline__ void syrk_reduce_strip(const double *part, int nchunk
 
 __global__ void __launch_bounds__(256) k_syrk_reduce(const double *part, int nchunk, int ntri,
                                                      int n, double *K) {
-  syrk_reduce_strip(part, nchunk, ntri, n, K, blockIdx.x, blockIdx.y);
+  syrk_reduce_sub(part, nchunk, ntri, n, K, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------- TRMM ---
@@ -1860,7 +1863,7 @@ static int mixed_setup_f16(Df *df, MixedState *ms, cudaStream_t s) {
   // element, like the FP64 B it is split from)
   BQC_TRY(jpass_ff_setup(df, s));
   {  // room for the J partials of the pieces
-    const int np = std::min(kJPieces, naux);
+    const int np = j_pieces(naux, df->npair);
     int slices = 0;
     for (int k = 0; k < np; ++k)
       slices += jpass_split(df->npair, (int)((int64_t)naux * (k + 1) / np) -
@@ -2094,7 +2097,7 @@ static int mixed_syrk(Df *df, int kind, int split, const CUtensorMap *Xh, const 
   else
     k_syrk<kKindTF32, 1><<<grid, kThreads, m.sy_smem[0], s>>>(*Xh, *Xh, *Xh, *Xh, q);
   BQC_LAUNCH_CHECK();
-  k_syrk_reduce<<<dim3((unsigned)m.ntri, kBM / 32), 256, 0, s>>>(df->Kpart.as<double>(), q.nchunk,
+  k_syrk_reduce<<<dim3((unsigned)m.ntri, kRedSub), 256, 0, s>>>(df->Kpart.as<double>(), q.nchunk,
                                                                   m.ntri, n, K);
   BQC_LAUNCH_CHECK();
   return BQC_OK;
@@ -2174,7 +2177,7 @@ struct SyRedGroup {
 __global__ void __launch_bounds__(256) k_syrk_reduce_grp(const __grid_constant__ SyRedGroup g) {
   const int k = blockIdx.z;
   if ((int)blockIdx.x >= g.ntri[k]) return;
-  syrk_reduce_strip(g.part[k], g.nchunk[k], g.ntri[k], g.n[k], g.K[k], blockIdx.x, blockIdx.y);
+  syrk_reduce_sub(g.part[k], g.nchunk[k], g.ntri[k], g.n[k], g.K[k], blockIdx.x, blockIdx.y);
 }
 
 static bool groupable(const Df *df) {
@@ -2330,7 +2333,7 @@ int group_syrk(Df *const *dfs, double *const *K, int n, cudaStream_t s) {
     k_syrk_grp<<<grid, kThreads, m0.sy_smem[1], s>>>(*tab);
     BQC_LAUNCH_CHECK();
   }
-  k_syrk_reduce_grp<<<dim3((unsigned)ntri_max, kBM / 32, (unsigned)n), 256, 0, s>>>(*red);
+  k_syrk_reduce_grp<<<dim3((unsigned)ntri_max, kRedSub, (unsigned)n), 256, 0, s>>>(*red);
   BQC_LAUNCH_CHECK();
   return BQC_OK;
 }
@@ -2370,7 +2373,7 @@ int jk_mixed_stored(Df *df, const double *C, int prec, double *J, double *K, cud
     // as the X pass and the SYRK together at the memory parallelism a J
     // block gets beside a persistent tensor-core CTA, so it has to start
     // early to end with them).
-    const int np = std::min(kJPieces, naux);
+    const int np = j_pieces(naux, df->npair);
     cudaStream_t ts = df->tcs, js = df->side;
     df->mark(0, s);
     BQC_TRY(mixed_xpass(df, C, kind, split, s, &ms->mapAh, &ms->mapAl, rows, nullptr, nullptr,
@@ -2755,7 +2758,7 @@ int direct_mixed_finish(Df *df, int split, double *K, cudaStream_t s) {
     k_syrk<kKindTF32, 1><<<grid, kThreads, m.sy_smem[0], s>>>(dm->mapYh, dm->mapYh, dm->mapYh,
                                                              dm->mapYh, q);
   BQC_LAUNCH_CHECK();
-  k_syrk_reduce<<<dim3((unsigned)m.ntri, kBM / 32), 256, 0, s>>>(dm->Kpart.as<double>(),
+  k_syrk_reduce<<<dim3((unsigned)m.ntri, kRedSub), 256, 0, s>>>(dm->Kpart.as<double>(),
                                                                   q.nchunk, m.ntri, n, K);
   BQC_LAUNCH_CHECK();
   return BQC_OK;
