@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <memory>
 #include <cstddef>
 #include <cstdint>
 #include <mutex>
@@ -72,6 +73,18 @@ constexpr int kBoysNM = kBoysMaxM + kBoysTaylor;
 
 // --------------------------------------------------------- context -----
 
+// Streams for independent small kernels (the shell classes of an integral
+// pass), leased from a context by a SideFork.
+constexpr int kSideStreams = 8;
+constexpr int kMaxSideSets = 8;
+struct SideSet {
+  cudaStream_t st[kSideStreams] = {};
+  cudaEvent_t fork = nullptr, join[kSideStreams] = {};
+  int prio = 0;
+  bool busy = false;
+  ~SideSet();
+};
+
 struct Ctx {
   int device = 0;
   size_t budget = 0;
@@ -83,10 +96,32 @@ struct Ctx {
   std::mutex mu;
   std::atomic<size_t> bytes_live{0};
   std::unordered_map<void *, size_t> sizes;  // live allocations (guarded by mu)
+  std::vector<std::unique_ptr<SideSet>> sides;  // guarded by mu; at most kMaxSideSets
 
   void *dmalloc(size_t bytes);
   void dfree(void *p, size_t bytes_hint = 0);
   int check_flag(cudaStream_t s);  // reads and clears the device flag
+};
+
+// Fork and join of one stream over a leased set: next() gives the stream of the
+// next independent launch (it starts after everything submitted to `main`
+// before the fork), join() makes `main` wait for all of them (also on
+// destruction, so an error path leaves nothing running beside `main`).  While
+// main is being captured, or with all sets leased, next() is main itself.
+class SideFork {
+ public:
+  SideFork(Ctx *ctx, cudaStream_t main);
+  ~SideFork() { join(); }
+  SideFork(const SideFork &) = delete;
+  SideFork &operator=(const SideFork &) = delete;
+  cudaStream_t next();
+  int join();
+
+ private:
+  Ctx *ctx_;
+  cudaStream_t main_;
+  SideSet *set_ = nullptr;
+  int n_ = 0;
 };
 
 // Device buffer owned by a context.

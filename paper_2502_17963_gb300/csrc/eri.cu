@@ -188,7 +188,11 @@ int launch_eri3c_variant(const Basis *b, const Eri3cPlan *plan, int p0, int p1, 
     BQC_TRY(list.alloc(b->ctx, (size_t)std::max<int64_t>(1, maxc) * 8));
     BQC_TRY(count.alloc(b->ctx, 8));
   }
-  for (int lc = 0; lc <= kMaxLAux; ++lc) {
+  // The classes are independent (every integral belongs to one) and a class of
+  // a small molecule is a handful of blocks, each a 50 us latency chain: they
+  // run beside each other, the heavy ones first.
+  SideFork fork(b->ctx, s);
+  for (int lc = kMaxLAux; lc >= 0; --lc) {
     const int na = b->auxl_off[lc + 1] - b->auxl_off[lc];
     if (na == 0) continue;
     // shells of this l whose functions meet [p0, p1): a contiguous sub-range
@@ -208,7 +212,7 @@ int launch_eri3c_variant(const Basis *b, const Eri3cPlan *plan, int p0, int p1, 
       }
       if (s0 < 0) continue;
     }
-    for (int cls = 0; cls < kNPairClass; ++cls) {
+    for (int cls = kNPairClass - 1; cls >= 0; --cls) {
       const int np = b->pair_off[cls + 1] - b->pair_off[cls];
       if (np == 0 || plan->total[cls][lc] == 0) continue;
       const int64_t *hp = plan->h_prefix.data() + plan->prefix_off[cls][lc];
@@ -236,11 +240,12 @@ int launch_eri3c_variant(const Basis *b, const Eri3cPlan *plan, int p0, int p1, 
       a.list = list.as<int64_t>();
       a.count = count.as<unsigned long long>();
       if (variant == 0)
-        BQC_TRY(dispatch3(lc, cls, a, ntrip, s));
-      else
+        BQC_TRY(dispatch3(lc, cls, a, ntrip, fork.next()));
+      else  // the variants share one survivor list: one after the other
         BQC_TRY(dispatch3v(lc, cls, a, ntrip, variant, s));
     }
   }
+  BQC_TRY(fork.join());
   if (variant == 2) BQC_CUDA_TRY(cudaStreamSynchronize(s));  // before the list is released
   return BQC_OK;
 }
@@ -309,8 +314,9 @@ static int launch_schwarz_cls(const SchwarzArgs &a, cudaStream_t s) {
   return BQC_OK;
 }
 
-int launch_schwarz_pairs(const Basis *b, double *Qpair, cudaStream_t s) {
-  for (int cls = 0; cls < kNPairClass; ++cls) {
+int launch_schwarz_pairs(const Basis *b, double *Qpair, cudaStream_t s0) {
+  SideFork fork(b->ctx, s0);
+  for (int cls = kNPairClass - 1; cls >= 0; --cls) {
     const int np = b->pair_off[cls + 1] - b->pair_off[cls];
     if (np == 0) continue;
     SchwarzArgs a;
@@ -320,6 +326,7 @@ int launch_schwarz_pairs(const Basis *b, double *Qpair, cudaStream_t s) {
     a.npair = np;
     a.Q = Qpair + b->pair_off[cls];
     int st = BQC_E_UNSUPPORTED;
+    const cudaStream_t s = fork.next();
     switch (cls) {
       case 0: st = launch_schwarz_cls<0, 0>(a, s); break;
       case 1: st = launch_schwarz_cls<1, 0>(a, s); break;
@@ -330,7 +337,7 @@ int launch_schwarz_pairs(const Basis *b, double *Qpair, cudaStream_t s) {
     }
     BQC_TRY(st);
   }
-  return BQC_OK;
+  return fork.join();
 }
 
 // ------------------------------------------------------- metric (P|Q) ----
@@ -405,9 +412,10 @@ static int int2c_q(int lq, const Int2cArgs &a, cudaStream_t s) {
   return BQC_E_UNSUPPORTED;
 }
 
-int launch_int2c(const Basis *b, double *V, cudaStream_t s) {
-  for (int lp = 0; lp <= kMaxLAux; ++lp)
-    for (int lq = 0; lq <= kMaxLAux; ++lq) {
+int launch_int2c(const Basis *b, double *V, cudaStream_t s0) {
+  SideFork fork(b->ctx, s0);
+  for (int lp = kMaxLAux; lp >= 0; --lp)
+    for (int lq = kMaxLAux; lq >= 0; --lq) {
       const int nP = b->auxl_off[lp + 1] - b->auxl_off[lp];
       const int nQ = b->auxl_off[lq + 1] - b->auxl_off[lq];
       if (!nP || !nQ) continue;
@@ -421,6 +429,7 @@ int launch_int2c(const Basis *b, double *V, cudaStream_t s) {
       a.V = V;
       a.naux = b->naux;
       int st = BQC_E_UNSUPPORTED;
+      const cudaStream_t s = fork.next();
       switch (lp) {
         case 0: st = int2c_q<0>(lq, a, s); break;
         case 1: st = int2c_q<1>(lq, a, s); break;
@@ -429,7 +438,7 @@ int launch_int2c(const Basis *b, double *V, cudaStream_t s) {
       }
       BQC_TRY(st);
     }
-  return BQC_OK;
+  return fork.join();
 }
 
 // -------------------------------------------------- one-electron parts ---
@@ -635,22 +644,49 @@ __global__ void k_diag_sqrt_max(const double *V, int naux, const int *fn_of_shel
   q[i] = sqrt(m);
 }
 
-// cut[P] = number of class pairs with Q_pair * Q_P >= tau (pairs sorted descending).
-__global__ void k_cut(const double *qpair, int np, const int *aux_list, int na,
-                      const double *qaux, double tau, int64_t *cut) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= na) return;
-  const double qp = qaux[aux_list[i]];
-  int lo = 0, hi = np;  // first index with qpair*qp < tau
-  if (tau > 0.0) {
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (qpair[mid] * qp >= tau) lo = mid + 1; else hi = mid;
+// Survivor prefixes of every (pair class, aux l), one block each:
+// prefix[i + 1] = prefix[i] + number of class pairs with Q_pair * Q_P >= tau
+// (pairs sorted descending) for the i-th aux shell of that l.
+struct CutArgs {
+  int pair_off[kNPairClass + 1], auxl_off[kMaxLAux + 2];
+  int64_t prefix_off[kNPairClass][kMaxLAux + 1];
+  const double *qpair, *qaux;
+  const int *aux_by_l;
+  int64_t *prefix;
+  double tau;
+};
+
+__global__ void __launch_bounds__(256) k_cut_prefix(const __grid_constant__ CutArgs a) {
+  using Scan = cub::BlockScan<int64_t, 256>;
+  __shared__ typename Scan::TempStorage tmp;
+  const int cls = blockIdx.x, lc = blockIdx.y;
+  const int po = a.pair_off[cls], np = a.pair_off[cls + 1] - po;
+  const int ao = a.auxl_off[lc], na = a.auxl_off[lc + 1] - ao;
+  int64_t *pre = a.prefix + a.prefix_off[cls][lc];
+  const double *qpair = a.qpair + po;
+  if (threadIdx.x == 0) pre[0] = 0;
+  int64_t base = 0;
+  for (int i0 = 0; i0 < na; i0 += 256) {
+    const int i = i0 + threadIdx.x;
+    int lo = 0;  // first index with qpair * qp < tau
+    if (i < na) {
+      int hi = np;
+      if (a.tau > 0.0) {
+        const double qp = a.qaux[a.aux_by_l[ao + i]];
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (qpair[mid] * qp >= a.tau) lo = mid + 1; else hi = mid;
+        }
+      } else {
+        lo = np;
+      }
     }
-  } else {
-    lo = np;
+    int64_t v = lo, sum, all;
+    Scan(tmp).InclusiveSum(v, sum, all);
+    if (i < na) pre[i + 1] = base + sum;
+    base += all;
+    __syncthreads();
   }
-  cut[i] = lo;
 }
 
 int eri3c_plan(const Basis *b, double tau, const double *V_diag_dev, cudaStream_t s,
@@ -669,53 +705,47 @@ int eri3c_plan(const Basis *b, double tau, const double *V_diag_dev, cudaStream_
   k_diag_sqrt_max<<<(nas + 127) / 128, 128, 0, s>>>(V_diag_dev, b->naux, b->aux.dev.fn,
                                                       b->aux.dev.l, nas, plan->d_qaux.as<double>());
   BQC_LAUNCH_CHECK();
-  // sort each class segment by decreasing Q
-  for (int cls = 0; cls < kNPairClass; ++cls) {
-    const int o = b->pair_off[cls], n = b->pair_off[cls + 1] - o;
-    if (!n) continue;
-    size_t tmp = 0;
-    const double *kin = qpair.as<double>() + o;
-    double *kout = plan->d_qpair_sorted.as<double>() + o;
-    const int2 *vin = b->d_pairs.as<int2>() + o;
-    int2 *vout = plan->d_pairs_sorted.as<int2>() + o;
-    BQC_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(nullptr, tmp, kin, kout, vin, vout, n,
-                                                           0, 64, s));
-    DBuf t;
-    BQC_TRY(t.alloc(ctx, std::max<size_t>(tmp, 16)));
-    BQC_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(t.p, tmp, kin, kout, vin, vout, n, 0,
-                                                           64, s));
-    BQC_CUDA_TRY(cudaStreamSynchronize(s));  // t is released at scope end
+  // sort each class segment by decreasing Q (beside each other; the scratch is
+  // released after the copy below)
+  DBuf tmp[kNPairClass];
+  {
+    size_t need[kNPairClass] = {};
+    for (int cls = 0; cls < kNPairClass; ++cls) {
+      const int n = b->pair_off[cls + 1] - b->pair_off[cls];
+      if (!n) continue;
+      BQC_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(
+          nullptr, need[cls], (const double *)nullptr, (double *)nullptr, (const int2 *)nullptr,
+          (int2 *)nullptr, n, 0, 64, s));
+      BQC_TRY(tmp[cls].alloc(ctx, std::max<size_t>(need[cls], 16)));
+    }
+    SideFork fork(ctx, s);
+    for (int cls = 0; cls < kNPairClass; ++cls) {
+      const int o = b->pair_off[cls], n = b->pair_off[cls + 1] - o;
+      if (!n) continue;
+      BQC_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(
+          tmp[cls].p, need[cls], qpair.as<double>() + o, plan->d_qpair_sorted.as<double>() + o,
+          b->d_pairs.as<int2>() + o, plan->d_pairs_sorted.as<int2>() + o, n, 0, 64, fork.next()));
+    }
+    BQC_TRY(fork.join());
   }
   // survivor counts and prefixes per (class, aux l)
+  CutArgs ca;
   int64_t off = 0;
   for (int cls = 0; cls < kNPairClass; ++cls)
     for (int lc = 0; lc <= kMaxLAux; ++lc) {
-      plan->prefix_off[cls][lc] = off;
+      plan->prefix_off[cls][lc] = ca.prefix_off[cls][lc] = off;
       off += (b->auxl_off[lc + 1] - b->auxl_off[lc]) + 1;
     }
   BQC_TRY(plan->d_prefix.alloc(ctx, off * sizeof(int64_t)));
-  BQC_CUDA_TRY(cudaMemsetAsync(plan->d_prefix.p, 0, off * sizeof(int64_t), s));
-  DBuf cut;
-  BQC_TRY(cut.alloc(ctx, std::max<int64_t>(1, nas) * sizeof(int64_t)));
-  for (int cls = 0; cls < kNPairClass; ++cls) {
-    const int po = b->pair_off[cls], pn = b->pair_off[cls + 1] - po;
-    for (int lc = 0; lc <= kMaxLAux; ++lc) {
-      const int ao = b->auxl_off[lc], an = b->auxl_off[lc + 1] - ao;
-      if (!an) continue;
-      int64_t *pre = plan->d_prefix.as<int64_t>() + plan->prefix_off[cls][lc];
-      if (!pn) continue;
-      k_cut<<<(an + 127) / 128, 128, 0, s>>>(plan->d_qpair_sorted.as<double>() + po, pn,
-                                             b->d_aux_by_l.as<int>() + ao, an,
-                                             plan->d_qaux.as<double>(), tau, cut.as<int64_t>());
-      BQC_LAUNCH_CHECK();
-      size_t tmp = 0;
-      BQC_CUDA_TRY(cub::DeviceScan::InclusiveSum(nullptr, tmp, cut.as<int64_t>(), pre + 1, an, s));
-      DBuf t;
-      BQC_TRY(t.alloc(ctx, std::max<size_t>(tmp, 16)));
-      BQC_CUDA_TRY(cub::DeviceScan::InclusiveSum(t.p, tmp, cut.as<int64_t>(), pre + 1, an, s));
-      BQC_CUDA_TRY(cudaStreamSynchronize(s));
-    }
-  }
+  std::copy(b->pair_off, b->pair_off + kNPairClass + 1, ca.pair_off);
+  std::copy(b->auxl_off, b->auxl_off + kMaxLAux + 2, ca.auxl_off);
+  ca.qpair = plan->d_qpair_sorted.as<double>();
+  ca.qaux = plan->d_qaux.as<double>();
+  ca.aux_by_l = b->d_aux_by_l.as<int>();
+  ca.prefix = plan->d_prefix.as<int64_t>();
+  ca.tau = tau;
+  k_cut_prefix<<<dim3(kNPairClass, kMaxLAux + 1), 256, 0, s>>>(ca);
+  BQC_LAUNCH_CHECK();
   // read the totals (one small copy)
   std::vector<int64_t> &h = plan->h_prefix;
   h.assign(off, 0);

@@ -330,16 +330,21 @@ int jk_4c(Df *df, const double *C, int prec, double *J, double *K, cudaStream_t 
   a.Jacc = pl->Jacc.as<double>();
   a.Kacc = pl->Kacc.as<double>();
   a.n = n;
-  for (int x = 0; x < kNPairClass; ++x)
-    for (int y = 0; y <= x; ++y) {
+  // The class pairs add into J and K atomically and are otherwise independent;
+  // one of a small molecule is a few blocks with a 50-200 us latency chain, so
+  // they run beside each other, the heavy ones first.
+  SideFork fork(b->ctx, s);
+  for (int x = kNPairClass - 1; x >= 0; --x)
+    for (int y = x; y >= 0; --y) {
       if (pl->total[x][y] == 0) continue;
       a.pX = pl->pairs.as<int2>() + b->pair_off[x];
       a.pY = pl->pairs.as<int2>() + b->pair_off[y];
       a.prefix = pl->prefix.as<int64_t>() + pl->pre_off[x][y];
       a.npX = b->pair_off[x + 1] - b->pair_off[x];
       a.same = x == y;
-      BQC_TRY(dispatch_xy(x, y, a, pl->total[x][y], s));
+      BQC_TRY(dispatch_xy(x, y, a, pl->total[x][y], fork.next()));
     }
+  BQC_TRY(fork.join());
   df->mark(3, s);
   const unsigned nb = (unsigned)(((int64_t)n * n + 255) / 256);
   k_sym_add<<<nb, 256, 0, s>>>(pl->Jacc.as<double>(), n, J);

@@ -96,6 +96,83 @@ int Ctx::check_flag(cudaStream_t s) {
   return BQC_OK;
 }
 
+SideSet::~SideSet() {
+  for (auto &x : st)
+    if (x) cudaStreamDestroy(x);
+  for (auto &e : join)
+    if (e) cudaEventDestroy(e);
+  if (fork) cudaEventDestroy(fork);
+}
+
+static std::unique_ptr<SideSet> make_side_set(int prio) {
+  auto s = std::make_unique<SideSet>();
+  s->prio = prio;
+  bool ok = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) == cudaSuccess;
+  for (int k = 0; k < kSideStreams && ok; ++k)
+    ok = cudaStreamCreateWithPriority(&s->st[k], cudaStreamNonBlocking, prio) == cudaSuccess &&
+         cudaEventCreateWithFlags(&s->join[k], cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();
+    s.reset();
+  }
+  return s;
+}
+
+SideFork::SideFork(Ctx *ctx, cudaStream_t main) : ctx_(ctx), main_(main) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  int prio = 0;
+  if (cudaStreamIsCapturing(main, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+      (main && cudaStreamGetPriority(main, &prio) != cudaSuccess)) {
+    cudaGetLastError();
+    return;
+  }
+  {
+    std::lock_guard<std::mutex> g(ctx->mu);
+    for (auto &s : ctx->sides)
+      if (!s->busy && s->prio == prio) set_ = s.get();
+    if (!set_ && ctx->sides.size() < (size_t)kMaxSideSets) {
+      auto s = make_side_set(prio);
+      if (s) {
+        set_ = s.get();
+        ctx->sides.push_back(std::move(s));
+      }
+    }
+    if (set_) set_->busy = true;
+  }
+  if (set_ && cudaEventRecord(set_->fork, main) != cudaSuccess) {
+    cudaGetLastError();
+    join();
+  }
+}
+
+cudaStream_t SideFork::next() {
+  if (!set_) return main_;
+  const int k = n_ % kSideStreams;
+  if (n_ < kSideStreams && cudaStreamWaitEvent(set_->st[k], set_->fork, 0) != cudaSuccess) {
+    cudaGetLastError();
+    return main_;
+  }
+  ++n_;
+  return set_->st[k];
+}
+
+int SideFork::join() {
+  if (!set_) return BQC_OK;
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < kSideStreams && k < n_; ++k) {
+    cudaError_t r = cudaEventRecord(set_->join[k], set_->st[k]);
+    if (r == cudaSuccess) r = cudaStreamWaitEvent(main_, set_->join[k], 0);
+    if (r != cudaSuccess) e = r;
+  }
+  {
+    std::lock_guard<std::mutex> g(ctx_->mu);
+    set_->busy = false;
+  }
+  set_ = nullptr;
+  BQC_CUDA_TRY(e);
+  return BQC_OK;
+}
+
 int DBuf::alloc(Ctx *c, size_t bytes) {
   release();
   ctx = c;
@@ -253,6 +330,7 @@ int bqc_ctx_destroy(bqc_ctx *ctx) {
   if (!ctx) return BQC_E_INVALID;
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
+  ctx->sides.clear();
   ctx->dfree(ctx->boys, (size_t)kBoysNT * kBoysNM * sizeof(double));
   ctx->dfree(ctx->flag, sizeof(int));
   delete ctx;
