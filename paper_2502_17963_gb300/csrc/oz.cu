@@ -310,42 +310,41 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_f16(kOzM, kOzN);
-      int64_t kg = 0, g = 0;
-      for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        const OzItem x = oz_item(p, it);
-        for (int c0 = x.kb0; c0 < x.kb1 && ok; c0 += kOzChain, ++g) {
-          const int c1 = min(x.kb1, c0 + kOzChain);
-          for (int kb = c0; kb < c1 && ok; ++kb, ++kg) {
-            const int st = (int)(kg % kOzStages);
-            ok = mbar_wait(full0 + 8 * st, (uint32_t)((kg / kOzStages) & 1), p.flag, 62);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t a = sbase + st * kOzStage, b = a + kOzSlices * kOzASlice;
+    constexpr uint32_t idesc = idesc_f16(kOzM, kOzN);
+    int64_t kg = 0, g = 0;
+    for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      const OzItem x = oz_item(p, it);
+      for (int c0 = x.kb0; c0 < x.kb1 && ok; c0 += kOzChain, ++g) {
+        const int c1 = min(x.kb1, c0 + kOzChain);
+        for (int kb = c0; kb < c1 && ok; ++kb, ++kg) {
+          const int st = (int)(kg % kOzStages);
+          ok = mbar_wait_warp(full0 + 8 * st, (uint32_t)((kg / kOzStages) & 1), p.flag, 62);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t a = sdesc_sw64(sbase + st * kOzStage);
+          const uint64_t b = a + ((kOzSlices * kOzASlice) >> 4);
 #pragma unroll
-            for (int d = 0; d < kOzLevels; ++d) {
-              if (kb == c0 && g > 0) {
-                ok = mbar_wait(tempty0 + 8 * d, (uint32_t)((g - 1) & 1), p.flag, 63);
-                if (!ok) break;
-                tc_fence_after();
-              }
-              uint32_t acc = kb != c0;
-#pragma unroll
-              for (int i = 0; i < kOzSlices; ++i) {
-                const int j = d - i;
-                if (j < 0 || j >= kOzSlices) continue;
-#pragma unroll
-                for (int k2 = 0; k2 < 2; ++k2) {
-                  mma_f16(tbase + d * kOzN, sdesc_sw64(a + i * kOzASlice + k2 * 32),
-                          sdesc_sw64(b + j * kOzBSlice + k2 * 32), idesc, acc);
-                  acc = 1;
-                }
-              }
-              if (kb == c1 - 1) mma_commit(tfull0 + 8 * d);
+          for (int d = 0; d < kOzLevels; ++d) {
+            if (kb == c0 && g > 0) {
+              ok = mbar_wait_warp(tempty0 + 8 * d, (uint32_t)((g - 1) & 1), p.flag, 63);
+              if (!ok) break;
+              tc_fence_after();
             }
-            if (ok) mma_commit(empty0 + 8 * st);
+            uint32_t acc = kb != c0;
+#pragma unroll
+            for (int i = 0; i < kOzSlices; ++i) {
+              const int j = d - i;
+              if (j < 0 || j >= kOzSlices) continue;
+#pragma unroll
+              for (int k2 = 0; k2 < 2; ++k2) {
+                mma_f16(tbase + d * kOzN, a + ((i * kOzASlice + k2 * 32) >> 4),
+                        b + ((j * kOzBSlice + k2 * 32) >> 4), idesc, acc);
+                acc = 1;
+              }
+            }
+            if (kb == c1 - 1) mma_commit(tfull0 + 8 * d);
           }
+          if (ok) mma_commit(empty0 + 8 * st);
         }
       }
     }

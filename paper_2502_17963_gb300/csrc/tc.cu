@@ -314,54 +314,52 @@ __device__ __forceinline__ void xpass_body(const LOC &loc, int64_t tiles, int st
         ok = mbar_wait(empty0 + 8 * (int)(j % stages), (uint32_t)((j / stages) & 1), flag, 15);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      int64_t kg = 0, g = 0;
-      for (int64_t t = tbeg; t < tiles && ok; t += tstep) {
-        const XTile T = loc.at(t);
-        const int kblocks = T.p->kblocks;
-        const int ngroups = (kblocks + kGroupKb - 1) / kGroupKb;
-        const uint32_t idesc = KD::idesc(kBM, T.xn);
-        for (int gr = 0; gr < ngroups && ok; ++gr, ++g) {
-          const int b = (int)(g & 1);
-          if (g >= 2) ok = mbar_wait(tempty0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), flag, 14);
+    int64_t kg = 0, g = 0;
+    for (int64_t t = tbeg; t < tiles && ok; t += tstep) {
+      const XTile T = loc.at(t);
+      const int kblocks = T.p->kblocks;
+      const int ngroups = (kblocks + kGroupKb - 1) / kGroupKb;
+      const uint32_t idesc = KD::idesc(kBM, T.xn);
+      for (int gr = 0; gr < ngroups && ok; ++gr, ++g) {
+        const int b = (int)(g & 1);
+        if (g >= 2) ok = mbar_wait_warp(tempty0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), flag, 14);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d = tbase + b * XN;
+        const int kb0 = gr * kGroupKb, kb1 = min(kblocks, kb0 + kGroupKb);
+        for (int kb = kb0; kb < kb1 && ok; ++kb, ++kg) {
+          const int s = (int)(kg % stages);
+          ok = mbar_wait_warp(full0 + 8 * s, (uint32_t)((kg / stages) & 1), flag, 12);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t d = tbase + b * XN;
-          const int kb0 = gr * kGroupKb, kb1 = min(kblocks, kb0 + kGroupKb);
-          for (int kb = kb0; kb < kb1 && ok; ++kb, ++kg) {
-            const int s = (int)(kg % stages);
-            ok = mbar_wait(full0 + 8 * s, (uint32_t)((kg / stages) & 1), flag, 12);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t ah = sbase + s * stage_bytes, al = ah + a_bytes;
-            const uint32_t ch = ah + NS * a_bytes, cl = ch + c_bytes;
-            if (SPLIT == 3) {
-              // cross terms first: their running sum stays ~2^-11 of the
-              // result, so the accumulator's truncation there is negligible;
-              // then the hi*hi terms
+          const uint32_t ah = sbase + s * stage_bytes, al = ah + a_bytes;
+          const uint32_t ch = ah + NS * a_bytes, cl = ch + c_bytes;
+          if (SPLIT == 3) {
+            // cross terms first: their running sum stays ~2^-11 of the
+            // result, so the accumulator's truncation there is negligible;
+            // then the hi*hi terms
 #pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4) {
-                const uint32_t acc = ((kb - kb0) | k4) != 0;
-                KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(cl + k4 * 32), acc, idesc);
-                KD::mma(d, sdesc_sw128(al + k4 * 32), sdesc_sw128(ch + k4 * 32), 1, idesc);
-              }
-#pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4)
-                KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(ch + k4 * 32), 1, idesc);
-            } else {
-#pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4) {
-                const uint32_t acc = ((kb - kb0) | k4) != 0;
-                KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(ch + k4 * 32), acc, idesc);
-              }
+            for (int k4 = 0; k4 < 4; ++k4) {
+              const uint32_t acc = ((kb - kb0) | k4) != 0;
+              KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(cl + k4 * 32), acc, idesc);
+              KD::mma(d, sdesc_sw128(al + k4 * 32), sdesc_sw128(ch + k4 * 32), 1, idesc);
             }
-            if (MC)
-              mma_commit_mc(empty0 + 8 * s, 3);
-            else
-              mma_commit(empty0 + 8 * s);
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4)
+              KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(ch + k4 * 32), 1, idesc);
+          } else {
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4) {
+              const uint32_t acc = ((kb - kb0) | k4) != 0;
+              KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(ch + k4 * 32), acc, idesc);
+            }
           }
-          mma_commit(tfull0 + 8 * b);
+          if (MC)
+            mma_commit_mc(empty0 + 8 * s, 3);
+          else
+            mma_commit(empty0 + 8 * s);
         }
+        mma_commit(tfull0 + 8 * b);
       }
     }
   } else {
@@ -750,49 +748,47 @@ __device__ __forceinline__ void syrk_body(const LOC &loc, int items, int stages,
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = KD::idesc(kBM, kBM);
-      int64_t kg = 0, g = 0;
-      for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        const SyItem I = loc.at(it);
-        int nkb;
-        int64_t P0;
-        chunk_kb(*I.p, I.chunk, P0, nkb);
-        for (int kb0 = 0; kb0 < nkb && ok; kb0 += kGroupKbS, ++g) {
-          const int b = (int)(g & 1);
-          if (g >= 2) ok = mbar_wait(tempty0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), flag, 24);
+    constexpr uint32_t idesc = KD::idesc(kBM, kBM);
+    int64_t kg = 0, g = 0;
+    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      const SyItem I = loc.at(it);
+      int nkb;
+      int64_t P0;
+      chunk_kb(*I.p, I.chunk, P0, nkb);
+      for (int kb0 = 0; kb0 < nkb && ok; kb0 += kGroupKbS, ++g) {
+        const int b = (int)(g & 1);
+        if (g >= 2) ok = mbar_wait_warp(tempty0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), flag, 24);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d = tbase + b * kBM;
+        const int kb1 = min(nkb, kb0 + kGroupKbS);
+        for (int kb = kb0; kb < kb1 && ok; ++kb, ++kg) {
+          const int s = (int)(kg % stages);
+          ok = mbar_wait_warp(full0 + 8 * s, (uint32_t)((kg / stages) & 1), flag, 22);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t d = tbase + b * kBM;
-          const int kb1 = min(nkb, kb0 + kGroupKbS);
-          for (int kb = kb0; kb < kb1 && ok; ++kb, ++kg) {
-            const int s = (int)(kg % stages);
-            ok = mbar_wait(full0 + 8 * s, (uint32_t)((kg / stages) & 1), flag, 22);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t hm = sbase + s * stage_bytes, hn = hm + kAStage;
-            const uint32_t lm = hm + 2 * kAStage, ln = hm + 3 * kAStage;
-            if (SPLIT == 3) {  // cross terms first, as in the X pass
+          const uint32_t hm = sbase + s * stage_bytes, hn = hm + kAStage;
+          const uint32_t lm = hm + 2 * kAStage, ln = hm + 3 * kAStage;
+          if (SPLIT == 3) {  // cross terms first, as in the X pass
 #pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4) {
-                const uint32_t acc = ((kb - kb0) | k4) != 0;
-                KD::mma(d, sdesc_sw128(hm + k4 * 32), sdesc_sw128(ln + k4 * 32), acc, idesc);
-                KD::mma(d, sdesc_sw128(lm + k4 * 32), sdesc_sw128(hn + k4 * 32), 1, idesc);
-              }
-#pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4)
-                KD::mma(d, sdesc_sw128(hm + k4 * 32), sdesc_sw128(hn + k4 * 32), 1, idesc);
-            } else {
-#pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4) {
-                const uint32_t acc = ((kb - kb0) | k4) != 0;
-                KD::mma(d, sdesc_sw128(hm + k4 * 32), sdesc_sw128(hn + k4 * 32), acc, idesc);
-              }
+            for (int k4 = 0; k4 < 4; ++k4) {
+              const uint32_t acc = ((kb - kb0) | k4) != 0;
+              KD::mma(d, sdesc_sw128(hm + k4 * 32), sdesc_sw128(ln + k4 * 32), acc, idesc);
+              KD::mma(d, sdesc_sw128(lm + k4 * 32), sdesc_sw128(hn + k4 * 32), 1, idesc);
             }
-            mma_commit(empty0 + 8 * s);
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4)
+              KD::mma(d, sdesc_sw128(hm + k4 * 32), sdesc_sw128(hn + k4 * 32), 1, idesc);
+          } else {
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4) {
+              const uint32_t acc = ((kb - kb0) | k4) != 0;
+              KD::mma(d, sdesc_sw128(hm + k4 * 32), sdesc_sw128(hn + k4 * 32), acc, idesc);
+            }
           }
-          mma_commit(tfull0 + 8 * b);
+          mma_commit(empty0 + 8 * s);
         }
+        mma_commit(tfull0 + 8 * b);
       }
     }
   } else {
@@ -1040,37 +1036,35 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = KD::idesc(kBM, kBM);
-      int64_t kg = 0, g = 0;
-      for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        for (int kb0 = 0; kb0 < p.kblocks && ok; kb0 += kGroupKbS, ++g) {
-          const int b = (int)(g & 1);
-          if (g >= 2) ok = mbar_wait(tempty0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), p.flag, 44);
+    constexpr uint32_t idesc = KD::idesc(kBM, kBM);
+    int64_t kg = 0, g = 0;
+    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      for (int kb0 = 0; kb0 < p.kblocks && ok; kb0 += kGroupKbS, ++g) {
+        const int b = (int)(g & 1);
+        if (g >= 2) ok = mbar_wait_warp(tempty0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), p.flag, 44);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d = tbase + b * kBM;
+        const int kb1 = min(p.kblocks, kb0 + kGroupKbS);
+        for (int kb = kb0; kb < kb1 && ok; ++kb, ++kg) {
+          const int st = (int)(kg % p.stages);
+          ok = mbar_wait_warp(full0 + 8 * st, (uint32_t)((kg / p.stages) & 1), p.flag, 42);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t d = tbase + b * kBM;
-          const int kb1 = min(p.kblocks, kb0 + kGroupKbS);
-          for (int kb = kb0; kb < kb1 && ok; ++kb, ++kg) {
-            const int st = (int)(kg % p.stages);
-            ok = mbar_wait(full0 + 8 * st, (uint32_t)((kg / p.stages) & 1), p.flag, 42);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t ah = sbase + st * stage_bytes, bh = ah + kAStage;
-            const uint32_t al = ah + 2 * kAStage, bl = ah + 3 * kAStage;
+          const uint32_t ah = sbase + st * stage_bytes, bh = ah + kAStage;
+          const uint32_t al = ah + 2 * kAStage, bl = ah + 3 * kAStage;
 #pragma unroll
-            for (int k4 = 0; k4 < 4; ++k4) {  // cross terms first
-              const uint32_t acc = ((kb - kb0) | k4) != 0;
-              KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(bl + k4 * 32), acc, idesc);
-              KD::mma(d, sdesc_sw128(al + k4 * 32), sdesc_sw128(bh + k4 * 32), 1, idesc);
-            }
-#pragma unroll
-            for (int k4 = 0; k4 < 4; ++k4)
-              KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(bh + k4 * 32), 1, idesc);
-            mma_commit(empty0 + 8 * st);
+          for (int k4 = 0; k4 < 4; ++k4) {  // cross terms first
+            const uint32_t acc = ((kb - kb0) | k4) != 0;
+            KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(bl + k4 * 32), acc, idesc);
+            KD::mma(d, sdesc_sw128(al + k4 * 32), sdesc_sw128(bh + k4 * 32), 1, idesc);
           }
-          mma_commit(tfull0 + 8 * b);
+#pragma unroll
+          for (int k4 = 0; k4 < 4; ++k4)
+            KD::mma(d, sdesc_sw128(ah + k4 * 32), sdesc_sw128(bh + k4 * 32), 1, idesc);
+          mma_commit(empty0 + 8 * st);
         }
+        mma_commit(tfull0 + 8 * b);
       }
     }
   } else {
@@ -1147,25 +1141,30 @@ __device__ __forceinline__ void syrk_reduce_sub(const double *part, int nchunk, 
   __shared__ double sm[8][33];
   int tm = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
   while ((tm + 1) * (tm + 2) / 2 <= t) ++tm;
+  while (tm * (tm + 1) / 2 > t) --tm;
   const int tn = t - tm * (tm + 1) / 2;
-  for (int e = threadIdx.x; e < 32 * kBM; e += blockDim.x) {
-    const int rr = e / kBM, c = e % kBM;
-    const int r = sr * 32 + rr;
-    double s = 0.0;
-    for (int ch = 0; ch < nchunk; ++ch) s += part[(((int64_t)ch * ntri + t) * kBM + r) * kBM + c];
-    strip[rr][c] = s;
+  const int r0 = (sub >> 2) * 8, c0 = (sub & 3) * 32;
+  if (tm * kBM + r0 >= n || tn * kBM + c0 >= n || (tm == tn && c0 > r0 + 7)) return;
+  const int rr = threadIdx.x >> 5, cc = threadIdx.x & 31;
+  const double *p = part + ((int64_t)t * kBM + r0 + rr) * kBM + c0 + cc;
+  const int64_t st = (int64_t)ntri * kBM * kBM;
+  double s = 0.0;
+  int ch = 0;
+  for (; ch + 16 <= nchunk; ch += 16) {
+    double v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __ldg(p + (ch + k) * st);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) s += v[k];
   }
+  for (; ch < nchunk; ++ch) s += __ldg(p + ch * st);
+  sm[rr][cc] = s;
+  const int mu = tm * kBM + r0 + rr, nu = tn * kBM + c0 + cc;
+  if (mu < n && nu < n && (tm != tn || nu <= mu)) K[(int64_t)mu * n + nu] = s;
   __syncthreads();
-  for (int e = threadIdx.x; e < 32 * kBM; e += blockDim.x) {
-    const int rr = e / kBM, c = e % kBM;
-    const int mu = tm * kBM + sr * 32 + rr, nu = tn * kBM + c;
-    if (mu < n && nu < n && (tm != tn || nu <= mu)) K[(int64_t)mu * n + nu] = strip[rr][c];
-  }
-  for (int e = threadIdx.x; e < 32 * kBM; e += blockDim.x) {
-    const int c = e / 32, rr = e % 32;
-    const int mu = tm * kBM + sr * 32 + rr, nu = tn * kBM + c;
-    if (mu < n && nu < n && (tm != tn || nu < mu)) K[(int64_t)nu * n + mu] = strip[rr][c];
-  }
+  const int r2 = threadIdx.x & 7, c2 = threadIdx.x >> 3;
+  const int mu2 = tm * kBM + r0 + r2, nu2 = tn * kBM + c0 + c2;
+  if (mu2 < n && nu2 < n && (tm != tn || nu2 < mu2)) K[(int64_t)nu2 * n + mu2] = sm[r2][c2];
 }
 
 __global__ void __launch_bounds__(256) k_syrk_reduce(const double *part, int nchunk, int ntri,
@@ -1255,48 +1254,46 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_tf32(kBM, kBM);
-      int64_t kg = 0, g = 0;
-      for (int64_t t = blockIdx.x; t < p.mtiles && ok; t += gridDim.x) {
-        for (int pt = p.ntp - 1; pt >= 0 && ok; --pt) {
-          const int nkb = kblocks_of(pt);
-          for (int kb0 = 0; kb0 < nkb && ok; kb0 += kGroupKbT, ++g) {
-            const int b = (int)(g & 1);
-            if (g >= 2)
-              ok = mbar_wait(tempty0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), p.flag, 34);
+    constexpr uint32_t idesc = idesc_tf32(kBM, kBM);
+    int64_t kg = 0, g = 0;
+    for (int64_t t = blockIdx.x; t < p.mtiles && ok; t += gridDim.x) {
+      for (int pt = p.ntp - 1; pt >= 0 && ok; --pt) {
+        const int nkb = kblocks_of(pt);
+        for (int kb0 = 0; kb0 < nkb && ok; kb0 += kGroupKbT, ++g) {
+          const int b = (int)(g & 1);
+          if (g >= 2)
+            ok = mbar_wait_warp(tempty0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), p.flag, 34);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t d = tbase + b * kBM;
+          const int kb1 = min(nkb, kb0 + kGroupKbT);
+          for (int kb = kb0; kb < kb1 && ok; ++kb, ++kg) {
+            const int st = (int)(kg % p.stages);
+            ok = mbar_wait_warp(full0 + 8 * st, (uint32_t)((kg / p.stages) & 1), p.flag, 32);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t d = tbase + b * kBM;
-            const int kb1 = min(nkb, kb0 + kGroupKbT);
-            for (int kb = kb0; kb < kb1 && ok; ++kb, ++kg) {
-              const int st = (int)(kg % p.stages);
-              ok = mbar_wait(full0 + 8 * st, (uint32_t)((kg / p.stages) & 1), p.flag, 32);
-              if (!ok) break;
-              tc_fence_after();
-              const uint32_t xh = sbase + st * stage_bytes, lh = xh + kAStage;
-              const uint32_t xl = xh + 2 * kAStage, ll = xh + 3 * kAStage;
-              if (SPLIT == 3) {  // cross terms first, as in the X pass
+            const uint32_t xh = sbase + st * stage_bytes, lh = xh + kAStage;
+            const uint32_t xl = xh + 2 * kAStage, ll = xh + 3 * kAStage;
+            if (SPLIT == 3) {  // cross terms first, as in the X pass
 #pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4) {
-                  const uint32_t acc = ((kb - kb0) | k4) != 0;
-                  mma_tf32(d, sdesc_sw128(xh + k4 * 32), sdesc_sw128(ll + k4 * 32), idesc, acc);
-                  mma_tf32(d, sdesc_sw128(xl + k4 * 32), sdesc_sw128(lh + k4 * 32), idesc, 1);
-                }
-#pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4)
-                  mma_tf32(d, sdesc_sw128(xh + k4 * 32), sdesc_sw128(lh + k4 * 32), idesc, 1);
-              } else {
-#pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4) {
-                  const uint32_t acc = ((kb - kb0) | k4) != 0;
-                  mma_tf32(d, sdesc_sw128(xh + k4 * 32), sdesc_sw128(lh + k4 * 32), idesc, acc);
-                }
+              for (int k4 = 0; k4 < 4; ++k4) {
+                const uint32_t acc = ((kb - kb0) | k4) != 0;
+                mma_tf32(d, sdesc_sw128(xh + k4 * 32), sdesc_sw128(ll + k4 * 32), idesc, acc);
+                mma_tf32(d, sdesc_sw128(xl + k4 * 32), sdesc_sw128(lh + k4 * 32), idesc, 1);
               }
-              mma_commit(empty0 + 8 * st);
+#pragma unroll
+              for (int k4 = 0; k4 < 4; ++k4)
+                mma_tf32(d, sdesc_sw128(xh + k4 * 32), sdesc_sw128(lh + k4 * 32), idesc, 1);
+            } else {
+#pragma unroll
+              for (int k4 = 0; k4 < 4; ++k4) {
+                const uint32_t acc = ((kb - kb0) | k4) != 0;
+                mma_tf32(d, sdesc_sw128(xh + k4 * 32), sdesc_sw128(lh + k4 * 32), idesc, acc);
+              }
             }
-            mma_commit(tfull0 + 8 * b);
+            mma_commit(empty0 + 8 * st);
           }
+          mma_commit(tfull0 + 8 * b);
         }
       }
     }
