@@ -191,15 +191,6 @@ __global__ void __launch_bounds__(256) k_jpass_ff_range(const float4 *__restrict
   jpass_ff_cols(B2, w2, Pa, Pb, npair, c2, Jp + (int64_t)(y0 + blockIdx.y) * npair);
 }
 
-// B (FP64) -> float pairs (hi, lo), hi = fl(B), lo = fl(B - hi).
-__global__ void k_split_ff(const double *__restrict__ B, int64_t count, float2 *__restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const double d = B[i];
-  const float h = (float)d;
-  out[i] = make_float2(h, (float)(d - (double)h));
-}
-
 // Grouped J pass of independent problems in one launch: problem k owns the
 // blocks [off[k], off[k + 1]) as xb[k] column blocks times sp[k] aux chunks.
 struct JGroup {
@@ -403,7 +394,7 @@ int jpass_fp64_range(Df *df, int P0, int P1, int y0, cudaStream_t s) {
   return BQC_OK;
 }
 
-int jpass_ff_setup(Df *df, cudaStream_t s) {
+int jpass_ff_alloc(Df *df) {
   const int64_t count = (int64_t)df->naux_loc * df->npair;
   BQC_TRY(df->B2f.alloc(df->ctx, (size_t)count * 8));
   BQC_TRY(df->w2f.alloc(df->ctx, (size_t)df->naux_loc * 8));
@@ -626,29 +617,40 @@ static OzJkPlan oz_jk_layout(int n, int no, int pc, int ns) {
   return p;
 }
 
+// Splits of a K contraction of length K: the count whose tiles fill whole waves
+// best, splits of at least one accumulation chain (128).
+static int oz_k_splits(int n, int K) {
+  int ns = 1;
+  double eff = 0.0;
+  for (int c = 1; c <= 2 * nsm && (c == 1 || c * 128 <= K); ++c) {
+    const int64_t items = tiles * c;
+    const double e = (double)items / ((double)((items + nsm - 1) / nsm) * nsm);
+    if (e > eff + 1e-3) {
+      eff = e;
+      ns = c;
+    }
+    if (items >= 2 * nsm) break;
+  }
+  return ns;
+}
+
 static OzJkPlan oz_jk_plan(int n, int naux, int no, size_t bytes) {
-  // K splits: the count whose tiles fill whole waves best, splits of at
-  // least one accumulation chain (128)
   const int64_t tiles = oz_tiles(n, n, true);
   const int nsm = sm_count();
   OzJkPlan best;
   for (int chunks = 1; chunks <= 64 && chunks <= naux; ++chunks) {
     const int pc = (naux + chunks - 1) / chunks;
-    int ns = 1;
-    double eff = 0.0;
-    for (int c = 1; c <= 2 * nsm && (c == 1 || c * 128 <= pc * no); ++c) {
-      const int64_t items = tiles * c;
-      const double e = (double)items / ((double)((items + nsm - 1) / nsm) * nsm);
-      if (e > eff + 1e-3) {
-        eff = e;
-        ns = c;
-      }
-      if (items >= 2 * nsm) break;
-    }
-    OzJkPlan p = oz_jk_layout(n, no, pc, ns);
+    OzJkPlan p = oz_jk_layout(n, no, pc, oz_k_splits(n, pc * no));
     if (p.total <= bytes) return p;
   }
   return best;
+static int oz_rows_of_b(const double *b, int64_t npair, int n, int np, void *slices, int *exps,
+                        OzOperand *o, cudaStream_t s);
+static int oz_rows_of_x(const double *X, int n, int no, int np, int ns, void *slices, int *exps,
+                        OzOperand *o, cudaStream_t s);
+static int oz_rows_of_c(const double *C, int n, int no, void *slices, int *exps, OzOperand *o,
+                        cudaStream_t s);
+
 }
 
 static size_t x64_bytes(int n, int naux, int no) {
@@ -666,54 +668,20 @@ static int jk_fp64_oz(Df *df, const OzJkPlan &p, const double *C, double *J, dou
   auto ints = [scr](size_t at) { return reinterpret_cast<int *>(scr + at); };
   df->mark(0, s);
   df->mark(1, s);
-  OzSrc c;  // C^T: rows i, contraction nu
-  c.kind = kOzCols;
-  c.p = C;
-  c.rows = no;
-  c.K = n;
-  c.ld = no;
-  BQC_TRY(oz_slice(c, oz_kblocks(n), scr + p.cs, ints(p.ce), s));
-  OzOperand oc;
-  oc.slices = scr + p.cs;
-  oc.exps = ints(p.ce);
-  oc.rows = no;
-  oc.K = n;
+  OzOperand oc, ob, ox;
+  BQC_TRY(oz_rows_of_c(C, n, no, scr + p.cs, ints(p.ce), &oc, s));
   const int ns = p.ns;
   for (int P0 = 0; P0 < naux; P0 += p.pc) {
     const int np = std::min(p.pc, naux - P0);
-    OzSrc b;  // rows (P, mu), contraction nu
-    b.kind = kOzSym;
-    b.p = df->B64.as<double>() + (int64_t)P0 * df->npair;
-    b.rows = (int64_t)np * n;
-    b.n2 = n;
-    b.sz = df->npair;
-    b.K = n;
-    BQC_TRY(oz_slice(b, oz_kblocks(n), scr + p.bs, ints(p.be), s));
-    OzOperand ob;
-    ob.slices = scr + p.bs;
-    ob.exps = ints(p.be);
-    ob.rows = b.rows;
-    ob.K = n;
+    BQC_TRY(oz_rows_of_b(df->B64.as<double>() + (int64_t)P0 * df->npair, df->npair, n, np,
+                         scr + p.bs, ints(p.be), &ob, s));
     BQC_TRY(oz_gemm(oc, ob, oz_kblocks(n), 1, 0, X, no, 0, 0, df->ctx->flag, s));
     k_wdot<<<np, 1024, 0, s>>>(X, C, (int64_t)n * no, df->w.as<double>() + P0);
     BQC_LAUNCH_CHECK();
-    // K partials: rows mu, contraction (P, i); a short last chunk may have
-    // fewer splits than the others, and adds to the first ones
-    OzSrc x;
-    x.kind = kOzRows;
-    x.p = X;
-    x.rows = n;
-    x.K = np * no;
-    x.k2 = no;
-    x.s1 = (int64_t)n * no;
-    x.ld = no;
-    const int kb = oz_split_kb(x.K, ns);
-    BQC_TRY(oz_slice(x, kb, scr + p.xs, ints(p.xe), s));
-    OzOperand ox;
-    ox.slices = scr + p.xs;
-    ox.exps = ints(p.xe);
-    ox.rows = n;
-    ox.K = x.K;
+    // K partials; a short last chunk may have fewer splits than the others, and
+    // adds to the first ones
+    BQC_TRY(oz_rows_of_x(X, n, no, np, ns, scr + p.xs, ints(p.xe), &ox, s));
+    const int kb = oz_split_kb(ox.K, ns);
     BQC_TRY(oz_gemm(ox, ox, kb, 1, P0 > 0, kp, n, (int64_t)n * n, 1, df->ctx->flag, s));
   }
   df->mark(2, s);
@@ -724,41 +692,118 @@ static int jk_fp64_oz(Df *df, const OzJkPlan &p, const double *C, double *J, dou
   return BQC_OK;
 }
 
-int jk_fp64_stored(Df *df, const double *C, double *J, double *K, cudaStream_t s) {
-  const Basis *b = df->basis;
-  const int n = b->nbf, naux = df->naux_loc, no = b->nocc;
-  const int64_t npair = df->npair;
-  double *X = df->X64.as<double>();
-  if (n <= kSmallN && df->X64.n >= x64_bytes(n, naux, no)) return jk_fp64_small(df, C, J, K, s);
-  if (n > kSmallN) {
-    const OzJkPlan p = oz_jk_plan(n, naux, no, df->X64.n);
-    if (p.pc) return jk_fp64_oz(df, p, C, J, K, s);
+// Rows (P, mu) of np packed symmetric matrices as a sliced operand.
+static int oz_rows_of_b(const double *b, int64_t npair, int n, int np, void *slices, int *exps,
+                        OzOperand *o, cudaStream_t s) {
+  OzSrc x;
+  x.kind = kOzSym;
+  x.p = b;
+  x.rows = (int64_t)np * n;
+  x.n2 = n;
+  x.sz = npair;
+  x.K = n;
+  o->slices = slices;
+  o->exps = exps;
+  o->rows = x.rows;
+  o->K = n;
+  return oz_slice(x, oz_kblocks(n), slices, exps, s);
+}
+
+// Rows mu of np matrices X[P][mu][i], contraction (P, i), in at most ns splits.
+static int oz_rows_of_x(const double *X, int n, int no, int np, int ns, void *slices, int *exps,
+                        OzOperand *o, cudaStream_t s) {
+  OzSrc x;
+  x.kind = kOzRows;
+  x.p = X;
+  x.rows = n;
+  x.K = np * no;
+  x.k2 = no;
+  x.s1 = (int64_t)n * no;
+  x.ld = no;
+  o->slices = slices;
+  o->exps = exps;
+  o->rows = n;
+  o->K = x.K;
+  return oz_slice(x, oz_split_kb(x.K, ns), slices, exps, s);
+}
+
+// C_occ^T: rows i, contraction nu.
+static int oz_rows_of_c(const double *C, int n, int no, void *slices, int *exps, OzOperand *o,
+                        cudaStream_t s) {
+  OzSrc c;
+  c.kind = kOzCols;
+  c.p = C;
+  c.rows = no;
+  c.K = n;
+  c.ld = no;
+  o->slices = slices;
+  o->exps = exps;
+  o->rows = no;
+  o->K = n;
+  return oz_slice(c, oz_kblocks(n), slices, exps, s);
+}
+
+static size_t x_of_b_fixed(int n, int no) { return oz_slice_bytes(no, n) + oz_exp_bytes(no, 1); }
+
+size_t x_of_b_bytes(int n, int no, int np) {
+  return x_of_b_fixed(n, no) + oz_slice_bytes((int64_t)np * n, n) +
+         oz_exp_bytes((int64_t)np * n, 1);
+}
+
+int x_of_b(Ctx *ctx, const double *b, int64_t npair, const double *C, int n, int no, int np,
+           double *X, void *scratch, size_t bytes, cudaStream_t s) {
+  int pc = std::min(np, 1 << 16);
+  while (pc > 0 && x_of_b_bytes(n, no, pc) > bytes) pc = pc > 8 ? pc * 7 / 8 : 0;
+  if (n > kSmallN && scratch && pc) {
+    char *scr = static_cast<char *>(scratch);
+    OzOperand oc, ob;
+    BQC_TRY(oz_rows_of_c(C, n, no, scr, reinterpret_cast<int *>(scr + oz_slice_bytes(no, n)), &oc,
+                         s));
+    scr += x_of_b_fixed(n, no);
+    int *be = reinterpret_cast<int *>(scr + oz_slice_bytes((int64_t)pc * n, n));
+    for (int P0 = 0; P0 < np; P0 += pc) {
+      BQC_TRY(oz_rows_of_b(b + (int64_t)P0 * npair, npair, n, std::min(pc, np - P0), scr, be, &ob,
+                           s));
+      BQC_TRY(oz_gemm(oc, ob, oz_kblocks(n), 1, 0, X + (int64_t)P0 * n * no, no, 0, 0, ctx->flag,
+                      s));
+    }
+    return BQC_OK;
   }
-  df->mark(0, s);
-  df->mark(1, s);
-  // X_P = Bsym_P C  (batched over P)
-  Gemm64Args g;
+  Gemm64Args g;  // batched over P
   g.M = n;
   g.N = no;
   g.K1 = 1;
   g.K2 = n;
-  g.A = df->B64.as<double>();
+  g.A = b;
   g.bsA = npair;
   g.B = C;
   g.ldb = no;
   g.C = X;
   g.ldc = no;
   g.bsC = (int64_t)n * no;
-  g.batch = naux;
-  BQC_TRY(launch_gemm64(kASym, false, g, s));
-  k_wdot<<<naux, 256, 0, s>>>(X, C, (int64_t)n * no, df->w.as<double>());
-  BQC_LAUNCH_CHECK();
-  df->mark(2, s);
-  // J pass
-  BQC_TRY(jpass_fp64(df, J, s));
-  df->mark(3, s);
-  // K = sum_{P,i} X_P,mu i X_P,nu i
-  Gemm64Args k;
+  g.batch = np;
+  return launch_gemm64(kASym, false, g, s);
+}
+
+int k_of_x(Ctx *ctx, const double *X, int n, int no, int naux, void *scratch, size_t bytes,
+           double *K, cudaStream_t s) {
+  for (int pc = std::min(naux, (1 << 30) / std::max(1, no)); scratch && pc >= 1; pc /= 2) {
+    const int ns = oz_splits(pc * no, oz_k_splits(n, pc * no));
+    const size_t kp = oz_align((size_t)ns * n * n * 8), xs = oz_slice_bytes(n, pc * no);
+    if (kp + xs + oz_exp_bytes(n, ns) > bytes) continue;
+    char *scr = static_cast<char *>(scratch);
+    double *part = reinterpret_cast<double *>(scr);
+    for (int P0 = 0; P0 < naux; P0 += pc) {
+      const int np = std::min(pc, naux - P0);
+      OzOperand ox;
+      BQC_TRY(oz_rows_of_x(X + (int64_t)P0 * n * no, n, no, np, ns, scr + kp,
+                           reinterpret_cast<int *>(scr + kp + xs), &ox, s));
+      BQC_TRY(oz_gemm(ox, ox, oz_split_kb(ox.K, ns), 1, P0 > 0, part, n, (int64_t)n * n, kOzLower,
+                      ctx->flag, s));
+    }
+    return oz_sym_reduce(part, ns, (int64_t)n * n, n, n, K, s);
+  }
+  Gemm64Args k;  // one launch over (P, i)
   k.M = n;
   k.N = n;
   k.K1 = naux;
@@ -773,7 +818,29 @@ int jk_fp64_stored(Df *df, const double *C, double *J, double *K, cudaStream_t s
   k.ldc = n;
   k.lower_only = 1;
   k.mirror = 1;
-  BQC_TRY(launch_gemm64(kAN, true, k, s));
+  return launch_gemm64(kAN, true, k, s);
+}
+
+int jk_fp64_stored(Df *df, const double *C, double *J, double *K, cudaStream_t s) {
+  const Basis *b = df->basis;
+  const int n = b->nbf, naux = df->naux_loc, no = b->nocc;
+  const int64_t npair = df->npair;
+  double *X = df->X64.as<double>();
+  if (n <= kSmallN && df->X64.n >= x64_bytes(n, naux, no)) return jk_fp64_small(df, C, J, K, s);
+  if (n > kSmallN) {
+    const OzJkPlan p = oz_jk_plan(n, naux, no, df->X64.n);
+    if (p.pc) return jk_fp64_oz(df, p, C, J, K, s);
+  }
+  df->mark(0, s);
+  df->mark(1, s);
+  BQC_TRY(x_of_b(df->ctx, df->B64.as<double>(), npair, C, n, no, naux, X, nullptr, 0, s));
+  k_wdot<<<naux, 256, 0, s>>>(X, C, (int64_t)n * no, df->w.as<double>());
+  BQC_LAUNCH_CHECK();
+  df->mark(2, s);
+  // J pass
+  BQC_TRY(jpass_fp64(df, J, s));
+  df->mark(3, s);
+  BQC_TRY(k_of_x(df->ctx, X, n, no, naux, nullptr, 0, K, s));
   df->mark(4, s);
   return BQC_OK;
 }
@@ -897,6 +964,13 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
   }
   // the FP64 X buffer (stored) or the raw block (direct), first used as the
   // scratch of the factorisation and of the metric solve
+  // direct mode: blocks of equal size (in multiples of 32, X's storage blocks;
+  // a block is padded to the largest), so that none is mostly padding and the
+  // one that the second integral pass finds in the buffer is no remainder
+  if (df->aux_block % 32 == 0 && naux > df->aux_block) {
+    const int nblk = (naux + df->aux_block - 1) / df->aux_block;
+    df->aux_block = std::min(df->aux_block, ((naux + nblk - 1) / nblk + 31) / 32 * 32);
+  }
   DBuf &scr = mode == BQC_DF_STORED ? df->X64 : df->raw;
   df->aux_block = std::max(1, std::min(o.aux_block, naux));
   if ((st = scr.alloc(ctx, mode == BQC_DF_STORED ? x64_bytes(n, df->naux_loc, no)

@@ -67,6 +67,7 @@ struct Df {
   DBuf Linv;   // Naux x Naux FP64 L^{-1}
   DBuf Xraw;   // FP64 path: Naux x N x nocc, then Y = L^{-1} X in place
   DBuf gamma;  // Naux FP64: gamma_Q = (Q|D), then c = V^{-1} gamma
+  DBuf Xscr;   // FP64 path: slices of the X pass
   DBuf D2;     // Npair FP64 packed density, off-diagonal doubled
   DBuf Kpart64;
   int aux_block = 1024;
@@ -107,7 +108,7 @@ struct Df {
   size_t device_bytes() const {
     return L.n + Vdiag.n + B64.n + B2f.n + w2f.n + X64.n + Jp.n + w.n + host_io.n + B32.n +
            X32.n + Ct32.n +
-           wpart.n + Kpart.n + raw.n + Linv.n + Xraw.n + gamma.n + D2.n +
+           wpart.n + Kpart.n + raw.n + Linv.n + Xraw.n + Xscr.n + gamma.n + D2.n +
            plan.d_pairs_sorted.n + plan.d_qpair_sorted.n + plan.d_qaux.n + plan.d_prefix.n +
            plan.d_qpair.n +
            mixed_bytes(mixed.get());
@@ -125,14 +126,22 @@ int jk_mixed_stored(Df *df, const double *C, int prec, double *J, double *K, cud
 int jk_k_rank2(Df *df, const double *Cw, const double *Cd, double *K, cudaStream_t s);
 int jk_fp64_stored(Df *df, const double *C, double *J, double *K, cudaStream_t s);
 // J = sum_P w_P B_P from the packed FP64 B and df->w (FP64), full symmetric.
+// X_P = B_P C (np packed rows b, X[P][mu][i]) and K = sum_P X_P X_P^T in FP64,
+// sliced on the tensor cores where the scratch allows, else on the DFMA GEMM.
+size_t x_of_b_bytes(int n, int no, int np);  // scratch for all rows at once
+int x_of_b(Ctx *ctx, const double *b, int64_t npair, const double *C, int n, int no, int np,
+           double *X, void *scratch, size_t bytes, cudaStream_t s);
+int k_of_x(Ctx *ctx, const double *X, int n, int no, int naux, void *scratch, size_t bytes,
+           double *K, cudaStream_t s);
 int jpass_fp64(Df *df, double *J, cudaStream_t s);
 // The FP64 J pass in pieces: partials of aux functions [P0, P1) (df->w) into
 // partial slices starting at y0, then the sum of nslice slices into J.
 int jpass_fp64_range(Df *df, int P0, int P1, int y0, cudaStream_t s);
 int jpass_unpack(Df *df, int nslice, double *J, cudaStream_t s);
 // The same J partials from the float-pair B and w (df->B2f, df->w2f) in
-// float-float arithmetic on the FP32 pipe; jpass_ff_setup builds B2f.
-int jpass_ff_setup(Df *df, cudaStream_t s);
+// float-float arithmetic on the FP32 pipe; jpass_ff_alloc makes room for them
+// (the FP16 shadow set-up fills B2f).
+int jpass_ff_alloc(Df *df);
 int jpass_ff_range(Df *df, int P0, int P1, int y0, cudaStream_t s);
 int jpass_split(int64_t npair, int naux, int min_aux = 8);
 // J[D] = sum_P (B_P : D) B_P in FP64 over the stored FP64 B for a symmetric

@@ -17,7 +17,6 @@
 
 #include "bqc_internal.h"
 #include "df_internal.h"
-#include "gemm64.cuh"
 
 namespace bqc {
 
@@ -143,9 +142,15 @@ int jk_direct(Df *df, const double *C, int prec, double *J, double *K, cudaStrea
     return BQC_E_UNSUPPORTED;
   }
   const bool mixed = prec != BQC_PREC_FP64;
+  const int q_last = (naux - 1) / bk * bk;
   const int split = prec == BQC_PREC_MIXED_TF32X3 ? 3 : 1;
   if (mixed && !df->dmixed) return BQC_E_INVALID;
-  if (!mixed && !df->Xraw.p) BQC_TRY(df->Xraw.alloc(ctx, (size_t)naux * n * no * 8));
+  if (!mixed && !df->Xraw.p) {
+    BQC_TRY(df->Xraw.alloc(ctx, (size_t)naux * n * no * 8));
+    // slices of 64 MB of (Q|..) rows; without them X runs on the DFMA GEMM
+    if (df->Xscr.alloc(ctx, std::min<size_t>((size_t)64 << 20, x_of_b_bytes(n, no, bk))) != BQC_OK)
+      df->Xscr.release();
+  }
   double *raw = df->raw.as<double>();
   double *gam = df->gamma.as<double>(), *cvec = gam + naux;
   df->mark(0, s);
@@ -163,20 +168,8 @@ int jk_direct(Df *df, const double *C, int prec, double *J, double *K, cudaStrea
     if (mixed) {
       BQC_TRY(direct_mixed_block(df, raw, q0, nq, split, s));
     } else {
-      Gemm64Args g;  // X_Q = (Q|..)sym C
-      g.M = n;
-      g.N = no;
-      g.K1 = 1;
-      g.K2 = n;
-      g.A = raw;
-      g.bsA = npair;
-      g.B = C;
-      g.ldb = no;
-      g.C = df->Xraw.as<double>() + (int64_t)q0 * n * no;
-      g.ldc = no;
-      g.bsC = (int64_t)n * no;
-      g.batch = nq;
-      BQC_TRY(launch_gemm64(kASym, false, g, s));
+      BQC_TRY(x_of_b(ctx, raw, npair, C, n, no, nq, df->Xraw.as<double>() + (int64_t)q0 * n * no,
+                     df->Xscr.p, df->Xscr.n, s));
     }
   }
   df->mark(2, s);
@@ -186,35 +179,24 @@ int jk_direct(Df *df, const double *C, int prec, double *J, double *K, cudaStrea
   k_lower_gemv_t<<<nb(naux, 128), 128, 0, s>>>(df->Linv.as<double>(), naux, cvec, gam);
   BQC_LAUNCH_CHECK();  // gam now holds c
   // K
+  const bool raw_lost = !mixed;  // the FP64 solve and K use the buffer as scratch
   if (mixed) {
     BQC_TRY(direct_mixed_finish(df, split, K, s));
   } else {
     BQC_TRY(trsm_lower_left(ctx, df->L.as<double>(), naux, df->Xraw.as<double>(),
                             (int64_t)n * no, (int64_t)n * no, df->raw.p, df->raw.n, s));
-    Gemm64Args k;
-    k.M = n;
-    k.N = n;
-    k.K1 = naux;
-    k.K2 = no;
-    k.A = df->Xraw.as<double>();
-    k.lda = no;
-    k.sA1 = (int64_t)n * no;
-    k.B = k.A;
-    k.ldb = no;
-    k.sB1 = (int64_t)n * no;
-    k.C = K;
-    k.ldc = n;
-    k.lower_only = 1;
-    k.mirror = 1;
-    BQC_TRY(launch_gemm64(kAN, true, k, s));
+    BQC_TRY(k_of_x(ctx, df->Xraw.as<double>(), n, no, naux, df->raw.p, df->raw.n, K, s));
   }
   df->mark(3, s);
-  // pass 2: J = sum_Q c_Q (Q|..)
+  // pass 2: J = sum_Q c_Q (Q|..), from the last block, which pass 1 left in the
+  // buffer, to the first
   BQC_CUDA_TRY(cudaMemsetAsync(df->Jp.p, 0, (size_t)npair * 8, s));
-  for (int q0 = 0; q0 < naux; q0 += bk) {
+  for (int q0 = q_last; q0 >= 0; q0 -= bk) {
     const int nq = std::min(bk, naux - q0);
-    BQC_CUDA_TRY(cudaMemsetAsync(raw, 0, (size_t)nq * npair * 8, s));
-    BQC_TRY(launch_eri3c(b, &df->plan, q0, q0 + nq, raw, npair, s));
+    if (q0 < q_last || raw_lost) {
+      BQC_CUDA_TRY(cudaMemsetAsync(raw, 0, (size_t)nq * npair * 8, s));
+      BQC_TRY(launch_eri3c(b, &df->plan, q0, q0 + nq, raw, npair, s));
+    }
     k_cols_axpy<<<nb(npair), 256, 0, s>>>(raw, nq, npair, gam + q0, df->Jp.as<double>());
     BQC_LAUNCH_CHECK();
   }

@@ -1466,25 +1466,81 @@ __global__ void __launch_bounds__(256) k_absmax_f64(const double *__restrict__ a
   if ((threadIdx.x & 31) == 0) atomic_max_nonneg(out, m);
 }
 
-// B (FP64 packed lower triangle) -> scaled full-square FP16 split shadows:
-// f = s_B B, Bh = fp16(f), Bl = fp16(f - Bh), rows zero-padded to ld.
-__global__ void k_expand_split16(const double *__restrict__ B, int n, int ld, int64_t npair,
-                                 int np, float sB, __half *__restrict__ Bh,
-                                 __half *__restrict__ Bl) {
-  const int64_t nn = (int64_t)n * ld;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nn * np) return;
-  const int64_t P = i / nn, rc = i % nn;
-  const int64_t r = rc / ld, c = rc % ld;
-  float h = 0.0f, l = 0.0f;
-  if (c < n) {
-    const int64_t hi = r > c ? r : c, lo = r > c ? c : r;
-    const float f = (float)(B[P * npair + hi * (hi + 1) / 2 + lo] * (double)sB);
-    h = __half2float(__float2half_rn(f));
-    l = f - h;
+// v as a float pair (hi, lo), hi = fl(v), lo = fl(v - hi), in integer
+// arithmetic: FP64 conversions run at the FP64 pipe's rate (1/64 of FP32),
+// which made a split of B four times slower than its memory traffic.
+__device__ __forceinline__ float2 split_pair(double v) {
+  const long long b = __double_as_longlong(v);
+  const int e = ((int)(b >> 52) & 0x7ff) - 1023;
+  if (e < -60 || e > 120) {  // zero, and magnitudes whose parts may leave float's normal range
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
   }
-  Bh[i] = __float2half_rn(h);
-  Bl[i] = __float2half_rn(l);
+  const long long m = (b & 0xfffffffffffffLL) | (1LL << 52);
+  // 24 leading bits, to nearest even
+  const int q = (int)((m + ((1LL << 28) - 1) + ((m >> 29) & 1)) >> 29);
+  const int rem = (int)(m - ((long long)q << 29));  // |rem| <= 2^28: v - hi = rem 2^(e - 52)
+  float h = __int_as_float((e + 127 - 23) << 23) * (float)q;
+  float l = __int_as_float((e + 127 - 52) << 23) * (float)rem;
+  if (b < 0) {
+    h = -h;
+    l = -l;
+  }
+  return make_float2(h, l);
+}
+
+// B (FP64 packed lower triangle) -> scaled full-square FP16 split shadows,
+// f = s_B fl(B), Bh = fp16(f), Bl = fp16(f - Bh), rows zero-padded to ld; and
+// the float pairs of the packed B for the J pass.  One 64 x 64 tile of one B_P
+// a block: B is read once and coalesced, its mirror image goes through shared
+// memory, FP16 pairs of columns are written (24 bytes a packed element of
+// traffic; (H2O)_24: 5.9 -> 2.0 ms with the former two kernels).
+__global__ void __launch_bounds__(256) k_expand_split16(const double *__restrict__ B, int n, int ld,
+                                                        int64_t npair, float sB,
+                                                        __half *__restrict__ Bh,
+                                                        __half *__restrict__ Bl,
+                                                        float2 *__restrict__ B2) {
+  __shared__ uint32_t t[64][65];  // Bh in the low half, Bl in the high half
+  const int64_t P = blockIdx.x;
+  const int y = blockIdx.y, tid = threadIdx.x;
+  int tm = (int)((sqrtf(8.0f * y + 1.0f) - 1.0f) * 0.5f);
+  while ((tm + 1) * (tm + 2) / 2 <= y) ++tm;
+  while (tm * (tm + 1) / 2 > y) --tm;
+  const int tn = y - tm * (tm + 1) / 2;
+#pragma unroll 4
+  for (int k = 0; k < 16; ++k) {
+    const int i = (tid >> 6) + 4 * k, j = tid & 63;
+    const int r = tm * 64 + i, c = tn * 64 + j;
+    uint32_t v = 0;
+    if (r < n && c <= r) {
+      const int64_t at = P * npair + (int64_t)r * (r + 1) / 2 + c;
+      const float2 p = split_pair(__ldg(B + at));
+      B2[at] = p;
+      const float f = p.x * sB;
+      const __half h = __float2half_rn(f), l = __float2half_rn(f - __half2float(h));
+      v = (uint32_t)__half_as_ushort(h) | ((uint32_t)__half_as_ushort(l) << 16);
+    }
+    if (tm != tn) {
+      t[i][j] = v;
+    } else if (j <= i) {
+      t[i][j] = v;
+      t[j][i] = v;
+    }
+  }
+  __syncthreads();
+  for (int side = 0; side < (tm == tn ? 1 : 2); ++side) {
+    const int r0 = (side ? tn : tm) * 64, c0 = (side ? tm : tn) * 64;
+#pragma unroll 4
+    for (int k = 0; k < 8; ++k) {
+      const int i = (tid >> 5) + 8 * k, j = 2 * (tid & 31);
+      const int r = r0 + i, c = c0 + j;
+      if (r >= n || c >= ld) continue;  // ld is even: both columns or none
+      const uint32_t u = side ? t[j][i] : t[i][j], w = side ? t[j + 1][i] : t[i][j + 1];
+      const int64_t o = (P * n + r) * ld + c;
+      *reinterpret_cast<uint32_t *>(Bh + o) = __byte_perm(u, w, 0x5410);
+      *reinterpret_cast<uint32_t *>(Bl + o) = __byte_perm(u, w, 0x7632);
+    }
+  }
 }
 
 // *out = max over rows of sum_c Bh[row][c]^2 (one warp per row; float bits).
@@ -1840,10 +1896,13 @@ static int mixed_setup_f16(Df *df, MixedState *ms, cudaStream_t s) {
   BQC_TRY(ms->Bh16.alloc(ctx, (size_t)naux * n * m.ld16 * 2));
   BQC_TRY(ms->Bl16.alloc(ctx, (size_t)naux * n * m.ld16 * 2));
   {
-    const int64_t tot = (int64_t)n * m.ld16 * naux;
-    k_expand_split16<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(
-        df->B64.as<double>(), n, m.ld16, df->npair, naux, sB, ms->Bh16.as<__half>(),
-        ms->Bl16.as<__half>());
+    // also the float-pair B for the J pass on the FP32 pipe (8 bytes per packed
+    // element, like the FP64 B it is split from)
+    BQC_TRY(jpass_ff_alloc(df));
+    const unsigned nt = (unsigned)((n + 63) / 64);
+    k_expand_split16<<<dim3((unsigned)naux, nt * (nt + 1) / 2), 256, 0, s>>>(
+        df->B64.as<double>(), n, m.ld16, df->npair, sB, ms->Bh16.as<__half>(),
+        ms->Bl16.as<__half>(), df->B2f.as<float2>());
     BQC_LAUNCH_CHECK();
   }
   BQC_CUDA_TRY(cudaMemsetAsync(stat.p, 0, 256, s));
@@ -1856,9 +1915,6 @@ static int mixed_setup_f16(Df *df, MixedState *ms, cudaStream_t s) {
   std::memcpy(&maxsq, &hb, 4);
   // |B row| <= |Bh row| / (1 - 2^-11); the factor also covers the float sums
   ms->rownorm = std::sqrt((double)maxsq) / (double)sB * (1.0 + 1.0 / 256.0);
-  // float-pair B for the J pass on the FP32 pipe (8 bytes per packed
-  // element, like the FP64 B it is split from)
-  BQC_TRY(jpass_ff_setup(df, s));
   {  // room for the J partials of the pieces
     const int np = j_pieces(naux, df->npair);
     int slices = 0;
