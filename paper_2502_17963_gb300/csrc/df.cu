@@ -397,11 +397,7 @@ int jpass_fp64_range(Df *df, int P0, int P1, int y0, cudaStream_t s) {
 int jpass_ff_alloc(Df *df) {
   const int64_t count = (int64_t)df->naux_loc * df->npair;
   BQC_TRY(df->B2f.alloc(df->ctx, (size_t)count * 8));
-  BQC_TRY(df->w2f.alloc(df->ctx, (size_t)df->naux_loc * 8));
-  k_split_ff<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(df->B64.as<double>(), count,
-                                                             df->B2f.as<float2>());
-  BQC_LAUNCH_CHECK();
-  return BQC_OK;
+  return df->w2f.alloc(df->ctx, (size_t)df->naux_loc * 8);
 }
 
 int jpass_ff_range(Df *df, int P0, int P1, int y0, cudaStream_t s) {
@@ -620,6 +616,8 @@ static OzJkPlan oz_jk_layout(int n, int no, int pc, int ns) {
 // Splits of a K contraction of length K: the count whose tiles fill whole waves
 // best, splits of at least one accumulation chain (128).
 static int oz_k_splits(int n, int K) {
+  const int64_t tiles = oz_tiles(n, n, true);
+  const int nsm = sm_count();
   int ns = 1;
   double eff = 0.0;
   for (int c = 1; c <= 2 * nsm && (c == 1 || c * 128 <= K); ++c) {
@@ -635,8 +633,6 @@ static int oz_k_splits(int n, int K) {
 }
 
 static OzJkPlan oz_jk_plan(int n, int naux, int no, size_t bytes) {
-  const int64_t tiles = oz_tiles(n, n, true);
-  const int nsm = sm_count();
   OzJkPlan best;
   for (int chunks = 1; chunks <= 64 && chunks <= naux; ++chunks) {
     const int pc = (naux + chunks - 1) / chunks;
@@ -644,14 +640,14 @@ static OzJkPlan oz_jk_plan(int n, int naux, int no, size_t bytes) {
     if (p.total <= bytes) return p;
   }
   return best;
+}
+
 static int oz_rows_of_b(const double *b, int64_t npair, int n, int np, void *slices, int *exps,
                         OzOperand *o, cudaStream_t s);
 static int oz_rows_of_x(const double *X, int n, int no, int np, int ns, void *slices, int *exps,
                         OzOperand *o, cudaStream_t s);
 static int oz_rows_of_c(const double *C, int n, int no, void *slices, int *exps, OzOperand *o,
                         cudaStream_t s);
-
-}
 
 static size_t x64_bytes(int n, int naux, int no) {
   const size_t x = (size_t)naux * n * no * 8;
@@ -964,6 +960,8 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
   }
   // the FP64 X buffer (stored) or the raw block (direct), first used as the
   // scratch of the factorisation and of the metric solve
+  DBuf &scr = mode == BQC_DF_STORED ? df->X64 : df->raw;
+  df->aux_block = std::max(1, std::min(o.aux_block, naux));
   // direct mode: blocks of equal size (in multiples of 32, X's storage blocks;
   // a block is padded to the largest), so that none is mostly padding and the
   // one that the second integral pass finds in the buffer is no remainder
@@ -971,8 +969,6 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
     const int nblk = (naux + df->aux_block - 1) / df->aux_block;
     df->aux_block = std::min(df->aux_block, ((naux + nblk - 1) / nblk + 31) / 32 * 32);
   }
-  DBuf &scr = mode == BQC_DF_STORED ? df->X64 : df->raw;
-  df->aux_block = std::max(1, std::min(o.aux_block, naux));
   if ((st = scr.alloc(ctx, mode == BQC_DF_STORED ? x64_bytes(n, df->naux_loc, no)
                                                  : (size_t)df->aux_block * npair * 8)) != BQC_OK)
     return fail(st);

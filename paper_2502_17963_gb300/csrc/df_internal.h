@@ -66,8 +66,8 @@ struct Df {
   DBuf raw;    // aux block x Npair FP64 raw integrals
   DBuf Linv;   // Naux x Naux FP64 L^{-1}
   DBuf Xraw;   // FP64 path: Naux x N x nocc, then Y = L^{-1} X in place
-  DBuf gamma;  // Naux FP64: gamma_Q = (Q|D), then c = V^{-1} gamma
   DBuf Xscr;   // FP64 path: slices of the X pass
+  DBuf gamma;  // Naux FP64: gamma_Q = (Q|D), then c = V^{-1} gamma
   DBuf D2;     // Npair FP64 packed density, off-diagonal doubled
   DBuf Kpart64;
   int aux_block = 1024;
@@ -125,7 +125,6 @@ int jk_mixed_stored(Df *df, const double *C, int prec, double *J, double *K, cud
 // on the split-FP16 tensor cores; BQC_E_UNSUPPORTED without FP16 shadows.
 int jk_k_rank2(Df *df, const double *Cw, const double *Cd, double *K, cudaStream_t s);
 int jk_fp64_stored(Df *df, const double *C, double *J, double *K, cudaStream_t s);
-// J = sum_P w_P B_P from the packed FP64 B and df->w (FP64), full symmetric.
 // X_P = B_P C (np packed rows b, X[P][mu][i]) and K = sum_P X_P X_P^T in FP64,
 // sliced on the tensor cores where the scratch allows, else on the DFMA GEMM.
 size_t x_of_b_bytes(int n, int no, int np);  // scratch for all rows at once
@@ -133,6 +132,7 @@ int x_of_b(Ctx *ctx, const double *b, int64_t npair, const double *C, int n, int
            double *X, void *scratch, size_t bytes, cudaStream_t s);
 int k_of_x(Ctx *ctx, const double *X, int n, int no, int naux, void *scratch, size_t bytes,
            double *K, cudaStream_t s);
+// J = sum_P w_P B_P from the packed FP64 B and df->w (FP64), full symmetric.
 int jpass_fp64(Df *df, double *J, cudaStream_t s);
 // The FP64 J pass in pieces: partials of aux functions [P0, P1) (df->w) into
 // partial slices starting at y0, then the sum of nslice slices into J.
