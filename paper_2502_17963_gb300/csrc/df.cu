@@ -50,43 +50,41 @@ __global__ void __launch_bounds__(1024) k_wdot(const double *X, const double *C,
 
 // J pass over packed FP64 B: out[col] = sum_{P in [Pa, Pb)} w_P B[P][col] for
 // the two adjacent columns c2, c2 + 1 a thread owns; P streams in increasing
-// order (one read of B, coalesced), eight 16-byte loads in flight per thread.
+// order (one read of B, coalesced), eight 16-byte loads in flight per thread,
+// or, for an odd number of columns (every second row off a 16-byte boundary:
+// half of all sizes), sixteen 8-byte ones.
 __device__ __forceinline__ void jpass64_cols(const double *__restrict__ B,
                                              const double *__restrict__ w, int Pa, int Pb,
                                              int64_t npair, int64_t c2, double *__restrict__ out) {
   double a0 = 0.0, a1 = 0.0;
-  if (c2 + 1 < npair && (npair % 2 == 0)) {
-    const double2 *b2 = reinterpret_cast<const double2 *>(B + c2);
-    const int64_t st = npair / 2;
-    int P = Pa;
-    for (; P + 8 <= Pb; P += 8) {
-      double2 v[8];
+  const bool two = c2 + 1 < npair, even = npair % 2 == 0;
+  const double *b = B + c2 + (int64_t)Pa * npair;
+  const int o1 = two ? 1 : 0;
+  auto load = [&](int64_t k) {
+    const double *p = b + k * npair;
+    return even ? __ldg(reinterpret_cast<const double2 *>(p))
+                : make_double2(__ldg(p), __ldg(p + o1));
+  };
+  int P = Pa;
+  for (; P + 8 <= Pb; P += 8, b += 8 * npair) {
+    double2 v[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = __ldg(b2 + (int64_t)(P + k) * st);
+    for (int k = 0; k < 8; ++k) v[k] = load(k);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const double wp = __ldg(w + P + k);
-        a0 = fma(wp, v[k].x, a0);
-        a1 = fma(wp, v[k].y, a1);
-      }
+    for (int k = 0; k < 8; ++k) {
+      const double wp = __ldg(w + P + k);
+      a0 = fma(wp, v[k].x, a0);
+      a1 = fma(wp, v[k].y, a1);
     }
-    for (; P < Pb; ++P) {
-      const double2 v = __ldg(b2 + (int64_t)P * st);
-      const double wp = __ldg(w + P);
-      a0 = fma(wp, v.x, a0);
-      a1 = fma(wp, v.y, a1);
-    }
-    out[c2] = a0;
-    out[c2 + 1] = a1;
-  } else {
-    for (int P = Pa; P < Pb; ++P) {
-      const double wp = __ldg(w + P);
-      a0 = fma(wp, B[(int64_t)P * npair + c2], a0);
-      if (c2 + 1 < npair) a1 = fma(wp, B[(int64_t)P * npair + c2 + 1], a1);
-    }
-    out[c2] = a0;
-    if (c2 + 1 < npair) out[c2 + 1] = a1;
   }
+  for (; P < Pb; ++P, b += npair) {
+    const double2 v = load(0);
+    const double wp = __ldg(w + P);
+    a0 = fma(wp, v.x, a0);
+    a1 = fma(wp, v.y, a1);
+  }
+  out[c2] = a0;
+  if (two) out[c2 + 1] = a1;
 }
 
 // Jp[y][col] = sum_{P in chunk y} w_P B[P][col]: gridDim.y aux chunks give
@@ -141,43 +139,35 @@ __device__ __forceinline__ void jpass_ff_cols(const float4 *__restrict__ B2,
                                               int64_t npair, int64_t c2,
                                               double *__restrict__ out) {
   float h0 = 0.0f, l0 = 0.0f, h1 = 0.0f, l1 = 0.0f;
-  if (c2 + 1 < npair && (npair % 2 == 0)) {
-    const float4 *b = B2 + c2 / 2;
-    const int64_t st = npair / 2;
-    int P = Pa;
-    for (; P + 8 <= Pb; P += 8) {
-      float4 v[8];
+  const bool two = c2 + 1 < npair, even = npair % 2 == 0;
+  const float2 *b = reinterpret_cast<const float2 *>(B2) + c2 + (int64_t)Pa * npair;
+  const int o1 = two ? 1 : 0;
+  auto load = [&](int64_t k) {  // as in jpass64_cols
+    const float2 *p = b + k * npair;
+    if (even) return __ldg(reinterpret_cast<const float4 *>(p));
+    const float2 x = __ldg(p), y = __ldg(p + o1);
+    return make_float4(x.x, x.y, y.x, y.y);
+  };
+  int P = Pa;
+  for (; P + 8 <= Pb; P += 8, b += 8 * npair) {
+    float4 v[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = __ldg(b + (int64_t)(P + k) * st);
+    for (int k = 0; k < 8; ++k) v[k] = load(k);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const float2 wp = __ldg(w2 + P + k);
-        ff_acc(h0, l0, wp.x, wp.y, v[k].x, v[k].y);
-        ff_acc(h1, l1, wp.x, wp.y, v[k].z, v[k].w);
-      }
+    for (int k = 0; k < 8; ++k) {
+      const float2 wp = __ldg(w2 + P + k);
+      ff_acc(h0, l0, wp.x, wp.y, v[k].x, v[k].y);
+      ff_acc(h1, l1, wp.x, wp.y, v[k].z, v[k].w);
     }
-    for (; P < Pb; ++P) {
-      const float4 v = __ldg(b + (int64_t)P * st);
-      const float2 wp = __ldg(w2 + P);
-      ff_acc(h0, l0, wp.x, wp.y, v.x, v.y);
-      ff_acc(h1, l1, wp.x, wp.y, v.z, v.w);
-    }
-    out[c2] = (double)h0 + (double)l0;
-    out[c2 + 1] = (double)h1 + (double)l1;
-  } else {
-    const float2 *b = reinterpret_cast<const float2 *>(B2);
-    for (int P = Pa; P < Pb; ++P) {
-      const float2 wp = __ldg(w2 + P);
-      const float2 v0 = __ldg(b + (int64_t)P * npair + c2);
-      ff_acc(h0, l0, wp.x, wp.y, v0.x, v0.y);
-      if (c2 + 1 < npair) {
-        const float2 v1 = __ldg(b + (int64_t)P * npair + c2 + 1);
-        ff_acc(h1, l1, wp.x, wp.y, v1.x, v1.y);
-      }
-    }
-    out[c2] = (double)h0 + (double)l0;
-    if (c2 + 1 < npair) out[c2 + 1] = (double)h1 + (double)l1;
   }
+  for (; P < Pb; ++P, b += npair) {
+    const float4 v = load(0);
+    const float2 wp = __ldg(w2 + P);
+    ff_acc(h0, l0, wp.x, wp.y, v.x, v.y);
+    ff_acc(h1, l1, wp.x, wp.y, v.z, v.w);
+  }
+  out[c2] = (double)h0 + (double)l0;
+  if (two) out[c2 + 1] = (double)h1 + (double)l1;
 }
 
 __global__ void __launch_bounds__(256) k_jpass_ff_range(const float4 *__restrict__ B2,
@@ -293,14 +283,23 @@ __global__ void k_pack_sym2(const double *__restrict__ D, int n, double *__restr
   D2[i] = (mu == nu ? 1.0 : 2.0) * D[(int64_t)mu * n + nu];
 }
 
-// w[P] = sum_c B[P][c] D2[c] over the packed FP64 B (one block per P).
+// w[P] = sum_c B[P][c] D2[c] over the packed FP64 B (one block per P; four
+// loads of B in flight a thread).
 __global__ void __launch_bounds__(256) k_bdot(const double *__restrict__ B, int64_t npair,
                                               const double *__restrict__ D2, double *w) {
   const double *b = B + (int64_t)blockIdx.x * npair;
-  double s = 0.0;
-  for (int64_t c = threadIdx.x; c < npair; c += blockDim.x) s = fma(b[c], D2[c], s);
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  int64_t c = threadIdx.x;
+  for (; c + 3 * 256 < npair; c += 4 * 256) {
+    double v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __ldg(b + c + 256 * k);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = fma(v[k], __ldg(D2 + c + 256 * k), s[k]);
+  }
+  for (; c < npair; c += 256) s[0] = fma(__ldg(b + c), __ldg(D2 + c), s[0]);
   __shared__ double red[256];
-  red[threadIdx.x] = s;
+  red[threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
   __syncthreads();
   for (int o = 128; o > 0; o >>= 1) {
     if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
@@ -324,28 +323,45 @@ __global__ void k_pack_sym2_ff(const double *__restrict__ D, int n, float2 *__re
 
 // w[P] = sum_c B[P][c] D2[c] from the float pairs of B and D2 in float-float
 // arithmetic (one block per P; the block's partial pairs summed in FP64);
-// also w as float pairs for the J pass.
+// also w as float pairs for the J pass.  Bound by the read of B: four
+// independent 16-byte loads of it in flight a thread (a row that starts off a
+// 16-byte boundary is peeled by one element).
 __global__ void __launch_bounds__(256) k_bdot_ff(const float2 *__restrict__ B2, int64_t npair,
                                                  const float2 *__restrict__ D2, double *w,
                                                  float2 *w2) {
-  const float2 *b = B2 + (int64_t)blockIdx.x * npair;
-  float h = 0.0f, l = 0.0f;
-  if (npair % 2 == 0) {
-    const float4 *b4 = reinterpret_cast<const float4 *>(b);
-    const float4 *d4 = reinterpret_cast<const float4 *>(D2);
-    for (int64_t c = threadIdx.x; c < npair / 2; c += blockDim.x) {
-      const float4 x = __ldg(b4 + c), d = __ldg(d4 + c);
-      ff_acc(h, l, d.x, d.y, x.x, x.y);
-      ff_acc(h, l, d.z, d.w, x.z, x.w);
-    }
-  } else {
-    for (int64_t c = threadIdx.x; c < npair; c += blockDim.x) {
-      const float2 x = __ldg(b + c), d = __ldg(D2 + c);
-      ff_acc(h, l, d.x, d.y, x.x, x.y);
+  const int64_t at = (int64_t)blockIdx.x * npair;
+  const int peel = (int)(at & 1);
+  const float2 *b = B2 + at + peel, *d = D2 + peel;
+  const int64_t n2 = (npair - peel) / 2;
+  float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, l[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  const float4 *b4 = reinterpret_cast<const float4 *>(b);
+  int64_t c = threadIdx.x;
+  for (; c + 3 * 256 < n2; c += 4 * 256) {
+    float4 x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = __ldg(b4 + c + 256 * k);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 d0 = __ldg(d + 2 * (c + 256 * k)), d1 = __ldg(d + 2 * (c + 256 * k) + 1);
+      ff_acc(h[k], l[k], d0.x, d0.y, x[k].x, x[k].y);
+      ff_acc(h[k], l[k], d1.x, d1.y, x[k].z, x[k].w);
     }
   }
+  for (; c < n2; c += 256) {
+    const float4 x = __ldg(b4 + c);
+    const float2 d0 = __ldg(d + 2 * c), d1 = __ldg(d + 2 * c + 1);
+    ff_acc(h[0], l[0], d0.x, d0.y, x.x, x.y);
+    ff_acc(h[0], l[0], d1.x, d1.y, x.z, x.w);
+  }
+  if (threadIdx.x == 0) {  // the peeled first and an odd last element
+    const float2 *b0 = B2 + at;
+    if (peel) ff_acc(h[1], l[1], D2[0].x, D2[0].y, b0[0].x, b0[0].y);
+    const int64_t e = npair - 1;
+    if ((npair - peel) & 1) ff_acc(h[2], l[2], D2[e].x, D2[e].y, b0[e].x, b0[e].y);
+  }
   __shared__ double red[256];
-  red[threadIdx.x] = (double)h + (double)l;
+  red[threadIdx.x] = (((double)h[0] + (double)l[0]) + ((double)h[1] + (double)l[1])) +
+                     (((double)h[2] + (double)l[2]) + ((double)h[3] + (double)l[3]));
   __syncthreads();
   for (int o = 128; o > 0; o >>= 1) {
     if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
