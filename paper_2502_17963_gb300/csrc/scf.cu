@@ -25,6 +25,7 @@
 
 #include "bqc_internal.h"
 #include "df_internal.h"
+#include "eigh.h"
 
 namespace bqc {
 
@@ -121,6 +122,68 @@ __global__ void k_inc_fock(int64_t n, const double *Fref, const double *Jp, cons
                            const double *Kp, const double *Km, double *F) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) F[i] = Fref[i] + 2.0 * (Jp[i] - Jm[i]) - (Kp[i] - Km[i]);
+}
+
+// The scalars of an SCF iteration in two launches and one copy to the host
+// (one library call and synchronisation each before): dot products a . b, and
+// for b == nullptr the largest |a|.  kDotBlocks partials each, summed in a
+// fixed order.
+constexpr int kDotBlocks = 64, kMaxDots = 40;
+struct DotArgs {
+  const double *a[kMaxDots], *b[kMaxDots];
+  int64_t n[kMaxDots];
+};
+
+__global__ void __launch_bounds__(256) k_dots(const __grid_constant__ DotArgs g, double *part) {
+  const double *a = g.a[blockIdx.y], *b = g.b[blockIdx.y];
+  const int64_t n = g.n[blockIdx.y];
+  double s = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += kDotBlocks * 256) {
+    if (b) {
+      s = fma(a[i], b[i], s);
+    } else {
+      const double v = fabs(a[i]);
+      s = v > s || isnan(v) ? v : s;
+    }
+  }
+  __shared__ double red[256];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) {
+      const double x = red[threadIdx.x], y = red[threadIdx.x + o];
+      red[threadIdx.x] = b ? x + y : (y > x || isnan(y) ? y : x);
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[blockIdx.y * kDotBlocks + blockIdx.x] = red[0];
+}
+
+__global__ void k_dots_sum(const __grid_constant__ DotArgs g, const double *part, int nd,
+                           double *out) {
+  const int k = threadIdx.x;
+  if (k >= nd) return;
+  double s = 0.0;
+#pragma unroll 8
+  for (int q = 0; q < kDotBlocks; ++q) {
+    const double v = part[k * kDotBlocks + q];
+    s = g.b[k] ? s + v : (v > s || isnan(v) ? v : s);
+  }
+  out[k] = s;
+}
+
+// out = sum over k < m of c[k] F[k]
+struct MixArgs {
+  const double *f[kMaxDots];
+  double c[kMaxDots];
+  int m;
+};
+__global__ void k_mix(int64_t n, const __grid_constant__ MixArgs g, double *out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double s = 0.0;
+  for (int k = 0; k < g.m; ++k) s = fma(g.c[k], g.f[k][i], s);
+  out[i] = s;
 }
 
 static inline unsigned nblk(int64_t n) { return (unsigned)((n + 255) / 256); }
@@ -256,15 +319,26 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
   BQC_LAUNCH_CHECK();
   const double one = 1.0, zero = 0.0;
   double *Xp = X.as<double>();
+  SmallGemm small;
+  EighRefiner refiner;
+  BQC_TRY(small.reserve(ctx, n));
+  BQC_TRY(refiner.reserve(ctx, w.sol, nmo));
+  // C (m x k) = op(A) op(B), column-major
+  auto mm = [&](bool tA, bool tB, int m, int cols, int k, const double *A, int lda, const double *B,
+                int ldb, double *Cm, int ldc) -> int {
+    if (small.takes(m, cols, k)) return small.run(tA, tB, m, cols, k, A, lda, B, ldb, Cm, ldc, s);
+    BQC_BLAS_TRY(cublasDgemm(w.blas, tA ? CUBLAS_OP_T : CUBLAS_OP_N, tB ? CUBLAS_OP_T : CUBLAS_OP_N,
+                             m, cols, k, &one, A, lda, B, ldb, &zero, Cm, ldc));
+    return BQC_OK;
+  };
   // diagonalise X^T M X -> C (n x nmo, column-major), eps
   auto diag = [&](const double *M) -> int {
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, nmo, n, &one, M, n, Xp, n,
-                             &zero, t1.as<double>(), n));
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_T, CUBLAS_OP_N, nmo, nmo, n, &one, Xp, n,
-                             t1.as<double>(), n, &zero, Fp.as<double>(), nmo));
-    BQC_TRY(eigh(w, ctx, Fp.as<double>(), nmo, ev.as<double>(), work, info, s));
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, nmo, nmo, &one, Xp, n,
-                             Fp.as<double>(), nmo, &zero, Cc.as<double>(), n));
+    BQC_TRY(mm(false, false, n, nmo, n, M, n, Xp, n, t1.as<double>(), n));
+    BQC_TRY(mm(true, false, nmo, nmo, n, Xp, n, t1.as<double>(), n, Fp.as<double>(), nmo));
+    bool done = false;
+    BQC_TRY(refiner.run(w.sol, small, Fp.as<double>(), nmo, ev.as<double>(), &done, s));
+    if (!done) BQC_TRY(eigh(w, ctx, Fp.as<double>(), nmo, ev.as<double>(), work, info, s));
+    BQC_TRY(mm(false, false, n, nmo, nmo, Xp, n, Fp.as<double>(), nmo, Cc.as<double>(), n));
     return BQC_OK;
   };
   BQC_TRY(diag(H.as<double>()));
@@ -278,6 +352,12 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
     BQC_TRY(hF[i].alloc(ctx, nn * 8));
     BQC_TRY(hE[i].alloc(ctx, (size_t)nmo * nmo * 8));
   }
+  // scalars of an iteration: energy, largest error, and the error's dot
+  // products with the stored ones (a larger subspace takes the library calls)
+  const bool fused_dots = space + 2 <= kMaxDots;
+  DBuf dots;
+  std::vector<double> hdots(kMaxDots, 0.0);
+  BQC_TRY(dots.alloc(ctx, (size_t)kMaxDots * (kDotBlocks + 1) * 8));
   std::vector<int> slot;  // DIIS entries in age order (slot indices)
   std::vector<double> Bm; // Gram matrix of errors in age order
   int stage = o.prec;
@@ -339,8 +419,7 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
   // errors of successive increments do not accumulate (no graph: the
   // eigen-decomposition reads its status on the host).
   auto incremental_build = [&]() -> int {
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_T, n, n, no, &one, Cc.as<double>(), n,
-                             Cc.as<double>(), n, &zero, Dk.as<double>(), n));
+    BQC_TRY(mm(false, true, n, n, no, Cc.as<double>(), n, Cc.as<double>(), n, Dk.as<double>(), n));
     const double mone = -1.0;
     BQC_BLAS_TRY(cublasDgeam(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, n, &one, Dk.as<double>(), n,
                              &mone, Dref.as<double>(), n, t1.as<double>(), n));
@@ -361,14 +440,11 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
       // Ct Ct^T = D_k), then dD = Cw Cd^T + Cd Cw^T with Cw = (Ca + Ct) / 2
       // and Cd = Ct - Ca small; K[dD] from W = B Cw and DY = B Cd carries
       // rounding relative to |W||DY|, not to |D|.
-      BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, no, n, &one, S.as<double>(),
-                               n, Ca.as<double>(), n, &zero, Sca.as<double>(), n));
-      BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_T, CUBLAS_OP_N, no, no, n, &one, Cc.as<double>(),
-                               n, Sca.as<double>(), n, &zero, Mo.as<double>(), no));
+      BQC_TRY(mm(false, false, n, no, n, S.as<double>(), n, Ca.as<double>(), n, Sca.as<double>(), n));
+      BQC_TRY(mm(true, false, no, no, n, Cc.as<double>(), n, Sca.as<double>(), n, Mo.as<double>(), no));
       // R = M (M^T M)^(-1/2), the orthogonal polar factor of M (= U V^T of
       // its SVD), from the eigen-decomposition of M^T M = V diag(lam) V^T
-      BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_T, CUBLAS_OP_N, no, no, no, &one, Mo.as<double>(),
-                               no, Mo.as<double>(), no, &zero, Uo.as<double>(), no));
+      BQC_TRY(mm(true, false, no, no, no, Mo.as<double>(), no, Mo.as<double>(), no, Uo.as<double>(), no));
       BQC_TRY(eigh(w, ctx, Uo.as<double>(), no, So.as<double>(), work, info, s));
       double lam_min = 0.0;
       BQC_CUDA_TRY(cudaMemcpyAsync(&lam_min, So.p, 8, cudaMemcpyDeviceToHost, s));
@@ -380,12 +456,9 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
                                                                 So.as<double>(), VTo.as<double>());
       BQC_LAUNCH_CHECK();
       // Sca (n x no, no longer needed) holds T = V diag(lam^-1/2) V^T
-      BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_T, no, no, no, &one, VTo.as<double>(),
-                               no, Uo.as<double>(), no, &zero, Sca.as<double>(), no));
-      BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, no, no, no, &one, Mo.as<double>(),
-                               no, Sca.as<double>(), no, &zero, Ro.as<double>(), no));
-      BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, no, no, &one, Cc.as<double>(),
-                               n, Ro.as<double>(), no, &zero, Ct.as<double>(), n));
+      BQC_TRY(mm(false, true, no, no, no, VTo.as<double>(), no, Uo.as<double>(), no, Sca.as<double>(), no));
+      BQC_TRY(mm(false, false, no, no, no, Mo.as<double>(), no, Sca.as<double>(), no, Ro.as<double>(), no));
+      BQC_TRY(mm(false, false, n, no, no, Cc.as<double>(), n, Ro.as<double>(), no, Ct.as<double>(), n));
       k_procrustes_pair<<<nblk((int64_t)n * no), 256, 0, s>>>(n, no, Ca.as<double>(),
                                                               Ct.as<double>(), Vp.as<double>(),
                                                               Vm.as<double>());
@@ -492,8 +565,7 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
       BQC_TRY(fock_build(stage));
     }
     if (!last_incremental) ++(stage == BQC_PREC_FP64 ? res->builds_fp64 : res->builds_mixed);
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_T, n, n, no, &one, Cc.as<double>(), n,
-                             Cc.as<double>(), n, &zero, D.as<double>(), n));
+    BQC_TRY(mm(false, true, n, n, no, Cc.as<double>(), n, Cc.as<double>(), n, D.as<double>(), n));
     if (inc_stage && !last_incremental) {
       // an anchor: the reference of the next increments
       BQC_CUDA_TRY(cudaMemcpyAsync(Facc.p, F.p, nn * 8, cudaMemcpyDeviceToDevice, s));
@@ -502,21 +574,19 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
         BQC_CUDA_TRY(
             cudaMemcpyAsync(Ca.p, Cc.p, (size_t)n * no * 8, cudaMemcpyDeviceToDevice, s));
     }
+    // H + F, in Fx (free until the extrapolation below)
     k_axpby3<<<nblk(nn), 256, 0, s>>>(nn, H.as<double>(), 1.0, F.as<double>(), 1.0, nullptr, 0.0,
-                                      t2.as<double>());
+                                      Fx.as<double>());
     BQC_LAUNCH_CHECK();
     double eel = 0.0;
-    BQC_BLAS_TRY(cublasDdot(w.blas, (int)nn, D.as<double>(), 1, t2.as<double>(), 1, &eel));
-    E = eel + b->enuc;
+    if (!fused_dots)
+      BQC_BLAS_TRY(cublasDdot(w.blas, (int)nn, D.as<double>(), 1, Fx.as<double>(), 1, &eel));
     // e = X^T (F D S - S D F) X
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, n, n, &one, F.as<double>(), n,
-                             D.as<double>(), n, &zero, t1.as<double>(), n));
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, n, n, &one, t1.as<double>(), n,
-                             S.as<double>(), n, &zero, t2.as<double>(), n));
+    BQC_TRY(mm(false, false, n, n, n, F.as<double>(), n, D.as<double>(), n, t1.as<double>(), n));
+    BQC_TRY(mm(false, false, n, n, n, t1.as<double>(), n, S.as<double>(), n, t2.as<double>(), n));
     k_antisym<<<nblk(nn), 256, 0, s>>>(n, t2.as<double>(), t1.as<double>());
     BQC_LAUNCH_CHECK();
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_N, CUBLAS_OP_N, n, nmo, n, &one, t1.as<double>(),
-                             n, Xp, n, &zero, t2.as<double>(), n));
+    BQC_TRY(mm(false, false, n, nmo, n, t1.as<double>(), n, Xp, n, t2.as<double>(), n));
     // choose the DIIS slot for this iteration's error
     int sl;
     if ((int)slot.size() < space) {
@@ -528,14 +598,40 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
       sl = slot.front();
     }
     double *err = hE[sl].as<double>();
-    BQC_BLAS_TRY(cublasDgemm(w.blas, CUBLAS_OP_T, CUBLAS_OP_N, nmo, nmo, n, &one, Xp, n,
-                             t2.as<double>(), n, &zero, err, nmo));
-    int imax = 1;
-    BQC_BLAS_TRY(cublasIdamax(w.blas, nmo * nmo, err, 1, &imax));
-    double hv = 0.0;
-    BQC_CUDA_TRY(cudaMemcpyAsync(&hv, err + (imax - 1), 8, cudaMemcpyDeviceToHost, s));
-    BQC_CUDA_TRY(cudaStreamSynchronize(s));
-    emax = std::fabs(hv);
+    BQC_TRY(mm(true, false, nmo, nmo, n, Xp, n, t2.as<double>(), n, err, nmo));
+    if (fused_dots) {
+      DotArgs g;
+      g.a[0] = D.as<double>();
+      g.b[0] = Fx.as<double>();
+      g.n[0] = nn;
+      g.a[1] = err;
+      g.b[1] = nullptr;
+      g.n[1] = (int64_t)nmo * nmo;
+      for (int i = 0; i < space; ++i) {  // unused slots hold nothing: 0 elements
+        const bool used = i == sl || std::find(slot.begin(), slot.end(), i) != slot.end();
+        g.a[2 + i] = hE[i].as<double>();
+        g.b[2 + i] = err;
+        g.n[2 + i] = used ? (int64_t)nmo * nmo : 0;
+      }
+      double *part = dots.as<double>() + kMaxDots;
+      k_dots<<<dim3(kDotBlocks, (unsigned)(space + 2)), 256, 0, s>>>(g, part);
+      BQC_LAUNCH_CHECK();
+      k_dots_sum<<<1, 64, 0, s>>>(g, part, space + 2, dots.as<double>());
+      BQC_LAUNCH_CHECK();
+      BQC_CUDA_TRY(cudaMemcpyAsync(hdots.data(), dots.p, (size_t)(space + 2) * 8,
+                                   cudaMemcpyDeviceToHost, s));
+      BQC_CUDA_TRY(cudaStreamSynchronize(s));
+      eel = hdots[0];
+      emax = hdots[1];
+    } else {
+      int imax = 1;
+      BQC_BLAS_TRY(cublasIdamax(w.blas, nmo * nmo, err, 1, &imax));
+      double hv = 0.0;
+      BQC_CUDA_TRY(cudaMemcpyAsync(&hv, err + (imax - 1), 8, cudaMemcpyDeviceToHost, s));
+      BQC_CUDA_TRY(cudaStreamSynchronize(s));
+      emax = std::fabs(hv);
+    }
+    E = eel + b->enuc;
     if (res->history && res->history_len < res->history_cap) {
       double *h = res->history + 3 * (size_t)res->history_len++;
       h[0] = last_incremental ? -1.0 : stage;
@@ -636,8 +732,9 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
         for (int j = 0; j < m; ++j) nb[(size_t)i * (m + 1) + j] = Bm[(size_t)i * m + j];
       for (int i = 0; i <= m; ++i) {
         const int si = (i < m) ? slot[i] : sl;
-        double d = 0.0;
-        BQC_BLAS_TRY(cublasDdot(w.blas, nmo * nmo, hE[si].as<double>(), 1, err, 1, &d));
+        double d = hdots[std::min(2 + si, kMaxDots - 1)];
+        if (!fused_dots)
+          BQC_BLAS_TRY(cublasDdot(w.blas, nmo * nmo, hE[si].as<double>(), 1, err, 1, &d));
         nb[(size_t)i * (m + 1) + m] = d;
         nb[(size_t)m * (m + 1) + i] = d;
       }
@@ -649,10 +746,21 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
     if (m >= 2) {
       std::vector<double> c;
       if (diis_solve(Bm, m, c)) {
-        BQC_CUDA_TRY(cudaMemsetAsync(Fx.p, 0, nn * 8, s));
-        for (int i = 0; i < m; ++i)
-          BQC_BLAS_TRY(cublasDaxpy(w.blas, (int)nn, &c[i], hF[slot[i]].as<double>(), 1,
-                                   Fx.as<double>(), 1));
+        if (m <= kMaxDots) {
+          MixArgs g;
+          g.m = m;
+          for (int i = 0; i < m; ++i) {
+            g.c[i] = c[i];
+            g.f[i] = hF[slot[i]].as<double>();
+          }
+          k_mix<<<nblk(nn), 256, 0, s>>>(nn, g, Fx.as<double>());
+          BQC_LAUNCH_CHECK();
+        } else {
+          BQC_CUDA_TRY(cudaMemsetAsync(Fx.p, 0, nn * 8, s));
+          for (int i = 0; i < m; ++i)
+            BQC_BLAS_TRY(cublasDaxpy(w.blas, (int)nn, &c[i], hF[slot[i]].as<double>(), 1,
+                                     Fx.as<double>(), 1));
+        }
         Fuse = Fx.as<double>();
       }
     }

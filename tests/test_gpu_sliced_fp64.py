@@ -92,3 +92,23 @@ def test_metric_solve(gpu_ctx, bqc, name):
     raw = df.int3c_screened(0, basis.naux)
     bound = basis.naux * 2.0 ** -50 * (L.abs() @ B.abs()).amax()
     assert (L @ B - raw).abs().max() <= bound
+
+
+# n = 50, 150 (plain small products), 275 and 325 (sliced ones)
+@pytest.mark.parametrize("name", ["w2", "w6", "w11", "w13"])
+def test_scf_orbitals(gpu_ctx, bqc, name):
+    """The SCF's orbitals (refined from an FP32 decomposition): C^T S C = 1,
+    with C = X U, to n 2^-50 of |X|^2 |S| (the products' rounding and the
+    refinement's, 2^-53 of the same terms each); ascending energies."""
+    import torch
+    basis = bqc.Basis(gpu_ctx, workload.molecule_for(name))
+    df = bqc.DF(gpu_ctx, basis, keep_fp32=bqc.SHADOW_F16)
+    r = bqc.scf_run(gpu_ctx, df, prec=bqc.PREC_MIXED_F16X3, keep_arrays=True)
+    assert r["converged"]
+    S = bqc.one_electron(basis)[0]
+    C = torch.as_tensor(r["C"], device="cuda")
+    eps = torch.as_tensor(r["eps"], device="cuda")
+    n = basis.nbf
+    bound = n * 2.0 ** -50 * (C.abs().T @ S.abs() @ C.abs()).max()
+    assert (C.T @ S @ C - torch.eye(C.shape[1], device="cuda", dtype=C.dtype)).abs().max() <= bound
+    assert (eps[1:] >= eps[:-1]).all()
