@@ -87,54 +87,6 @@ __device__ __forceinline__ double boys_one(const double *__restrict__ tab, int m
   return f;
 }
 
-// F_m(T) for m = m0, m0 + step, ... <= mmax, scaled, into out[m]: the expansion
-// point and the powers' factors d / j are shared by the orders of a lane.
-__device__ __forceinline__ void boys_scaled(const double *__restrict__ tab, double T, double scale,
-                                            int m0, int step, int mmax,
-                                            double *__restrict__ out) {
-  if (T < kBoysTCut) {
-    const double x = fma(T, 1.0 / kBoysH, 6755399441055744.0);  // 1.5 2^52: k in the low word
-    const int k = __double2loint(x);
-    const double d = fma(x - 6755399441055744.0, kBoysH, -T);  // -(T - k h)
-    double dj[8];
-#pragma unroll
-    for (int j = 1; j < 8; ++j) dj[j] = d * (1.0 / j);
-    for (int m = m0; m <= mmax; m += step) {
-      const double *row = tab + (size_t)k * kBoysNM + m;
-      double r = __ldg(row + 7);
-#pragma unroll
-      for (int j = 7; j >= 1; --j) r = fma(r, dj[j], __ldg(row + j - 1));
-      out[m] = scale * r;
-    }
-    return;
-  }
-  const double e = exp(-T), inv2T = 0.5 / T;
-  double f = 0.5 * sqrt(3.141592653589793 / T);
-  for (int j = 0; j <= mmax; ++j) {
-    if (j >= m0 && (j - m0) % step == 0) out[j] = scale * f;
-    f = ((2 * j + 1) * f - e) * inv2T;
-  }
-}
-
-// k v for k = 1 .. KM from the multiples (an integer select: a conversion and
-// a product would be two more instructions of the FP64 pipe, which bounds these
-// kernels).
-template <int KM>
-struct Multiples {
-  double v[KM < 1 ? 1 : KM];
-  __device__ __forceinline__ explicit Multiples(double x) {
-    v[0] = x;
-#pragma unroll
-    for (int k = 1; k < KM; ++k) v[k] = v[k - 1] + x;
-  }
-  __device__ __forceinline__ double pick(int k) const {
-    double r = v[0];
-#pragma unroll
-    for (int q = 1; q < KM; ++q) r = k == q + 1 ? v[q] : r;
-    return r;
-  }
-};
-
 // --------------------------------------------------- OS/HGP engine -------
 
 template <int I, int N, class Fn>
@@ -293,11 +245,11 @@ __device__ __forceinline__ void os_vrr_accumulate(const PrimQ &g, const double *
   using O = Os<LA, LB, LC, LD>;
   constexpr int L = O::L, E = O::E, F = O::F;
   // level 0: [0|0]^m
-  boys_scaled(boys, g.T, g.pref, gl, G, L, s1);
+  {
+    const double e = g.T >= kBoysTCut ? exp(-g.T) : 0.0;
+    for (int m = gl; m <= L; m += G) s1[m] = g.pref * boys_one(boys, m, g.T, e);
+  }
   __syncwarp();
-  const Multiples<E - 1> mp(g.inv2p);
-  const Multiples<F - 1> mq(g.inv2q);
-  const Multiples<E> mpq(g.inv2pq);
   // bra levels e = 1..E on f = 0
   static_for<1, E + 1>([&](auto ei) {
     constexpr int e = decltype(ei)::value;
@@ -316,8 +268,7 @@ __device__ __forceinline__ void os_vrr_accumulate(const PrimQ &g, const double *
       if (nd >= 2) {
         i1[d] -= 1;
         const int e2 = cart_index(i1[0], i1[1], i1[2]);
-        v = fma(mp.pick(nd - 1),
-                fma(-g.rho_p, s1[e2 * (L + 1) + m + 1], s1[e2 * (L + 1) + m]), v);
+        v += (nd - 1) * g.inv2p * (s1[e2 * (L + 1) + m] - g.rho_p * s1[e2 * (L + 1) + m + 1]);
       }
       s1[ci * (L + 1) + m] = v;
     }
@@ -356,8 +307,7 @@ __device__ __forceinline__ void os_vrr_accumulate(const PrimQ &g, const double *
           j1[d] -= 1;
           const int f2 = cart_index(j1[0], j1[1], j1[2]) - ncum(f - 2);
           std::integral_constant<int, f - 2> lv2;
-          v = fma(mq.pick(nd - 1), fma(-g.rho_q, get(lv2, ecum, f2, m + 1), get(lv2, ecum, f2, m)),
-                  v);
+          v += (nd - 1) * g.inv2q * (get(lv2, ecum, f2, m) - g.rho_q * get(lv2, ecum, f2, m + 1));
         }
       }
       const int ed = ne[d];
@@ -365,7 +315,7 @@ __device__ __forceinline__ void os_vrr_accumulate(const PrimQ &g, const double *
         int i1[3] = {ne[0], ne[1], ne[2]};
         i1[d] -= 1;
         const int e1 = cart_index(i1[0], i1[1], i1[2]);
-        v = fma(mpq.pick(ed), get(lv1, e1, f1, m + 1), v);
+        v += ed * g.inv2pq * get(lv1, e1, f1, m + 1);
       }
       gk[O::loff(f) + (er * NF + fc) * LM + m] = v;
     }
@@ -614,11 +564,8 @@ __device__ __forceinline__ void eri3c_triplet(const Eri3cArgs &a, double *scr, i
       const int64_t col = (int64_t)mu * (mu + 1) / 2 + nu;
       const int64_t o = (int64_t)(P - a.p0) * a.ld + col;
       if (o < 0 || o >= a.out_elems) { atomicExch(a.flag, 3); continue; }
-      double v = res[idx];  // s and p components need no factor
-      if (LA >= 2) v *= c_cnorm[ncum(LA) + ia];
-      if (LB >= 2) v *= c_cnorm[ncum(LB) + ib];
-      if (LC >= 2) v *= c_cnorm[ncum(LC) + ic];
-      a.out[o] = v;
+      a.out[o] = res[idx] * c_cnorm[ncum(LA) + ia] * c_cnorm[ncum(LB) + ib] *
+                 c_cnorm[ncum(LC) + ic];
     }
   }
 }
