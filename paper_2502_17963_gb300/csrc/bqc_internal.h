@@ -203,9 +203,6 @@ struct Eri3cPlan {
   double tau = 0.0;
   DBuf d_pairs_sorted;  // int2 per pair, sorted within class
   DBuf d_qpair_sorted;  // double per pair
-  DBuf d_pair_data;     // primitive pairs of the sorted pairs, pair_stride doubles each
-  int pair_stride = 0;
-  mutable DBuf d_pair_data_orig;  // in the unsorted order, made by the first screening variant
   DBuf d_qaux;          // double per aux shell
   DBuf d_qpair;         // double per pair, in the basis' (unsorted) pair order
   DBuf d_prefix;        // per (pair class, aux l): n_aux(l)+1 int64 prefix

@@ -119,9 +119,7 @@ __global__ void __launch_bounds__(256) k_eri3c(Eri3cArgs a) {
       const int mid = (lo + hi) >> 1;
       if (a.prefix[mid] <= t) lo = mid; else hi = mid;
     }
-    const int64_t k = t - a.prefix[lo];
-    eri3c_triplet<LC, LA, LB>(a, scr, gl, a.aux_list[lo], a.pairs[k], active,
-                              a.pdata ? a.pdata + k * a.pstride : nullptr);
+    eri3c_triplet<LC, LA, LB>(a, scr, gl, a.aux_list[lo], a.pairs[t - a.prefix[lo]], active);
     __syncwarp();
   }
 }
@@ -181,11 +179,6 @@ int launch_eri3c_variant(const Basis *b, const Eri3cPlan *plan, int p0, int p1, 
   if (p0 < 0 || p1 > b->naux || p0 > p1 || variant < 0 || variant > 2) return BQC_E_INVALID;
   if (p0 == p1) return BQC_OK;
   DBuf list, count;
-  if (variant != 0 && plan->d_pair_data.p && !plan->d_pair_data_orig.p) {
-    int stride = 0;
-    BQC_TRY(pair_data_build(b, b->d_pairs.as<int2>(), b->npair_sh, &plan->d_pair_data_orig, &stride,
-                            s));
-  }
   if (variant == 2) {
     int64_t maxc = 0;
     for (int lc = 0; lc <= kMaxLAux; ++lc)
@@ -230,10 +223,6 @@ int launch_eri3c_variant(const Basis *b, const Eri3cPlan *plan, int p0, int p1, 
       a.aux = b->aux.dev;
       a.boys = b->ctx->boys;
       a.pairs = plan->d_pairs_sorted.as<int2>() + b->pair_off[cls];
-      a.pstride = plan->pair_stride;
-      a.pdata = plan->d_pair_data.p
-                    ? plan->d_pair_data.as<double>() + (int64_t)b->pair_off[cls] * a.pstride
-                    : nullptr;
       a.aux_list = b->d_aux_by_l.as<int>() + b->auxl_off[lc] + s0;
       a.prefix = plan->d_prefix.as<int64_t>() + plan->prefix_off[cls][lc] + s0;
       a.n_aux = s1 - s0;
@@ -244,9 +233,6 @@ int launch_eri3c_variant(const Basis *b, const Eri3cPlan *plan, int p0, int p1, 
       a.flag = b->ctx->flag;
       a.out_elems = (int64_t)(p1 - p0) * ld;
       a.pairs_orig = b->d_pairs.as<int2>() + b->pair_off[cls];
-      a.pdata_orig = plan->d_pair_data_orig.p ? plan->d_pair_data_orig.as<double>() +
-                                                    (int64_t)b->pair_off[cls] * a.pstride
-                                              : nullptr;
       a.qpair_orig = plan->d_qpair.as<double>() + b->pair_off[cls];
       a.qaux = plan->d_qaux.as<double>();
       a.tau = plan->tau;
@@ -382,7 +368,7 @@ __global__ void __launch_bounds__(256) k_int2c(Int2cArgs a) {
     if (!active) t = total - 1;
     const int iP = a.listP[t / a.nQ], iQ = a.listQ[t % a.nQ];
     const ShellRef sp = load_shell(a.aux, iP), sq = load_shell(a.aux, iQ);
-    const double *res = os_quartet<LP, 0, LQ, 0, G, true>(
+    const double *res = os_quartet<LP, 0, LQ, 0, G>(
         a.boys, scr, gl, sp, a.aux.exps + sp.poff, a.aux.coefs + sp.poff, nullptr, nullptr,
         nullptr, sq, a.aux.exps + sq.poff, a.aux.coefs + sq.poff, nullptr, nullptr, nullptr);
     if (active) {
@@ -498,9 +484,8 @@ __global__ void __launch_bounds__(256) k_nuclear(OneArgs a) {
       for (int ia = 0; ia < sa.nprim; ++ia)
         for (int ib = 0; ib < sb.nprim; ++ib) {
           PrimQ g;
-          prim_setup_point(make_pair(ea[ia], sa.xyz, eb[ib], sb.xyz, -Z * ca[ia] * cb[ib]), sa.xyz,
-                           C, g);
-          os_vrr_accumulate<LA, LB, 0, 0, G, true>(g, a.boys, acc, s1, nullptr, gl);
+          prim_setup(ea[ia], sa.xyz, eb[ib], sb.xyz, 0.0, C, 0.0, C, -Z * ca[ia] * cb[ib], 1, g);
+          os_vrr_accumulate<LA, LB, 0, 0, G>(g, a.boys, acc, s1, nullptr, gl);
         }
     }
     double AB[3], CD[3] = {0.0, 0.0, 0.0};
@@ -743,8 +728,6 @@ int eri3c_plan(const Basis *b, double tau, const double *V_diag_dev, cudaStream_
     }
     BQC_TRY(fork.join());
   }
-  BQC_TRY(pair_data_build(b, plan->d_pairs_sorted.as<int2>(), np, &plan->d_pair_data,
-                          &plan->pair_stride, s));
   // survivor counts and prefixes per (class, aux l)
   CutArgs ca;
   int64_t off = 0;

@@ -39,8 +39,7 @@ __global__ void __launch_bounds__(256) k_eri3c_ring(Eri3cArgs a) {
   auto consume = [&](int cnt) {
     const bool act = gw < cnt;
     const int64_t c = ring[(head + (act ? gw : 0)) & 63];
-    eri3c_triplet<LC, LA, LB>(a, scr, gl, a.aux_list[c / a.np], a.pairs_orig[c % a.np], act,
-                              a.pdata_orig ? a.pdata_orig + (c % a.np) * a.pstride : nullptr);
+    eri3c_triplet<LC, LA, LB>(a, scr, gl, a.aux_list[c / a.np], a.pairs_orig[c % a.np], act);
     __syncwarp();
     head += cnt;
   };
@@ -96,8 +95,7 @@ __global__ void __launch_bounds__(256) k_eri3c_list(Eri3cArgs a) {
     const bool active = t < total;
     if (!active) t = total - 1;
     const int64_t c = a.list[t];
-    eri3c_triplet<LC, LA, LB>(a, scr, gl, a.aux_list[c / a.np], a.pairs_orig[c % a.np], active,
-                              a.pdata_orig ? a.pdata_orig + (c % a.np) * a.pstride : nullptr);
+    eri3c_triplet<LC, LA, LB>(a, scr, gl, a.aux_list[c / a.np], a.pairs_orig[c % a.np], active);
     __syncwarp();
   }
 }

@@ -38,8 +38,6 @@ struct Jk4Args {
   ShellSetDev orb;
   const double *boys;
   const int2 *pX, *pY;      // sorted pairs of the two classes
-  const double *dX, *dY;    // their stored primitive pairs, or null
-  int pstride;
   const int64_t *prefix;    // npX + 1 kept-quartet prefix over the pairs of X
   int npX;
   int same;                 // X == Y
@@ -77,26 +75,18 @@ __global__ void __launch_bounds__(256) k_jk4c(Jk4Args a) {
     const int2 p = a.pX[lo], q = a.pY[jq];
     const ShellRef sa = load_shell(a.orb, p.x), sb = load_shell(a.orb, p.y);
     const ShellRef sc = load_shell(a.orb, q.x), sd = load_shell(a.orb, q.y);
-    double *res = const_cast<double *>(os_quartet<LA, LB, LC, LD, G>(
+    const double *res = os_quartet<LA, LB, LC, LD, G>(
         a.boys, scr, gl, sa, a.orb.exps + sa.poff, a.orb.coefs + sa.poff, &sb,
         a.orb.exps + sb.poff, a.orb.coefs + sb.poff, sc, a.orb.exps + sc.poff,
-        a.orb.coefs + sc.poff, &sd, a.orb.exps + sd.poff, a.orb.coefs + sd.poff,
-        a.dX ? a.dX + (int64_t)lo * a.pstride : nullptr,
-        a.dY ? a.dY + (int64_t)jq * a.pstride : nullptr));
-    // normalise once: each integral enters six contractions
-    for (int e = gl; e < O::NOUT; e += G) {
-      const int id = e % ND, ic = e / ND % NC, ib = e / (ND * NC) % NB, ia = e / (ND * NC * NB);
-      res[e] *= (c_cnorm[ncum(LA) + ia] * c_cnorm[ncum(LB) + ib]) *
-                (c_cnorm[ncum(LC) + ic] * c_cnorm[ncum(LD) + id]);
-    }
-    __syncwarp();
+        a.orb.coefs + sc.poff, &sd, a.orb.exps + sd.poff, a.orb.coefs + sd.poff);
     if (active) {
       double w = 1.0;
       if (p.x == p.y) w *= 0.5;
       if (q.x == q.y) w *= 0.5;
       if (a.same && jq == lo) w *= 0.5;
       auto val = [&](int ia, int ib, int ic, int id) {
-        return res[((ia * NB + ib) * NC + ic) * ND + id];
+        return res[((ia * NB + ib) * NC + ic) * ND + id] * c_cnorm[ncum(LA) + ia] *
+               c_cnorm[ncum(LB) + ib] * c_cnorm[ncum(LC) + ic] * c_cnorm[ncum(LD) + id];
       };
       const double *D = a.D;
       // J_ij += 2 w sum_kl v D_kl
@@ -229,8 +219,6 @@ struct Jk4Plan {
   int64_t total[kNPairClass][kNPairClass] = {{0}};
   int64_t kept = 0, candidates = 0;
   DBuf D, Jacc, Kacc;
-  DBuf pair_data;  // primitive pairs of the sorted pairs, pair_stride doubles each
-  int pair_stride = 0;
 };
 
 void Jk4Deleter::operator()(Jk4Plan *p) const { delete p; }
@@ -299,7 +287,6 @@ int jk4c_setup(Df *df, cudaStream_t s) {
   BQC_TRY(pl->prefix.alloc(ctx, pre.size() * 8));
   BQC_CUDA_TRY(cudaMemcpyAsync(pl->pairs.p, sp.data(), np * sizeof(int2), cudaMemcpyHostToDevice, s));
   BQC_CUDA_TRY(cudaMemcpyAsync(pl->prefix.p, pre.data(), pre.size() * 8, cudaMemcpyHostToDevice, s));
-  BQC_TRY(pair_data_build(b, pl->pairs.as<int2>(), np, &pl->pair_data, &pl->pair_stride, s));
   const int n = b->nbf;
   BQC_TRY(pl->D.alloc(ctx, (size_t)n * n * 8));
   BQC_TRY(pl->Jacc.alloc(ctx, (size_t)n * n * 8));
@@ -352,10 +339,6 @@ int jk_4c(Df *df, const double *C, int prec, double *J, double *K, cudaStream_t 
       if (pl->total[x][y] == 0) continue;
       a.pX = pl->pairs.as<int2>() + b->pair_off[x];
       a.pY = pl->pairs.as<int2>() + b->pair_off[y];
-      const double *pd = pl->pair_data.as<double>();
-      a.pstride = pl->pair_stride;
-      a.dX = pd ? pd + (int64_t)b->pair_off[x] * a.pstride : nullptr;
-      a.dY = pd ? pd + (int64_t)b->pair_off[y] * a.pstride : nullptr;
       a.prefix = pl->prefix.as<int64_t>() + pl->pre_off[x][y];
       a.npX = b->pair_off[x + 1] - b->pair_off[x];
       a.same = x == y;

@@ -149,85 +149,67 @@ struct PrimQ {
   double inv2p, rho_p, inv2q, rho_q, inv2pq, T, pref;
 };
 
-// One primitive pair: exponent sum p, its inverse, product centre P, and the
-// Gaussian product factor times the coefficients.
-struct PrimPair {
-  double p, ip, K, P[3];
-};
-constexpr int kPairDbl = 6;  // doubles of a stored PrimPair
-
-__device__ __forceinline__ PrimPair make_pair(double a, const double *A, double b, const double *B,
-                                              double w) {
-  PrimPair r;
-  r.p = a + b;
-  r.ip = 1.0 / r.p;
-  double AB2 = 0.0;
+// Geometry of a primitive quartet (a,b|c,d).  point != 0: ket is a point
+// charge at C (nuclear attraction): rho = p, W = C, prefactor 2 pi / p.
+__device__ __forceinline__ void prim_setup(double a, const double *A, double b, const double *B,
+                                           double c, const double *C, double d, const double *D,
+                                           double cabcd, int point, PrimQ &g) {
+  const double p = a + b, ip = 1.0 / p;
+  double P[3], AB2 = 0.0;
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
-    r.P[x] = (a * A[x] + b * B[x]) * r.ip;
+    P[x] = (a * A[x] + b * B[x]) * ip;
     const double t = A[x] - B[x];
     AB2 += t * t;
+    g.PA[x] = P[x] - A[x];
   }
-  r.K = w * exp(-a * b * r.ip * AB2);
-  return r;
-}
-
-__device__ __forceinline__ PrimPair load_pair(const double *__restrict__ d) {
-  PrimPair r;
-  r.p = __ldg(d);
-  r.ip = __ldg(d + 1);
-  r.K = __ldg(d + 2);
+  const double Kab = exp(-a * b * ip * AB2);
+  if (point) {
+    double PC2 = 0.0;
 #pragma unroll
-  for (int x = 0; x < 3; ++x) r.P[x] = __ldg(d + 3 + x);
-  return r;
-}
-
-// Point charge at C as the ket (nuclear attraction): rho = p, W = C, prefactor
-// 2 pi / p.
-__device__ __forceinline__ void prim_setup_point(const PrimPair &bra, const double *A,
-                                                 const double *C, PrimQ &g) {
-  double PC2 = 0.0;
+    for (int x = 0; x < 3; ++x) {
+      const double t = C[x] - P[x];
+      g.WP[x] = t;
+      PC2 += t * t;
+      g.QC[x] = 0.0;
+      g.WQ[x] = 0.0;
+    }
+    g.inv2p = 0.5 * ip;
+    g.rho_p = 1.0;
+    g.inv2q = g.rho_q = g.inv2pq = 0.0;
+    g.T = p * PC2;
+    g.pref = 2.0 * 3.141592653589793 * ip * Kab * cabcd;
+    return;
+  }
+  const double q = c + d, iq = 1.0 / q;
+  double Q[3], CD2 = 0.0;
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
-    const double t = C[x] - bra.P[x];
-    g.PA[x] = bra.P[x] - A[x];
-    g.WP[x] = t;
-    PC2 += t * t;
-    g.QC[x] = 0.0;
-    g.WQ[x] = 0.0;
+    Q[x] = (c * C[x] + d * D[x]) * iq;
+    const double t = C[x] - D[x];
+    CD2 += t * t;
+    g.QC[x] = Q[x] - C[x];
   }
-  g.inv2p = 0.5 * bra.ip;
-  g.rho_p = 1.0;
-  g.inv2q = g.rho_q = g.inv2pq = 0.0;
-  g.T = bra.p * PC2;
-  g.pref = 2.0 * 3.141592653589793 * bra.ip * bra.K;
-}
-
-// Geometry of a primitive quartet (a,b|c,d), A and C the first centres.
-__device__ __forceinline__ void prim_setup(const PrimPair &bra, const double *A,
-                                           const PrimPair &ket, const double *C, PrimQ &g) {
-  const double p = bra.p, q = ket.p;
+  const double Kcd = (d == 0.0) ? 1.0 : exp(-c * d * iq * CD2);
   const double ipq = 1.0 / (p + q);
   const double rho = p * q * ipq;
   double PQ2 = 0.0;
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
-    const double t = bra.P[x] - ket.P[x];
-    const double u = t * ipq;
-    g.PA[x] = bra.P[x] - A[x];
-    g.QC[x] = ket.P[x] - C[x];
-    g.WP[x] = -q * u;  // W - P = -q (P - Q) / (p + q)
-    g.WQ[x] = p * u;
+    const double W = (p * P[x] + q * Q[x]) * ipq;
+    g.WP[x] = W - P[x];
+    g.WQ[x] = W - Q[x];
+    const double t = P[x] - Q[x];
     PQ2 += t * t;
   }
-  g.inv2p = 0.5 * bra.ip;
-  g.rho_p = rho * bra.ip;
-  g.inv2q = 0.5 * ket.ip;
-  g.rho_q = rho * ket.ip;
+  g.inv2p = 0.5 * ip;
+  g.rho_p = rho * ip;
+  g.inv2q = 0.5 * iq;
+  g.rho_q = rho * iq;
   g.inv2pq = 0.5 * ipq;
   g.T = rho * PQ2;
   // 2 pi^{5/2} = 34.98683665524972
-  g.pref = 34.98683665524972 * bra.ip * ket.ip * sqrt(ipq) * bra.K * ket.K;
+  g.pref = 34.98683665524972 * ip * iq * sqrt(ipq) * Kab * Kcd * cabcd;
 }
 
 __device__ __forceinline__ int first_dir(const unsigned char *n) {
@@ -236,8 +218,7 @@ __device__ __forceinline__ int first_dir(const unsigned char *n) {
 
 // VRR for one primitive quartet and accumulation into acc.  Group-cooperative:
 // lane gl of G.  scr: S1 table then ket levels.  The caller syncs after.
-// KET1: the ket is a single centre (Q = C), so the QC terms vanish.
-template <int LA, int LB, int LC, int LD, int G, bool KET1>
+template <int LA, int LB, int LC, int LD, int G>
 __device__ __forceinline__ void os_vrr_accumulate(const PrimQ &g, const double *__restrict__ boys,
                                                   double *__restrict__ acc,
                                                   double *__restrict__ s1,
@@ -300,8 +281,7 @@ __device__ __forceinline__ void os_vrr_accumulate(const PrimQ &g, const double *
       j1[d] -= 1;
       const int f1 = cart_index(j1[0], j1[1], j1[2]) - ncum(f - 1);
       std::integral_constant<int, f - 1> lv1;
-      double v = g.WQ[d] * get(lv1, ecum, f1, m + 1);
-      if (!KET1) v += g.QC[d] * get(lv1, ecum, f1, m);
+      double v = g.QC[d] * get(lv1, ecum, f1, m) + g.WQ[d] * get(lv1, ecum, f1, m + 1);
       if constexpr (f >= 2) {
         if (nd >= 2) {
           j1[d] -= 1;
@@ -414,16 +394,12 @@ __device__ __forceinline__ ShellRef load_shell(const ShellSetDev &s, int i) {
 }
 
 // One quartet (a b|c d) by a group; d may be "unit" (exponent 0 at C) and b
-// may be unit too.  Result via os_hrr.  pab, pcd: the shell pairs' stored
-// primitive pairs (built once by k_pair_data), or null to form them here, in
-// every lane of the group: a division, an exponential and some thirty more FP64
-// operations of about 135 a primitive quartet.
-template <int LA, int LB, int LC, int LD, int G, bool KET1 = false>
+// may be unit too.  Result via os_hrr.
+template <int LA, int LB, int LC, int LD, int G>
 __device__ __forceinline__ const double *os_quartet(
     const double *boys, double *scr, int gl, const ShellRef &sa, const double *ea,
     const double *ca, const ShellRef *sb, const double *eb, const double *cb, const ShellRef &sc,
-    const double *ec, const double *cc, const ShellRef *sd, const double *ed, const double *cd,
-    const double *pab = nullptr, const double *pcd = nullptr) {
+    const double *ec, const double *cc, const ShellRef *sd, const double *ed, const double *cd) {
   using O = Os<LA, LB, LC, LD>;
   double *acc = scr;
   double *s1 = scr + O::ACC;
@@ -434,29 +410,16 @@ __device__ __forceinline__ const double *os_quartet(
   const double *D = sd ? sd->xyz : sc.xyz;
   const int nb = sb ? sb->nprim : 1, nd = sd ? sd->nprim : 1;
   for (int ia = 0; ia < sa.nprim; ++ia)
-    for (int ib = 0; ib < nb; ++ib) {
-      const PrimPair bra = pab ? load_pair(pab + kPairDbl * (ia * nb + ib))
-                               : make_pair(ea[ia], sa.xyz, sb ? eb[ib] : 0.0, B,
-                                           sb ? ca[ia] * cb[ib] : ca[ia]);
+    for (int ib = 0; ib < nb; ++ib)
       for (int ic = 0; ic < sc.nprim; ++ic)
         for (int id = 0; id < nd; ++id) {
-          PrimPair ket;
-          if (KET1) {
-            ket.p = ec[ic];
-            ket.ip = 1.0 / ket.p;
-            ket.K = cc[ic];
-#pragma unroll
-            for (int x = 0; x < 3; ++x) ket.P[x] = sc.xyz[x];
-          } else if (pcd) {
-            ket = load_pair(pcd + kPairDbl * (ic * nd + id));
-          } else {
-            ket = make_pair(ec[ic], sc.xyz, sd ? ed[id] : 0.0, D, sd ? cc[ic] * cd[id] : cc[ic]);
-          }
           PrimQ g;
-          prim_setup(bra, sa.xyz, ket, sc.xyz, g);
-          os_vrr_accumulate<LA, LB, LC, LD, G, KET1>(g, boys, acc, s1, gk, gl);
+          const double xb = sb ? eb[ib] : 0.0, wb = sb ? cb[ib] : 1.0;
+          const double xd = sd ? ed[id] : 0.0, wd = sd ? cd[id] : 1.0;
+          prim_setup(ea[ia], sa.xyz, xb, B, ec[ic], sc.xyz, xd, D, ca[ia] * wb * cc[ic] * wd, 0,
+                     g);
+          os_vrr_accumulate<LA, LB, LC, LD, G>(g, boys, acc, s1, gk, gl);
         }
-    }
   double AB[3], CD[3];
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
@@ -468,51 +431,12 @@ __device__ __forceinline__ const double *os_quartet(
   return os_hrr<LA, LB, LC, LD, G>(acc, bufA, bufB, gl, AB, CD);
 }
 
-// Primitive pairs of n shell pairs, stride doubles apart (room for the largest
-// product of primitive counts).
-static __global__ void k_pair_data(ShellSetDev orb, const int2 *pairs, int64_t n, int stride,
-                                   double *out) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const int2 pr = pairs[k];
-  const ShellRef a = load_shell(orb, pr.x), b = load_shell(orb, pr.y);
-  double *o = out + k * stride;
-  for (int ia = 0; ia < a.nprim; ++ia)
-    for (int ib = 0; ib < b.nprim; ++ib, o += kPairDbl) {
-      const PrimPair r = make_pair(orb.exps[a.poff + ia], a.xyz, orb.exps[b.poff + ib], b.xyz,
-                                   orb.coefs[a.poff + ia] * orb.coefs[b.poff + ib]);
-      o[0] = r.p;
-      o[1] = r.ip;
-      o[2] = r.K;
-      o[3] = r.P[0];
-      o[4] = r.P[1];
-      o[5] = r.P[2];
-    }
-}
-
-// Builds it for n pairs into `out` (at most 256 MB; without it, or without
-// memory for it, the kernels form the pairs themselves).
-static int pair_data_build(const Basis *b, const int2 *pairs, int64_t n, DBuf *out, int *stride,
-                           cudaStream_t s) {
-  int mp = 1;
-  for (int v : b->orb.nprim) mp = v > mp ? v : mp;
-  *stride = kPairDbl * mp * mp;
-  const size_t bytes = (size_t)n * *stride * sizeof(double);
-  if (!n || bytes > ((size_t)256 << 20) || out->alloc(b->ctx, bytes) != BQC_OK) return BQC_OK;
-  k_pair_data<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(b->orb.dev, pairs, n, *stride,
-                                                          out->as<double>());
-  BQC_LAUNCH_CHECK();
-  return BQC_OK;
-}
-
 // ------------------------------------------------ three-centre triplet ----
 
 struct Eri3cArgs {
   ShellSetDev orb, aux;
   const double *boys;
   const int2 *pairs;       // class segment, sorted by Schwarz factor
-  const double *pdata;     // its stored primitive pairs (null: formed in the kernel)
-  int pstride;             // doubles per shell pair there
   const int *aux_list;     // aux shells of this l
   const int64_t *prefix;   // n_aux + 1 survivor prefix
   int n_aux;
@@ -524,7 +448,6 @@ struct Eri3cArgs {
   // screening-ablation variants (ring buffer, index list): the class's pairs
   // in their original order with their Schwarz factors, the aux-shell factors
   const int2 *pairs_orig;
-  const double *pdata_orig;  // as pdata, in the original order
   const double *qpair_orig;
   const double *qaux;
   double tau;
@@ -538,17 +461,16 @@ struct Eri3cArgs {
 // triplet (so the warp stays convergent) and write nothing.
 template <int LC, int LA, int LB>
 __device__ __forceinline__ void eri3c_triplet(const Eri3cArgs &a, double *scr, int gl, int Pi,
-                                              int2 pr, bool active,
-                                              const double *pab = nullptr) {
+                                              int2 pr, bool active) {
   using O = Os<LA, LB, LC, 0>;
   constexpr int G = O::G;
   const ShellRef sc = load_shell(a.aux, Pi);
   const ShellRef sa = load_shell(a.orb, pr.x);
   const ShellRef sb = load_shell(a.orb, pr.y);
-  const double *res = os_quartet<LA, LB, LC, 0, G, true>(
+  const double *res = os_quartet<LA, LB, LC, 0, G>(
       a.boys, scr, gl, sa, a.orb.exps + sa.poff, a.orb.coefs + sa.poff, &sb,
       a.orb.exps + sb.poff, a.orb.coefs + sb.poff, sc, a.aux.exps + sc.poff,
-      a.aux.coefs + sc.poff, nullptr, nullptr, nullptr, pab);
+      a.aux.coefs + sc.poff, nullptr, nullptr, nullptr);
   if (active) {
     constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC);
     const bool diag = pr.x == pr.y;
