@@ -229,11 +229,8 @@ int launch_eri3c_variant(const Basis *b, const Eri3cPlan *plan, int p0, int p1, 
 int dgemm(bool transA, bool transB, int M, int N, int K, double alpha, const double *A,
           int64_t lda, const double *B, int64_t ldb, double beta, double *C, int64_t ldc,
           cudaStream_t s);
-// In-place lower Cholesky of an n x n SPD matrix (upper part zeroed).  With
-// enough scratch (device memory, overwritten) the trailing updates run on the
-// tensor cores.
-int cholesky_lower(Ctx *ctx, double *A, int n, void *scratch, size_t scratch_bytes,
-                   cudaStream_t s);
+// In-place lower Cholesky of an n x n SPD matrix (upper part zeroed).
+int cholesky_lower(Ctx *ctx, double *A, int n, cudaStream_t s);
 // In-place X := L^{-1} X for L n x n lower, X n x ncol with leading dim ld.
 // With enough scratch (device memory, overwritten) on the tensor cores.
 int trsm_lower_left(Ctx *ctx, const double *L, int n, double *X, int64_t ncol, int64_t ld,

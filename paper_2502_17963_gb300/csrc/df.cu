@@ -572,6 +572,16 @@ __global__ void __launch_bounds__(256) k_jk64_small_sum(const double *__restrict
   out[nu * n + mu] = s;
 }
 
+static size_t jk64_small_smem(int n, int no) {
+  return ((size_t)n * (n | 1) + (size_t)n * no + (size_t)n * (no | 1)) * 8;
+}
+
+// With nearly as many occupied orbitals as functions B_P, C and X_P may not fit
+// beside one another in shared memory.
+static bool jk64_small(int n, int no) {
+  return n <= kSmallN && jk64_small_smem(n, no) <= (size_t)220 * 1024;
+}
+
 static int jk64_small_slices(int naux) { return std::min(naux, 2 * sm_count()); }
 
 // Bytes of the FP64 X buffer: X, or the scratch of the small and the sliced
@@ -581,7 +591,7 @@ static size_t x64_bytes(int n, int naux, int no);
 static int jk_fp64_small(Df *df, const double *C, double *J, double *K, cudaStream_t s) {
   const int n = df->basis->nbf, naux = df->naux_loc, no = df->basis->nocc;
   const int npair = n * (n + 1) / 2, nsl = jk64_small_slices(naux);
-  const size_t smem = ((size_t)n * (n | 1) + (size_t)n * no + (size_t)n * (no | 1)) * 8;
+  const size_t smem = jk64_small_smem(n, no);
   BQC_CUDA_TRY(cudaFuncSetAttribute(k_jk64_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem));
   df->mark(0, s);
@@ -667,7 +677,7 @@ static int oz_rows_of_c(const double *C, int n, int no, void *slices, int *exps,
 
 static size_t x64_bytes(int n, int naux, int no) {
   const size_t x = (size_t)naux * n * no * 8;
-  const size_t more = n <= kSmallN ? (size_t)jk64_small_slices(naux) * n * (n + 1) * 8
+  const size_t more = jk64_small(n, no) ? (size_t)jk64_small_slices(naux) * n * (n + 1) * 8
                                    : oz_jk_plan(n, naux, no, SIZE_MAX).total;
   return std::max(x, std::min<size_t>(more, (size_t)32 << 20));
 }
@@ -838,8 +848,9 @@ int jk_fp64_stored(Df *df, const double *C, double *J, double *K, cudaStream_t s
   const int n = b->nbf, naux = df->naux_loc, no = b->nocc;
   const int64_t npair = df->npair;
   double *X = df->X64.as<double>();
-  if (n <= kSmallN && df->X64.n >= x64_bytes(n, naux, no)) return jk_fp64_small(df, C, J, K, s);
-  if (n > kSmallN) {
+  if (jk64_small(n, no) && df->X64.n >= x64_bytes(n, naux, no))
+    return jk_fp64_small(df, C, J, K, s);
+  if (n > 64) {
     const OzJkPlan p = oz_jk_plan(n, naux, no, df->X64.n);
     if (p.pc) return jk_fp64_oz(df, p, C, J, K, s);
   }
@@ -995,7 +1006,7 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
   if (cudaMemcpyAsync(df->Vdiag.p, df->L.p, (size_t)naux * naux * 8, cudaMemcpyDeviceToDevice,
                       s) != cudaSuccess)
     return fail(BQC_E_CUDA);
-  if ((st = cholesky_lower(ctx, df->L.as<double>(), naux, scr.p, scr.n, s)) != BQC_OK) return fail(st);
+  if ((st = cholesky_lower(ctx, df->L.as<double>(), naux, s)) != BQC_OK) return fail(st);
   if ((st = ctx->check_flag(s)) != BQC_OK) return fail(st);
   if ((st = eri3c_plan(basis, o.schwarz, df->Vdiag.as<double>(), s, &df->plan)) != BQC_OK)
     return fail(st);

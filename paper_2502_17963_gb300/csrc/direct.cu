@@ -9,7 +9,7 @@
 // (These equal the stored-mode J and K: J = sum_P B_P (B_P:D) with
 // B = L^{-1}(Q|..) gives sum_{QQ'} (Q|..) (V^{-1})_{QQ'} (Q'|D).)
 // Integrals and the gamma / c / J parts are FP64; X, Y and K run either in
-// FP64 (DFMA, small systems) or on the tensor cores (tc.cu).
+// FP64 (sliced products, oz.cu) or in split TF32 (tc.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -114,7 +114,7 @@ int direct_setup(Df *df, cudaStream_t s) {
   k_identity<<<nb((int64_t)naux * naux), 256, 0, s>>>(df->Linv.as<double>(), naux);
   BQC_LAUNCH_CHECK();
   BQC_TRY(trsm_lower_left(ctx, df->L.as<double>(), naux, df->Linv.as<double>(), naux, naux,
-                          df->raw.p, df->raw.n, s));
+                          nullptr, 0, s));
   BQC_TRY(df->gamma.alloc(ctx, (size_t)naux * 8 * 2));
   BQC_TRY(df->D2.alloc(ctx, (size_t)df->npair * 8));
   BQC_TRY(df->Jp.alloc(ctx, (size_t)df->npair * 8));

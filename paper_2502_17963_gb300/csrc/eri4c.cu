@@ -75,18 +75,24 @@ __global__ void __launch_bounds__(256) k_jk4c(Jk4Args a) {
     const int2 p = a.pX[lo], q = a.pY[jq];
     const ShellRef sa = load_shell(a.orb, p.x), sb = load_shell(a.orb, p.y);
     const ShellRef sc = load_shell(a.orb, q.x), sd = load_shell(a.orb, q.y);
-    const double *res = os_quartet<LA, LB, LC, LD, G>(
+    double *res = const_cast<double *>(os_quartet<LA, LB, LC, LD, G>(
         a.boys, scr, gl, sa, a.orb.exps + sa.poff, a.orb.coefs + sa.poff, &sb,
         a.orb.exps + sb.poff, a.orb.coefs + sb.poff, sc, a.orb.exps + sc.poff,
-        a.orb.coefs + sc.poff, &sd, a.orb.exps + sd.poff, a.orb.coefs + sd.poff);
+        a.orb.coefs + sc.poff, &sd, a.orb.exps + sd.poff, a.orb.coefs + sd.poff));
+    // normalise once: each integral enters six contractions
+    for (int e = gl; e < O::NOUT; e += G) {
+      const int id = e % ND, ic = e / ND % NC, ib = e / (ND * NC) % NB, ia = e / (ND * NC * NB);
+      res[e] *= (c_cnorm[ncum(LA) + ia] * c_cnorm[ncum(LB) + ib]) *
+                (c_cnorm[ncum(LC) + ic] * c_cnorm[ncum(LD) + id]);
+    }
+    __syncwarp();
     if (active) {
       double w = 1.0;
       if (p.x == p.y) w *= 0.5;
       if (q.x == q.y) w *= 0.5;
       if (a.same && jq == lo) w *= 0.5;
       auto val = [&](int ia, int ib, int ic, int id) {
-        return res[((ia * NB + ib) * NC + ic) * ND + id] * c_cnorm[ncum(LA) + ia] *
-               c_cnorm[ncum(LB) + ib] * c_cnorm[ncum(LC) + ic] * c_cnorm[ncum(LD) + id];
+        return res[((ia * NB + ib) * NC + ic) * ND + id];
       };
       const double *D = a.D;
       // J_ij += 2 w sum_kl v D_kl

@@ -1,12 +1,13 @@
-// FP64 dense kernels of the DF pipeline: a DFMA GEMM (the plain-FP64
-// contractions and the metric solve), blocked Cholesky of the Coulomb metric
+// FP64 dense kernels of the DF pipeline: blocked Cholesky of the Coulomb metric
 // V = L L^T, and the in-place triangular solve B = L^{-1} (Q|mu nu) that
 // turns raw three-centre integrals into the Cholesky-decomposed ERIs (CD-ERIs) of
 // Sec. 2.2.
 //
-// On GB300 FP64 runs at ~1.2 TFLOP/s (about 2 DFMA per clock per SM), so a
-// 64x64 register-blocked tile already saturates the FP64 pipe; the kernels
-// are written for that pipe, not for the tensor cores.
+// On GB300 FP64 runs at ~1.2 TFLOP/s (about 2 DFMA per clock per SM, a quarter
+// of that for a lone warp), so the products of both run as sliced FP16 products
+// on the tensor cores (oz.cu) when the caller has scratch for the slices; the
+// 64x64 register-blocked DFMA GEMM (gemm64.cuh) serves without it.  Set-up of
+// (H2O)_24 (Naux = 1800): 575 ms on the DFMA pipe, about 60 ms so.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -42,193 +43,78 @@ int dgemm(bool tA, bool tB, int M, int N, int K, double alpha, const double *A, 
 
 constexpr int kNB = 64;
 
-// 1 / sqrt(d) for a positive normal d: FP32 seed of the mantissa and one
-// third-order step, y (1 + e/2 + 3 e^2/8) with e = 1 - m y^2 (the binomial
-// series), whose error is of the order of the seed's 2^-22 cubed.  A warp's
-// FP64 instruction occupies its scheduler for 64 clocks here, so the library's
-// sqrt and division would be most of a factorisation.
-__device__ __forceinline__ double rsqrt_pos(double d) {
-  const int hi = __double2hiint(d);
-  const int k = ((hi >> 20) - 1023) >> 1;  // d = m 4^k, 1 <= m < 4
-  const double m = __hiloint2double(hi - (k << 21), __double2loint(d));
-  const double y = (double)rsqrtf((float)m);
-  const double e = fma(-m * y, y, 1.0);
-  const double r = fma(y * e, fma(0.375, e, 0.5), y);
-  return __hiloint2double(__double2hiint(r) - (k << 20), __double2loint(r));
-}
-
-// Cholesky of the kNB x kNB diagonal block at (k0, k0) in shared memory, by
-// 16-column steps: one warp factors the 16 x 16 block in registers (a lane
-// holds half a row; no block-wide barrier per column), four warps solve the
-// rows below it, all threads update the rest.  Writes L (lower) and zeros
-// above; flag <- 1 when not positive.  A serial chain on one SM.
-constexpr int kPB = 16;
+// Unblocked Cholesky of the kNB x kNB diagonal block at (k0, k0), in shared
+// memory; writes L (lower) and zeros above.  flag <- 1 when not positive.
 __global__ void __launch_bounds__(256) k_potrf_diag(double *A, int n, int k0, int *flag) {
   __shared__ double a[kNB][kNB + 1];
-  __shared__ double dinv[kPB];
-  const int nb = min(kNB, n - k0), t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  for (int i = t; i < kNB * kNB; i += 256) {
+  const int nb = min(kNB, n - k0);
+  for (int i = threadIdx.x; i < kNB * kNB; i += blockDim.x) {
     const int r = i / kNB, c = i % kNB;
-    // a ragged block is padded with the identity
-    a[r][c] = (r < nb && c < nb) ? A[(int64_t)(k0 + r) * n + k0 + c] : (r == c ? 1.0 : 0.0);
+    a[r][c] = (r < nb && c < nb) ? A[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
   }
   __syncthreads();
-  for (int j0 = 0; j0 < nb; j0 += kPB) {
-    if (warp == 0) {
-      // lane r + 16 h: columns 8 h .. 8 h + 7 of row r
-      const int r = lane & (kPB - 1), h = lane >> 4;
-      double x[8], di = 1.0;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) x[c] = a[j0 + r][j0 + 8 * h + c];
-#pragma unroll
-      for (int c = 0; c < kPB; ++c) {
-        const int hc = c >> 3, cc = c & 7;
-        double d = __shfl_sync(0xffffffffu, x[cc], c + 16 * hc);
-        if (!(d >= 2.2250738585072014e-308 && d <= 1.7976931348623157e308)) {
-          if (lane == 0) atomicExch(flag, 1);
-          d = 1.0;
-        }
-        const double iv = rsqrt_pos(d);
-        // column c of L in every lane of its row (from the half that holds it)
-        const double l = __shfl_sync(0xffffffffu, x[cc], r + 16 * hc) * iv;
-        if (r == c) di = iv;
-        if (h == hc) x[cc] = l;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const double lq = __shfl_sync(0xffffffffu, l, 8 * h + q);
-          if (8 + q > c && (q > cc || hc == 0)) {  // columns past c exist in some half
-            if (8 * h + q > c) x[q] = fma(-l, lq, x[q]);
-          }
-        }
+  for (int j = 0; j < nb; ++j) {
+    if (threadIdx.x == 0) {
+      const double d = a[j][j];
+      if (!(d > 0.0)) {
+        atomicExch(flag, 1);
+        a[j][j] = 1.0;
+      } else {
+        a[j][j] = sqrt(d);
       }
-#pragma unroll
-      for (int c = 0; c < 8; ++c) a[j0 + r][j0 + 8 * h + c] = 8 * h + c <= r ? x[c] : 0.0;
-      if (h == 0) dinv[r] = di;
     }
     __syncthreads();
-    const int r1 = j0 + kPB;
-    // rows below, spread over four warps (a scheduler each)
-    if (warp < 4 && lane < 12 && r1 + warp * 12 + lane < kNB) {
-      const int r = r1 + warp * 12 + lane;
-      double x[kPB];
-#pragma unroll
-      for (int c = 0; c < kPB; ++c) x[c] = a[r][j0 + c];
-#pragma unroll
-      for (int c = 0; c < kPB; ++c) {
-        x[c] *= dinv[c];
-#pragma unroll
-        for (int l = c + 1; l < kPB; ++l) x[l] = fma(-x[c], a[j0 + l][j0 + c], x[l]);
-      }
-#pragma unroll
-      for (int c = 0; c < kPB; ++c) a[r][j0 + c] = x[c];
-    }
+    const double djj = a[j][j];
+    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) a[i][j] /= djj;
     __syncthreads();
-    // a 16 x 16 grid of threads over the remaining square's lower part
-    const int tx = t & 15, ty = t >> 4;
-    for (int r = r1 + ty; r < kNB; r += 16)
-      for (int c = r1 + tx; c <= r; c += 16) {
-        double v = a[r][c];
-#pragma unroll
-        for (int l = 0; l < kPB; ++l) v = fma(-a[r][j0 + l], a[c][j0 + l], v);
-        a[r][c] = v;
-      }
+    const int m = nb - j - 1;
+    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+      const int r = j + 1 + t / m, c = j + 1 + t % m;
+      if (c <= r) a[r][c] -= a[r][j] * a[c][j];
+    }
     __syncthreads();
   }
-  for (int i = t; i < nb * nb; i += 256) {
+  for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) {
     const int r = i / nb, c = i % nb;
     A[(int64_t)(k0 + r) * n + k0 + c] = (c <= r) ? a[r][c] : 0.0;
   }
 }
 
-// Rows below the diagonal block: A_rk := A_rk L_kk^{-T}, also zeroing the
-// block above the diagonal.  16 rows a block, one element a thread: the
-// 16-column steps are X_b := (A_b - sum_{c < b} X_c L_bc^T) L_bb^{-T} with the
-// explicit inverses of the four 16 x 16 diagonal blocks, which four warps make
-// first (a thread per row of 64 columns kept one scheduler of four busy:
-// 104 us a panel).
-__global__ void __launch_bounds__(256) k_chol_panel(double *A, int n, int k0) {
+// Rows below the diagonal block: A_rk := A_rk L_kk^{-T} (forward substitution
+// per row, one thread per row); also zeroes the block above the diagonal.
+__global__ void __launch_bounds__(128) k_chol_panel(double *A, int n, int k0) {
   __shared__ double L[kNB][kNB + 1];
-  __shared__ double x[kPB][kNB + 1];
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  for (int i = t; i < kNB * kNB; i += 256)
-    L[i / kNB][i % kNB] = A[(int64_t)(k0 + i / kNB) * n + k0 + i % kNB];
-  const int row0 = k0 + kNB + blockIdx.x * kPB;
-  for (int i = t; i < kPB * kNB; i += 256) {
-    const int r = row0 + i / kNB;
-    x[i / kNB][i % kNB] = r < n ? A[(int64_t)r * n + k0 + i % kNB] : 0.0;
+  const int nb = min(kNB, n - k0);
+  for (int i = threadIdx.x; i < kNB * kNB; i += blockDim.x) {
+    const int r = i / kNB, c = i % kNB;
+    L[r][c] = (r < nb && c < nb) ? A[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
   }
   __syncthreads();
-  if (warp < 4 && lane < kPB) {  // column `lane` of the inverse
-    const int b0 = warp * kPB;
-    double y[kPB];
-#pragma unroll
-    for (int r = 0; r < kPB; ++r) y[r] = r == lane ? 1.0 : 0.0;
-#pragma unroll
-    for (int r = 0; r < kPB; ++r) {
-      y[r] /= L[b0 + r][b0 + r];
-#pragma unroll
-      for (int l = r + 1; l < kPB; ++l) y[l] = fma(-y[r], L[b0 + l][b0 + r], y[l]);
+  const int row = k0 + nb + blockIdx.x * blockDim.x + threadIdx.x;
+  if (row < n) {
+    double x[kNB];
+    double *ar = A + (int64_t)row * n + k0;
+    for (int j = 0; j < nb; ++j) {
+      double v = ar[j];
+      for (int l = 0; l < j; ++l) v -= x[l] * L[j][l];
+      x[j] = v / L[j][j];
     }
-    __syncwarp(0xffffu);  // the block is not read again: its inverse replaces it
-#pragma unroll
-    for (int r = 0; r < kPB; ++r) L[b0 + r][b0 + lane] = y[r];
-  }
-  const int rr = t >> 4, cc = t & 15;
-  for (int b = 0; b < 4; ++b) {
-    __syncthreads();
-    double v = x[rr][b * kPB + cc];
-    for (int l = 0; l < b * kPB; ++l) v = fma(-x[rr][l], L[b * kPB + cc][l], v);
-    __syncwarp();  // a row's 16 threads are in one warp
-    x[rr][b * kPB + cc] = v;
-    __syncwarp();
-    double y = 0.0;
-#pragma unroll
-    for (int l = 0; l < kPB; ++l) y = fma(x[rr][b * kPB + l], L[b * kPB + cc][b * kPB + l], y);
-    __syncwarp();
-    x[rr][b * kPB + cc] = y;
-  }
-  __syncthreads();
-  for (int i = t; i < kPB * kNB; i += 256) {
-    const int r = row0 + i / kNB;
-    if (r < n) A[(int64_t)r * n + k0 + i % kNB] = x[i / kNB][i % kNB];
-  }
-  // upper block (rows k0 .., columns row0 ..) = 0
-  for (int i = t; i < kPB * kNB; i += 256) {
-    const int c = row0 + i % kPB;
-    if (c < n) A[(int64_t)(k0 + i / kPB) * n + c] = 0.0;
+    for (int j = 0; j < nb; ++j) ar[j] = x[j];
+    // upper block (row k0 + j, column `row`) = 0
+    for (int j = 0; j < nb; ++j) A[(int64_t)(k0 + j) * n + row] = 0.0;
   }
 }
 
-int cholesky_lower(Ctx *ctx, double *A, int n, void *scratch, size_t scratch_bytes,
-                   cudaStream_t s) {
+int cholesky_lower(Ctx *ctx, double *A, int n, cudaStream_t s) {
   for (int k0 = 0; k0 < n; k0 += kNB) {
     const int nb = std::min(kNB, n - k0);
     k_potrf_diag<<<1, 256, 0, s>>>(A, n, k0, ctx->flag);
     BQC_LAUNCH_CHECK();
     const int rem = n - k0 - nb;
     if (rem <= 0) break;
-    k_chol_panel<<<(rem + kPB - 1) / kPB, 256, 0, s>>>(A, n, k0);
+    k_chol_panel<<<(rem + 127) / 128, 128, 0, s>>>(A, n, k0);
     BQC_LAUNCH_CHECK();
     // trailing update, lower triangle only: A22 -= L21 L21^T
-    const double *L21 = A + (int64_t)(k0 + nb) * n + k0;
-    double *A22 = A + (int64_t)(k0 + nb) * n + k0 + nb;
-    if (oz_slice_bytes(rem, nb) + oz_exp_bytes(rem, 1) <= scratch_bytes) {
-      OzSrc x;
-      x.kind = kOzRows;
-      x.p = L21;
-      x.rows = rem;
-      x.K = nb;
-      x.ld = n;
-      OzOperand o;
-      o.slices = scratch;
-      int *e = reinterpret_cast<int *>(static_cast<char *>(scratch) + oz_slice_bytes(rem, nb));
-      o.exps = e;
-      o.rows = rem;
-      o.K = nb;
-      BQC_TRY(oz_slice(x, oz_kblocks(nb), scratch, e, s));
-      BQC_TRY(oz_gemm(o, o, oz_kblocks(nb), -1, 1, A22, n, 0, kOzUpper, ctx->flag, s));
-      continue;
-    }
     Gemm64Args g;
     g.M = rem;
     g.N = rem;
@@ -236,13 +122,13 @@ int cholesky_lower(Ctx *ctx, double *A, int n, void *scratch, size_t scratch_byt
     g.K2 = nb;
     g.alpha = -1.0;
     g.beta = 1.0;
-    g.A = L21;
+    g.A = A + (int64_t)(k0 + nb) * n + k0;
     g.lda = n;
     g.sA1 = 0;
     g.B = g.A;
     g.ldb = n;
     g.sB1 = 0;
-    g.C = A22;
+    g.C = A + (int64_t)(k0 + nb) * n + k0 + nb;
     g.ldc = n;
     g.lower_only = 1;
     BQC_TRY(launch_gemm64(kAN, true, g, s));

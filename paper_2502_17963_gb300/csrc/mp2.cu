@@ -7,7 +7,8 @@
 //   E2 = sum_{ijab} (ia|jb) [2 (ia|jb) - (ib|ja)] / (e_i + e_j - e_a - e_b)
 // (Szabo & Ostlund Eq. 6.74) is accumulated with the denominator applied in
 // place, one block of occupied pairs at a time, so no four-index array is
-// ever held.  FP64: the register-blocked DFMA GEMM of gemm64.cuh;
+// ever held.  FP64: sliced tensor-core products (oz.cu), (H2O)_10 in 6.7 ms
+// against 96.8 on the DFMA GEMM of gemm64.cuh, which serves small systems;
 // MIXED_F16X3: the pair blocks on the tensor cores (tc.cu).
 #include <cuda_runtime.h>
 
@@ -238,9 +239,9 @@ static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec
     BQC_TRY(Bt.alloc(ctx, (size_t)naux * Q * 8));
     const int bi = mp2_block(no, nv);
     int pc = 0;
-    if (n > 64 && Ts.alloc(ctx, oz_slice_bytes(Q, naux) + oz_exp_bytes(Q, 1)) == BQC_OK)
+    if (n > (prec == BQC_PREC_FP64 ? 64 : 112) && Ts.alloc(ctx, oz_slice_bytes(Q, naux) + oz_exp_bytes(Q, 1)) == BQC_OK)
       pc = mp2_transform_pc(n, naux, no, nv, Ts.n);
-    const bool oz = prec == BQC_PREC_FP64 && Ts.p;
+    bool oz = prec == BQC_PREC_FP64 && Ts.p;
     if (pc)
       BQC_TRY(mp2_transform_oz(df, C, nmo, Bt.as<double>(), Ts.as<char>(), pc, s));
     else
@@ -265,7 +266,14 @@ static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec
       q.ld = Q;
       BQC_TRY(oz_slice(q, oz_kblocks(naux), Ts.p, te, s));
     }
-    BQC_TRY(V.alloc(ctx, (size_t)bi * nv * bi * nv * 8));
+    if (V.alloc(ctx, (size_t)bi * nv * bi * nv * 8) != BQC_OK) {
+      if (!oz) return BQC_E_OOM;
+      // the slices' memory is what the pair block lacks: do without them
+      BQC_CUDA_TRY(cudaStreamSynchronize(s));
+      Ts.release();
+      oz = false;
+      BQC_TRY(V.alloc(ctx, (size_t)bi * nv * bi * nv * 8));
+    }
     for (int i0 = 0; i0 < no; i0 += bi) {
       const int ni = std::min(bi, no - i0);
       for (int j0 = 0; j0 <= i0; j0 += bi) {

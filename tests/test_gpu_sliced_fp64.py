@@ -61,6 +61,38 @@ def test_fp64_fock_build(gpu_ctx, bqc, name, spread):
     assert torch.equal(K, K.T) and torch.equal(J, J.T)
 
 
+def test_fp64_fock_build_many_occupied(gpu_ctx, bqc):
+    """As many occupied orbitals as functions (twelve argon atoms in three s
+    and two p shells each, N = nocc = 108): the small build's B_P, C and X_P do
+    not fit in shared memory together, and the sliced products take over."""
+    import torch
+    from types import SimpleNamespace as NS
+    k = np.arange(12)
+    xyz = 6.0 * np.stack([k % 3, k // 3 % 2, k // 6], axis=1).astype(float)
+
+    def shells(rules):
+        return [NS(atom=a, l=l, exps=[e], coefs=[1.0]) for a in range(12) for l, e in rules]
+
+    mol = NS(Z=np.full(12, 18, dtype=np.int32), xyz=xyz,
+             orb=shells([(0, 0.3), (0, 1.0), (0, 3.0), (1, 0.4), (1, 1.2)]),
+             aux=shells([(0, 0.8), (0, 2.5), (1, 1.0), (2, 1.1)]))
+    basis = bqc.Basis(gpu_ctx, mol)
+    n, no = basis.nbf, basis.nocc
+    assert n == no == 108
+    df = bqc.DF(gpu_ctx, basis, keep_fp32=False)
+    B = _full(torch, df.copy(0), n)
+    rng = np.random.default_rng(3)
+    C = torch.tensor(rng.standard_normal((n, no)) / np.sqrt(n), device="cuda")
+    J, K = df.jk(C, bqc.PREC_FP64)
+    X = B @ C
+    Kr = torch.einsum("pmi,pni->mn", X, X)
+    Jr = torch.einsum("p,pmn->mn", (X * C).sum((1, 2)), B)
+    # N Naux nocc terms of 2^-53 of the largest products, as above
+    eps = 16 * 2.0 ** -53
+    assert (K - Kr).abs().max() <= eps * basis.naux * no * n * X.abs().max() ** 2
+    assert (J - Jr).abs().max() <= eps * basis.naux * no * n * (X.abs().max() * B.abs().max())
+
+
 def test_fp64_fock_build_nan(gpu_ctx, bqc):
     """A NaN or an infinity in one orbital reaches every element of J and K."""
     import torch
