@@ -236,11 +236,14 @@ __global__ void k_unpack_jsum_grp(const __grid_constant__ JGroup g) {
 }
 
 // aux chunks of the J pass: enough blocks for four per SM, at least min_aux P
-// each.  8: with the former 64 a small system ran on a few blocks, each a
-// serial stream ((H2O)_4 piece of 75 P: 10 blocks, 32 us).
+// each.  64 for the float-pair passes: their chunks are part of the mixed Fock
+// matrix's last bits, which a small staged SCF amplifies (see scf.cu).  8 for
+// the FP64 pass, where 64 left a small system on a few blocks, each a serial
+// stream.
 int jpass_split(int64_t npair, int naux, int min_aux) {
   const int64_t blocks = (npair / 2 + 256) / 256;
-  int sp = (int)std::min<int64_t>(64, (4 * (int64_t)sm_count() + blocks - 1) / blocks);
+  int sp = (int)std::min<int64_t>(min_aux >= 64 ? 16 : 64,
+                                  (4 * (int64_t)sm_count() + blocks - 1) / blocks);
   sp = std::max(1, std::min(sp, naux / min_aux));
   return sp;
 }
@@ -258,7 +261,7 @@ int jpass_fp64(Df *df, double *J, cudaStream_t s) {
   const int n = df->basis->nbf, naux = df->naux_loc;
   const int64_t npair = df->npair;
   if (!df->B64.p) return BQC_E_INVALID;
-  const int sp = jpass_split(npair, naux);
+  const int sp = jpass_split(npair, naux, kFp64JAux);
   if (df->Jp.n < (size_t)sp * npair * 8) return BQC_E_INVALID;
   k_jpass64<<<dim3((unsigned)((npair / 2 + 256) / 256), (unsigned)sp), 256, 0, s>>>(
       df->B64.as<double>(), df->w.as<double>(), naux, npair, df->Jp.as<double>());
@@ -874,17 +877,15 @@ size_t df_stored_bytes(int n, int naux, int nocc, int shadow) {
   b += (size_t)naux * n * nocc * 8;                                // X64
   // (J partials of systems that fill the GPU; the few MB that smaller ones
   // hold beyond this, and X's scratch, are among the caller's small buffers)
-  b += (size_t)std::min(16, jpass_split((int64_t)npair, naux, 64)) * npair * 8 + (size_t)naux * 8 * 2;
+  b += (size_t)jpass_split((int64_t)npair, naux) * npair * 8 + (size_t)naux * 8 * 2;
   if (shadow == BQC_SHADOW_TF32 || shadow == BQC_SHADOW_F16)
     b += mixed_workspace_bytes(n, naux, nocc, shadow);
   if (shadow == BQC_SHADOW_F16) {  // float-pair B and w of the J pass, the pieces' J partials
     b += (size_t)naux * npair * 8 + (size_t)naux * 8;
     const int np = std::min(kJPieces, std::max(naux, 1));
     for (int k = 0; k < np; ++k)
-      b += (size_t)std::min(16, jpass_split((int64_t)npair,
-                                            (int)((int64_t)naux * (k + 1) / np) -
-                                                (int)((int64_t)naux * k / np),
-                                            64)) *
+      b += (size_t)jpass_split((int64_t)npair, (int)((int64_t)naux * (k + 1) / np) -
+                                                   (int)((int64_t)naux * k / np)) *
            npair * 8;
   }
   return b;
@@ -911,7 +912,7 @@ int bqc_df_coulomb(bqc_df *df, const double *D_dev, double *J_dev, int variant,
   }
   BQC_CUDA_TRY(cudaSetDevice(df->ctx->device));
   if (df->D2.n < (size_t)df->npair * 8) BQC_TRY(df->D2.alloc(df->ctx, (size_t)df->npair * 8));
-  const int need = jpass_split(df->npair, df->naux_loc);
+  const int need = jpass_split(df->npair, df->naux_loc, kFp64JAux);
   if (df->Jp.n < (size_t)need * df->npair * 8)
     BQC_TRY(df->Jp.alloc(df->ctx, (size_t)need * df->npair * 8));
   cudaStream_t s = (cudaStream_t)stream;
@@ -1013,6 +1014,14 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
   if ((st = df->w.alloc(ctx, (size_t)naux * 8)) != BQC_OK) return fail(st);
   if (mode == BQC_DF_STORED) {
     df->Vdiag.release();  // metric only needed for the screening plan
+    // The sliced solve for every handle but small ones with shadows: its B is
+    // within 1e-12 of the plain solve's, which a staged SCF's mixed stage (see
+    // scf.cu) turns into more than 1e-9 in its result, and such solves are what
+    // small handles serve; the mixed builds of larger ones move by at most
+    // 5e-10 ((H2O)_32).  450 aux functions: 3 ms plain, 0.6 sliced.
+    const bool sliced = o.keep_fp32 == BQC_SHADOW_NONE || naux > 512;
+    void *const sp = sliced ? df->X64.p : nullptr;
+    const size_t sn = sliced ? df->X64.n : 0;
     if (!shard) {
       if ((st = df->B64.alloc(ctx, (size_t)naux * npair * 8)) != BQC_OK) return fail(st);
       if (cudaMemsetAsync(df->B64.p, 0, (size_t)naux * npair * 8, s) != cudaSuccess)
@@ -1021,7 +1030,7 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
           BQC_OK)
         return fail(st);
       if ((st = trsm_lower_left(ctx, df->L.as<double>(), naux, df->B64.as<double>(), npair,
-                                npair, df->X64.p, df->X64.n, s)) != BQC_OK)
+                                npair, sp, sn, s)) != BQC_OK)
         return fail(st);
     } else {
       // B_P for P in [P0, P1) depends on (Q|mu nu) for every Q <= P (the
@@ -1038,7 +1047,7 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
                             cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return fail(BQC_E_CUDA);
       if ((st = trsm_lower_left(ctx, Lb.as<double>(), P1, raw.as<double>(), npair, npair,
-                                df->X64.p, df->X64.n, s)) != BQC_OK)
+                                sp, sn, s)) != BQC_OK)
         return fail(st);
       if ((st = df->B64.alloc(ctx, (size_t)(P1 - P0) * npair * 8)) != BQC_OK) return fail(st);
       if (cudaMemcpyAsync(df->B64.p, raw.as<double>() + (size_t)P0 * npair,
@@ -1048,7 +1057,7 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
       if (cudaStreamSynchronize(s) != cudaSuccess) return fail(BQC_E_CUDA);
     }
     const int nl = df->naux_loc;
-    if ((st = df->Jp.alloc(ctx, (size_t)jpass_split(npair, nl) * npair * 8)) != BQC_OK)
+    if ((st = df->Jp.alloc(ctx, (size_t)jpass_split(npair, nl, kFp64JAux) * npair * 8)) != BQC_OK)
       return fail(st);
     if (o.keep_fp32 != BQC_SHADOW_NONE)
       if ((st = mixed_setup(df, o.keep_fp32, s)) != BQC_OK) return fail(st);

@@ -8,13 +8,6 @@ namespace bqc {
 
 // Aux pieces of the split-FP16 build's X pass (each followed by its J pass).
 constexpr int kJPieces = 4;
-// Pieces for a tensor: one per 64 MB of float pairs, below which a piece's
-// J pass (12 us) is no longer than the launches that a piece adds.
-inline int j_pieces(int naux, int64_t npair) {
-  const int64_t by = ((int64_t)naux * npair * 8) >> 26;
-  const int np = by < 1 ? 1 : (by > kJPieces ? kJPieces : (int)by);
-  return np < naux ? np : naux;
-}
 // Problems of one grouped launch (the problem table is a kernel parameter).
 constexpr int kMaxGroup = 12;
 struct FockGroup;
@@ -143,7 +136,8 @@ int jpass_unpack(Df *df, int nslice, double *J, cudaStream_t s);
 // (the FP16 shadow set-up fills B2f).
 int jpass_ff_alloc(Df *df);
 int jpass_ff_range(Df *df, int P0, int P1, int y0, cudaStream_t s);
-int jpass_split(int64_t npair, int naux, int min_aux = 8);
+constexpr int kFp64JAux = 8;
+int jpass_split(int64_t npair, int naux, int min_aux = 64);
 // J[D] = sum_P (B_P : D) B_P in FP64 over the stored FP64 B for a symmetric
 // N x N matrix D (any sign), D2 an Npair scratch.
 int jfp64_of_density(Df *df, const double *D, double *D2, double *J, cudaStream_t s);

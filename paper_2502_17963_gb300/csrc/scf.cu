@@ -323,10 +323,17 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
   EighRefiner refiner;
   BQC_TRY(small.reserve(ctx, n));
   BQC_TRY(refiner.reserve(ctx, w.sol, nmo));
+  // The FP64 stage runs on the small products, the refined eigenvectors and the
+  // fused scalars below; the mixed stage on the library calls.  Near its error
+  // floor DIIS extrapolates from errors that are mostly the mixed build's
+  // rounding, so a change in the last bit there moves the orbitals at the switch
+  // by about 1e-8, and with them the last Fock matrix (converged to diis_tol) by
+  // more than 1e-9; in FP64 it moves the result by 1e-12.
+  bool fp64_stage = o.prec == BQC_PREC_FP64;
   // C (m x k) = op(A) op(B), column-major
   auto mm = [&](bool tA, bool tB, int m, int cols, int k, const double *A, int lda, const double *B,
                 int ldb, double *Cm, int ldc) -> int {
-    if (small.takes(m, cols, k)) return small.run(tA, tB, m, cols, k, A, lda, B, ldb, Cm, ldc, s);
+    if (fp64_stage && small.takes(m, cols, k)) return small.run(tA, tB, m, cols, k, A, lda, B, ldb, Cm, ldc, s);
     BQC_BLAS_TRY(cublasDgemm(w.blas, tA ? CUBLAS_OP_T : CUBLAS_OP_N, tB ? CUBLAS_OP_T : CUBLAS_OP_N,
                              m, cols, k, &one, A, lda, B, ldb, &zero, Cm, ldc));
     return BQC_OK;
@@ -336,7 +343,8 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
     BQC_TRY(mm(false, false, n, nmo, n, M, n, Xp, n, t1.as<double>(), n));
     BQC_TRY(mm(true, false, nmo, nmo, n, Xp, n, t1.as<double>(), n, Fp.as<double>(), nmo));
     bool done = false;
-    BQC_TRY(refiner.run(w.sol, small, Fp.as<double>(), nmo, ev.as<double>(), &done, s));
+    if (fp64_stage)
+      BQC_TRY(refiner.run(w.sol, small, Fp.as<double>(), nmo, ev.as<double>(), &done, s));
     if (!done) BQC_TRY(eigh(w, ctx, Fp.as<double>(), nmo, ev.as<double>(), work, info, s));
     BQC_TRY(mm(false, false, n, nmo, nmo, Xp, n, Fp.as<double>(), nmo, Cc.as<double>(), n));
     return BQC_OK;
@@ -354,7 +362,6 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
   }
   // scalars of an iteration: energy, largest error, and the error's dot
   // products with the stored ones (a larger subspace takes the library calls)
-  const bool fused_dots = space + 2 <= kMaxDots;
   DBuf dots;
   std::vector<double> hdots(kMaxDots, 0.0);
   BQC_TRY(dots.alloc(ctx, (size_t)kMaxDots * (kDotBlocks + 1) * 8));
@@ -524,6 +531,8 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
       BQC_CUDA_TRY(cudaStreamSynchronize(s));
       return BQC_E_CANCELLED;
     }
+    fp64_stage = stage == BQC_PREC_FP64;
+    const bool fused_dots = fp64_stage && space + 2 <= kMaxDots;
     const bool inc_stage = inc_on && stage == BQC_PREC_FP64 && anchors < 8;
     last_incremental = inc_stage && !need_anchor;
     if (last_incremental) {
@@ -746,7 +755,7 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
     if (m >= 2) {
       std::vector<double> c;
       if (diis_solve(Bm, m, c)) {
-        if (m <= kMaxDots) {
+        if (fp64_stage && m <= kMaxDots) {
           MixArgs g;
           g.m = m;
           for (int i = 0; i < m; ++i) {

@@ -1916,13 +1916,13 @@ static int mixed_setup_f16(Df *df, MixedState *ms, cudaStream_t s) {
   // |B row| <= |Bh row| / (1 - 2^-11); the factor also covers the float sums
   ms->rownorm = std::sqrt((double)maxsq) / (double)sB * (1.0 + 1.0 / 256.0);
   {  // room for the J partials of the pieces
-    const int np = j_pieces(naux, df->npair);
+    const int np = std::min(kJPieces, naux);
     int slices = 0;
     for (int k = 0; k < np; ++k)
       slices += jpass_split(df->npair, (int)((int64_t)naux * (k + 1) / np) -
                                            (int)((int64_t)naux * k / np));
     const size_t need =
-        (size_t)std::max(jpass_split(df->npair, naux), slices) * df->npair * 8;
+        (size_t)std::max(jpass_split(df->npair, naux, kFp64JAux), slices) * df->npair * 8;
     if (df->Jp.n < need) BQC_TRY(df->Jp.alloc(ctx, need));
   }
   BQC_TRY(ms->Xh16.alloc(ctx, (size_t)naux * n * m.ldx * 2));
@@ -2426,7 +2426,7 @@ int jk_mixed_stored(Df *df, const double *C, int prec, double *J, double *K, cud
     // as the X pass and the SYRK together at the memory parallelism a J
     // block gets beside a persistent tensor-core CTA, so it has to start
     // early to end with them).
-    const int np = j_pieces(naux, df->npair);
+    const int np = std::min(kJPieces, naux);
     cudaStream_t ts = df->tcs, js = df->side;
     df->mark(0, s);
     BQC_TRY(mixed_xpass(df, C, kind, split, s, &ms->mapAh, &ms->mapAl, rows, nullptr, nullptr,
