@@ -1018,7 +1018,8 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
     // within 1e-12 of the plain solve's, which a staged SCF's mixed stage (see
     // scf.cu) turns into more than 1e-9 in its result, and such solves are what
     // small handles serve; the mixed builds of larger ones move by at most
-    // 5e-10 ((H2O)_32).  450 aux functions: 3 ms plain, 0.6 sliced.
+    // 5e-10 ((H2O)_32).  Set-up of (H2O)_8, 600 aux functions: 12.2 ms with the
+    // plain solve, 5.5 with the sliced one.
     const bool sliced = o.keep_fp32 == BQC_SHADOW_NONE || naux > 512;
     void *const sp = sliced ? df->X64.p : nullptr;
     const size_t sn = sliced ? df->X64.n : 0;

@@ -1133,7 +1133,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // K = sum over chunks of the FP64 partial tiles, symmetric.  One block per
 // (lower tile, 8 x 32 sub-tile), one element a thread: small systems have one
 // tile and over a hundred chunks, so the blocks have to come from the tile and
-// the loads of 16 chunks be in flight ((H2O)_4: 387 -> 12 us).  The mirror
+// the loads of 16 chunks be in flight ((H2O)_4: 387 -> 22 us).  The mirror
 // image is written through shared memory.
 constexpr int kRedSub = (kBM / 8) * (kBM / 32);
 __device__ __forceinline__ void syrk_reduce_sub(const double *part, int nchunk, int ntri, int n,
