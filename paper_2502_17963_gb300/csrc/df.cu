@@ -1014,13 +1014,15 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
   if ((st = df->w.alloc(ctx, (size_t)naux * 8)) != BQC_OK) return fail(st);
   if (mode == BQC_DF_STORED) {
     df->Vdiag.release();  // metric only needed for the screening plan
-    // The sliced solve for every handle but small ones with shadows: its B is
-    // within 1e-12 of the plain solve's, which a staged SCF's mixed stage (see
-    // scf.cu) turns into more than 1e-9 in its result, and such solves are what
-    // small handles serve; the mixed builds of larger ones move by at most
-    // 5e-10 ((H2O)_32).  Set-up of (H2O)_8, 600 aux functions: 12.2 ms with the
-    // plain solve, 5.5 with the sliced one.
-    const bool sliced = o.keep_fp32 == BQC_SHADOW_NONE || naux > 512;
+    // The sliced solve for handles without shadows only.  Its B is within 1e-12
+    // of the substitution's and as near to 64 bits, but a split shadow keeps 22
+    // bits: a few elements in a million of B then round the other way, which
+    // moves the split-FP16 K of (H2O)_32 by 7e-10 of its norm and single elements
+    // by 7e-8, and a staged SCF's mixed stage (see scf.cu) turns a change of B's
+    // last bits into more than 1e-9 of its last Fock matrix ((H2O)_8: 4e-9,
+    // (H2O)_12: 4e-9, against 1e-12).  What it costs: set-up of (H2O)_24 with FP16
+    // shadows 570 ms, with the sliced solve 77.
+    const bool sliced = o.keep_fp32 == BQC_SHADOW_NONE;
     void *const sp = sliced ? df->X64.p : nullptr;
     const size_t sn = sliced ? df->X64.n : 0;
     if (!shard) {
