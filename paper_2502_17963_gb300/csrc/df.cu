@@ -236,13 +236,14 @@ __global__ void k_unpack_jsum_grp(const __grid_constant__ JGroup g) {
 }
 
 // aux chunks of the J pass: enough blocks for four per SM, at least min_aux P
-// each.  64 for the float-pair passes: their chunks are part of the mixed Fock
-// matrix's last bits, which a small staged SCF amplifies (see scf.cu).  8 for
-// the FP64 pass, where 64 left a small system on a few blocks, each a serial
-// stream.
+// each.  64 for the passes of mixed builds (float-pair or FP64): their chunks are
+// part of the mixed Fock matrix's last bits, which a staged SCF amplifies (see
+// scf.cu; with 8 in the TF32x3 build its (H2O)_5 result moved by 1.3e-9).  8 for
+// the J pass of FP64 builds, where 64 left a small system on a few blocks, each
+// a serial stream.
 int jpass_split(int64_t npair, int naux, int min_aux) {
   const int64_t blocks = (npair / 2 + 256) / 256;
-  int sp = (int)std::min<int64_t>(min_aux >= 64 ? 16 : 64,
+  int sp = (int)std::min<int64_t>(min_aux >= kMixedJAux ? 16 : 64,
                                   (4 * (int64_t)sm_count() + blocks - 1) / blocks);
   sp = std::max(1, std::min(sp, naux / min_aux));
   return sp;
@@ -257,11 +258,11 @@ __global__ void k_unpack_sym(const double *Jp, int n, double *J) {
   J[i] = Jp[hi * (hi + 1) / 2 + lo];
 }
 
-int jpass_fp64(Df *df, double *J, cudaStream_t s) {
+int jpass_fp64(Df *df, double *J, cudaStream_t s, int min_aux) {
   const int n = df->basis->nbf, naux = df->naux_loc;
   const int64_t npair = df->npair;
   if (!df->B64.p) return BQC_E_INVALID;
-  const int sp = jpass_split(npair, naux, kFp64JAux);
+  const int sp = jpass_split(npair, naux, min_aux);
   if (df->Jp.n < (size_t)sp * npair * 8) return BQC_E_INVALID;
   k_jpass64<<<dim3((unsigned)((npair / 2 + 256) / 256), (unsigned)sp), 256, 0, s>>>(
       df->B64.as<double>(), df->w.as<double>(), naux, npair, df->Jp.as<double>());

@@ -125,8 +125,10 @@ int x_of_b(Ctx *ctx, const double *b, int64_t npair, const double *C, int n, int
            double *X, void *scratch, size_t bytes, cudaStream_t s);
 int k_of_x(Ctx *ctx, const double *X, int n, int no, int naux, void *scratch, size_t bytes,
            double *K, cudaStream_t s);
-// J = sum_P w_P B_P from the packed FP64 B and df->w (FP64), full symmetric.
-int jpass_fp64(Df *df, double *J, cudaStream_t s);
+// J = sum_P w_P B_P from the packed FP64 B and df->w (FP64), full symmetric;
+// chunks of at least min_aux aux functions (jpass_split).
+constexpr int kFp64JAux = 8, kMixedJAux = 64;
+int jpass_fp64(Df *df, double *J, cudaStream_t s, int min_aux = kFp64JAux);
 // The FP64 J pass in pieces: partials of aux functions [P0, P1) (df->w) into
 // partial slices starting at y0, then the sum of nslice slices into J.
 int jpass_fp64_range(Df *df, int P0, int P1, int y0, cudaStream_t s);
@@ -136,8 +138,7 @@ int jpass_unpack(Df *df, int nslice, double *J, cudaStream_t s);
 // (the FP16 shadow set-up fills B2f).
 int jpass_ff_alloc(Df *df);
 int jpass_ff_range(Df *df, int P0, int P1, int y0, cudaStream_t s);
-constexpr int kFp64JAux = 8;
-int jpass_split(int64_t npair, int naux, int min_aux = 64);
+int jpass_split(int64_t npair, int naux, int min_aux = kMixedJAux);
 // J[D] = sum_P (B_P : D) B_P in FP64 over the stored FP64 B for a symmetric
 // N x N matrix D (any sign), D2 an Npair scratch.
 int jfp64_of_density(Df *df, const double *D, double *D2, double *J, cudaStream_t s);

@@ -2475,7 +2475,7 @@ int jk_mixed_stored(Df *df, const double *C, int prec, double *J, double *K, cud
     js = df->side;
   }
   if (j64) {
-    BQC_TRY(jpass_fp64(df, J, js));
+    BQC_TRY(jpass_fp64(df, J, js, kMixedJAux));
   } else {
     const dim3 jgrid((unsigned)((n + 1) / 2),
                      (unsigned)(((n - 1) / 4 + 2 + kJThreads - 1) / kJThreads));
