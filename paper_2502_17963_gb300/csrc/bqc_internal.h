@@ -124,6 +124,14 @@ class SideFork {
   int n_ = 0;
 };
 
+// Waits for a stream at the end of a scope.  Declared after a function's device
+// buffers, it keeps an early return from giving back memory (to an arena that
+// another solve allocates from) that launched work still uses.
+struct StreamGuard {
+  cudaStream_t s;
+  ~StreamGuard() { cudaStreamSynchronize(s); }
+};
+
 // Device buffer owned by a context.
 struct DBuf {
   Ctx *ctx = nullptr;

@@ -701,23 +701,33 @@ int eri3c_plan(const Basis *b, double tau, const double *V_diag_dev, cudaStream_
   BQC_TRY(plan->d_qaux.alloc(ctx, nas * sizeof(double)));
   DBuf &qpair = plan->d_qpair;
   BQC_TRY(qpair.alloc(ctx, np * sizeof(double)));
+  // all memory before the first launch; an error waits for launched work before
+  // the sorts' scratch goes back
+  DBuf tmp[kNPairClass];
+  StreamGuard guard{s};
+  size_t need[kNPairClass] = {};
+  for (int cls = 0; cls < kNPairClass; ++cls) {
+    const int n = b->pair_off[cls + 1] - b->pair_off[cls];
+    if (!n) continue;
+    BQC_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(
+        nullptr, need[cls], (const double *)nullptr, (double *)nullptr, (const int2 *)nullptr,
+        (int2 *)nullptr, n, 0, 64, s));
+    BQC_TRY(tmp[cls].alloc(ctx, std::max<size_t>(need[cls], 16)));
+  }
+  CutArgs ca;
+  int64_t off = 0;
+  for (int cls = 0; cls < kNPairClass; ++cls)
+    for (int lc = 0; lc <= kMaxLAux; ++lc) {
+      plan->prefix_off[cls][lc] = ca.prefix_off[cls][lc] = off;
+      off += (b->auxl_off[lc + 1] - b->auxl_off[lc]) + 1;
+    }
+  BQC_TRY(plan->d_prefix.alloc(ctx, off * sizeof(int64_t)));
   BQC_TRY(launch_schwarz_pairs(b, qpair.as<double>(), s));
   k_diag_sqrt_max<<<(nas + 127) / 128, 128, 0, s>>>(V_diag_dev, b->naux, b->aux.dev.fn,
                                                       b->aux.dev.l, nas, plan->d_qaux.as<double>());
   BQC_LAUNCH_CHECK();
-  // sort each class segment by decreasing Q (beside each other; the scratch is
-  // released after the copy below)
-  DBuf tmp[kNPairClass];
+  // sort each class segment by decreasing Q (beside each other)
   {
-    size_t need[kNPairClass] = {};
-    for (int cls = 0; cls < kNPairClass; ++cls) {
-      const int n = b->pair_off[cls + 1] - b->pair_off[cls];
-      if (!n) continue;
-      BQC_CUDA_TRY(cub::DeviceRadixSort::SortPairsDescending(
-          nullptr, need[cls], (const double *)nullptr, (double *)nullptr, (const int2 *)nullptr,
-          (int2 *)nullptr, n, 0, 64, s));
-      BQC_TRY(tmp[cls].alloc(ctx, std::max<size_t>(need[cls], 16)));
-    }
     SideFork fork(ctx, s);
     for (int cls = 0; cls < kNPairClass; ++cls) {
       const int o = b->pair_off[cls], n = b->pair_off[cls + 1] - o;
@@ -729,14 +739,6 @@ int eri3c_plan(const Basis *b, double tau, const double *V_diag_dev, cudaStream_
     BQC_TRY(fork.join());
   }
   // survivor counts and prefixes per (class, aux l)
-  CutArgs ca;
-  int64_t off = 0;
-  for (int cls = 0; cls < kNPairClass; ++cls)
-    for (int lc = 0; lc <= kMaxLAux; ++lc) {
-      plan->prefix_off[cls][lc] = ca.prefix_off[cls][lc] = off;
-      off += (b->auxl_off[lc + 1] - b->auxl_off[lc]) + 1;
-    }
-  BQC_TRY(plan->d_prefix.alloc(ctx, off * sizeof(int64_t)));
   std::copy(b->pair_off, b->pair_off + kNPairClass + 1, ca.pair_off);
   std::copy(b->auxl_off, b->auxl_off + kMaxLAux + 2, ca.auxl_off);
   ca.qpair = plan->d_qpair_sorted.as<double>();

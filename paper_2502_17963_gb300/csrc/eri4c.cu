@@ -240,6 +240,7 @@ int jk4c_setup(Df *df, cudaStream_t s) {
   pl->tau = df->opts.schwarz;
   const int64_t np = b->npair_sh;
   DBuf q;
+  StreamGuard guard{s};
   BQC_TRY(q.alloc(ctx, (size_t)std::max<int64_t>(1, np) * 8));
   BQC_TRY(launch_schwarz_pairs(b, q.as<double>(), s));
   std::vector<double> hq(np);

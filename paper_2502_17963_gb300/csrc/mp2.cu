@@ -231,8 +231,10 @@ static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec
   const int n = b->nbf, naux = b->naux, no = b->nocc, nv = nmo - no;
   Ctx *ctx = df->ctx;
   DBuf Bt, V, ep, out, Ts;
+  std::unique_ptr<Mp2Tc, Mp2TcDeleter> tcs;
   BQC_TRY(ep.alloc(ctx, (size_t)no * no * 8));
   BQC_TRY(out.alloc(ctx, 8));
+  StreamGuard guard{s};
   BQC_CUDA_TRY(cudaMemsetAsync(ep.p, 0, ep.n, s));
   if (nv > 0) {
     const int64_t Q = (int64_t)no * nv;
@@ -246,7 +248,6 @@ static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec
       BQC_TRY(mp2_transform_oz(df, C, nmo, Bt.as<double>(), Ts.as<char>(), pc, s));
     else
       BQC_TRY(mp2_transform_dfma(df, C, nmo, Bt.as<double>(), s));
-    std::unique_ptr<Mp2Tc, Mp2TcDeleter> tcs;
     if (prec == BQC_PREC_MIXED_F16X3) {
       if (Ts.p) {
         BQC_CUDA_TRY(cudaStreamSynchronize(s));

@@ -478,8 +478,9 @@ int bqc_int3c(const bqc_basis *b, double schwarz, double *out, bqc_stream_t stre
   const int64_t npair = (int64_t)b->nbf * (b->nbf + 1) / 2;
   DBuf V;
   BQC_TRY(V.alloc(b->ctx, (size_t)b->naux * b->naux * sizeof(double)));
-  BQC_TRY(launch_int2c(b, V.as<double>(), s));
   Eri3cPlan plan;
+  StreamGuard guard{s};
+  BQC_TRY(launch_int2c(b, V.as<double>(), s));
   BQC_TRY(eri3c_plan(b, schwarz, V.as<double>(), s, &plan));
   BQC_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)b->naux * npair * sizeof(double), s));
   BQC_TRY(launch_eri3c(b, &plan, 0, b->naux, out, npair, s));

@@ -300,6 +300,7 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
     BQC_TRY(p->alloc(ctx, nn * 8));
   BQC_TRY(ev.alloc(ctx, (size_t)n * 8));
   BQC_TRY(Crm.alloc(ctx, (size_t)n * no * 8));
+  StreamGuard guard{s};
   BQC_TRY(launch_one_electron(b, S.as<double>(), T.as<double>(), V.as<double>(), s));
   k_axpby3<<<nblk(nn), 256, 0, s>>>(nn, T.as<double>(), 1.0, V.as<double>(), 1.0, nullptr, 0.0,
                                     H.as<double>());
@@ -321,6 +322,7 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
   double *Xp = X.as<double>();
   SmallGemm small;
   EighRefiner refiner;
+  StreamGuard guard_eigh{s};
   BQC_TRY(small.reserve(ctx, n));
   BQC_TRY(refiner.reserve(ctx, w.sol, nmo));
   // The FP64 stage runs on the small products, the refined eigenvectors and the
@@ -356,13 +358,14 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
   }
   const int space = std::max(1, o.diis_space);
   std::vector<DBuf> hF(space), hE(space);
+  // scalars of an iteration: energy, largest error, and the error's dot
+  // products with the stored ones (a larger subspace takes the library calls)
+  DBuf dots;
+  StreamGuard guard_diis{s};
   for (int i = 0; i < space; ++i) {
     BQC_TRY(hF[i].alloc(ctx, nn * 8));
     BQC_TRY(hE[i].alloc(ctx, (size_t)nmo * nmo * 8));
   }
-  // scalars of an iteration: energy, largest error, and the error's dot
-  // products with the stored ones (a larger subspace takes the library calls)
-  DBuf dots;
   std::vector<double> hdots(kMaxDots, 0.0);
   BQC_TRY(dots.alloc(ctx, (size_t)kMaxDots * (kDotBlocks + 1) * 8));
   std::vector<int> slot;  // DIIS entries in age order (slot indices)
@@ -396,6 +399,7 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
   const bool rank2 = inc_on && mixed_prec == BQC_PREC_MIXED_F16X3 &&
                      df->mode == BQC_DF_STORED && df->B64.p && df->mixed && !df->is_shard();
   DBuf Ca, Sca, Mo, Uo, VTo, So, Ro, Ct;
+  StreamGuard guard_inc{s};
   if (inc_on) {
     for (DBuf *p : {&Facc, &Dref, &Dk, &J2, &K2, &Jx}) BQC_TRY(p->alloc(ctx, nn * 8));
     BQC_TRY(evd.alloc(ctx, (size_t)n * 8));

@@ -2899,6 +2899,7 @@ int mp2_tc_setup(Ctx *ctx, const double *Bt, int naux, int nocc, int nv, int *fl
   m->ldp = round_up(naux, 8);
   // scale: largest |B_P,ia| to at most 2^14
   DBuf stat;
+  StreamGuard guard{s};
   BQC_TRY(stat.alloc(ctx, 256));
   BQC_CUDA_TRY(cudaMemsetAsync(stat.p, 0, 256, s));
   const int64_t nb = (int64_t)naux * m->Q;
