@@ -93,6 +93,11 @@ typedef void (*bqc_free_fn)(void *ptr, void *user);
 int bqc_ctx_create(int device, size_t hbm_budget, bqc_alloc_fn alloc, bqc_free_fn dealloc,
                    void *alloc_user, bqc_ctx **out);
 int bqc_ctx_destroy(bqc_ctx *ctx);
+/* 1 if this context's kernels may use cluster multicast loads, else 0.  They do
+ * only where the process sees a single GPU and the environment's WORLD_SIZE,
+ * read at creation, is unset or at most 1: replicas and shards on several GPUs
+ * run the plain loads, with the same results. */
+int bqc_ctx_multicast(const bqc_ctx *ctx);
 
 /* One contracted Cartesian shell.  exps/coefs: nprim entries each; coefs
  * multiply unit-normalised primitives. */

@@ -147,6 +147,7 @@ _SIGS = {
     "bqc_jk_grouped": (ip, [ip, ctypes.POINTER(vp), ctypes.POINTER(vp), ctypes.POINTER(vp),
                             ctypes.POINTER(vp), vp]),
     "bqc_df_coulomb": (ip, [vp, vp, vp, ip, vp]),
+    "bqc_ctx_multicast": (ip, [vp]),
     "bqc_wait_selftest": (ip, [vp, ctypes.c_longlong, vp]),
     "bqc_mp2": (ip, [vp, vp, vp, ip, ip, ctypes.POINTER(ctypes.c_double), vp]),
 }
@@ -219,6 +220,11 @@ class Context:
         check(L.bqc_ctx_create(device, hbm_budget, self._afn, self._ffn, None,
                                ctypes.byref(h)), "bqc_ctx_create")
         self.h = h
+
+    @property
+    def multicast(self) -> bool:
+        """Whether kernels of this context may use cluster multicast loads."""
+        return bool(lib().bqc_ctx_multicast(self.h))
 
     def close(self):
         if getattr(self, "h", None):

@@ -91,6 +91,9 @@ struct Ctx {
   bqc_alloc_fn alloc = nullptr;
   bqc_free_fn dealloc = nullptr;
   void *user = nullptr;
+  // cluster multicast loads (the split-FP16 X pass): only where this process has
+  // the one GPU there is and is no rank of a larger job (replicas, aux shards)
+  bool multicast = false;
   double *boys = nullptr;  // device table [kBoysNT][kBoysNM]
   int *flag = nullptr;     // device error word (0 = fine)
   std::mutex mu;

@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 
@@ -308,6 +309,8 @@ int bqc_ctx_create(int device, size_t hbm_budget, bqc_alloc_fn alloc, bqc_free_f
   c->alloc = alloc;
   c->dealloc = dealloc;
   c->user = alloc_user;
+  const char *world = std::getenv("WORLD_SIZE");
+  c->multicast = ndev == 1 && (!world || std::atoi(world) <= 1);
   c->flag = (int *)c->dmalloc(sizeof(int));
   if (!c->flag) {
     delete c;
@@ -325,6 +328,8 @@ int bqc_ctx_create(int device, size_t hbm_budget, bqc_alloc_fn alloc, bqc_free_f
   *out = c;
   return BQC_OK;
 }
+
+int bqc_ctx_multicast(const bqc_ctx *ctx) { return ctx && ctx->multicast ? 1 : 0; }
 
 int bqc_ctx_destroy(bqc_ctx *ctx) {
   if (!ctx) return BQC_E_INVALID;

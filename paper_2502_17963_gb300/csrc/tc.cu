@@ -1723,7 +1723,8 @@ struct MixedState {
   int shadow = BQC_SHADOW_TF32;
   CUtensorMap mapAh, mapAl, mapCh, mapCl, mapXh, mapXl;
   // split-FP16 X pass in cluster pairs: C boxes of xn / 2 rows, and the
-  // number of two-CTA clusters that fit at once (0: pairs not used)
+  // number of two-CTA clusters that fit at once (0: pairs not used, the plain
+  // kernel serves with the same result; Ctx::multicast)
   CUtensorMap mapChH, mapClH;
   int mc_clusters = 0;
   DBuf Bl, Xl, Cl, Cf, wpart, w32;
@@ -1948,7 +1949,7 @@ static int mixed_setup_f16(Df *df, MixedState *ms, cudaStream_t s) {
     BQC_TRY(make_tmap_f16(&ms->mapChH, ms->Ch16.p, 2, dims, str, hbox));
     BQC_TRY(make_tmap_f16(&ms->mapClH, ms->Cl16.p, 2, dims, str, hbox));
   }
-  BQC_TRY(xpass_mc_setup(ms, m.xn, m.xp_smem[1]));
+  if (ctx->multicast) BQC_TRY(xpass_mc_setup(ms, m.xn, m.xp_smem[1]));
   {  // X split as (ldx, N, Naux)
     const uint64_t dims[3] = {(uint64_t)m.ldx, (uint64_t)n, (uint64_t)naux};
     const uint64_t str[2] = {(uint64_t)m.ldx * 2, (uint64_t)n * m.ldx * 2};
