@@ -425,6 +425,15 @@ enum { BQC_SWITCH_NONE = 0, BQC_SWITCH_STAGE_TOL = 1, BQC_SWITCH_FLOOR = 2 };
 int bqc_scf_run(bqc_ctx *ctx, bqc_df *df, const bqc_scf_opts *opts, bqc_stream_t stream,
                 bqc_scf_result *out);
 
+/* Symmetric eigen-decomposition of the SCF's FP64 stage (up to 320 functions an
+ * FP32 decomposition refined to FP64 by products, cuSOLVER's FP64 one above and
+ * where the refinement does not apply), exposed for testing: A_dev (n x n,
+ * symmetric) receives the orthonormal eigenvectors as its rows (row k belongs
+ * to w_dev[k]), w_dev n ascending eigenvalues; *refined (host, may be NULL) says
+ * whether the refined decomposition served.  Synchronises the stream. */
+int bqc_eigh(bqc_ctx *ctx, int n, double *A_dev, double *w_dev, int *refined,
+             bqc_stream_t stream);
+
 /* ------------------------------------------------------------ serving --- */
 
 typedef enum {

@@ -148,6 +148,7 @@ _SIGS = {
                             ctypes.POINTER(vp), vp]),
     "bqc_df_coulomb": (ip, [vp, vp, vp, ip, vp]),
     "bqc_ctx_multicast": (ip, [vp]),
+    "bqc_eigh": (ip, [vp, ip, vp, vp, ctypes.POINTER(ctypes.c_int), vp]),
     "bqc_wait_selftest": (ip, [vp, ctypes.c_longlong, vp]),
     "bqc_mp2": (ip, [vp, vp, vp, ip, ip, ctypes.POINTER(ctypes.c_double), vp]),
 }
@@ -481,6 +482,18 @@ def scf_run(ctx: Context, df: DF, prec: int = PREC_FP64, diis_tol: float = 1e-8,
     if keep_arrays:
         out.update(C=Cbuf[: n * r.nmo].view(n, r.nmo), eps=eps[: r.nmo], F=F)
     return out
+
+
+def eigh(ctx: Context, A, stream=None):
+    """(w, V, refined): eigenvalues and eigenvectors (columns of V) of a symmetric
+    device matrix by the SCF's FP64-stage decomposition."""
+    import torch
+    V = A.to(torch.float64).contiguous().clone()
+    w = _empty((V.shape[0],))
+    r = ctypes.c_int()
+    check(lib().bqc_eigh(ctx.h, V.shape[0], _ptr(V), _ptr(w), ctypes.byref(r),
+                         _stream_ptr(stream)), "bqc_eigh")
+    return w, V.T, bool(r.value)
 
 
 class Server:

@@ -12,17 +12,22 @@
 //   E_ij = (J^T H J)_ij / (l_j - l_i) between clusters,
 //   X := X (1 - Rt / 2) J (1 + E).
 // A cluster is a run of eigenvalues with gaps below 128 times the largest
-// off-diagonal g of H, so |E| < 1/128 and a round squares the error; three
-// rounds take FP32's 1e-6 to below FP64's rounding.  The result is accepted
-// when g has fallen below 1e-12 of the largest eigenvalue before the last
-// round; otherwise (a cluster of more than eight, no convergence) the caller
-// falls back to the FP64 decomposition.
+// off-diagonal g of H, so |E| < 1/128 and a round squares the error, or below
+// 1e-8 of the largest eigenvalue: three rounds take g from FP32's 1e-6 to FP64's
+// rounding (1e-15), and E between two levels that such a g still couples would
+// leave E^2 in X^T X - 1 (with a gap limit of 1e-12, 1e-10 and more for levels
+// 1e-11 to 1e-10 apart).  From the third round on the vectors are then made
+// orthonormal, X (3 - X^T X) / 2, and the result is accepted when g had fallen
+// below 1e-12 of the largest eigenvalue and the R = X^T X - 1 measured before
+// that step below 1e-9, which leaves 3/4 R^2.  Otherwise (a cluster of more than
+// eight, no convergence) the caller falls back to the FP64 decomposition.
 #include <cublas_v2.h>
 #include <cuda_runtime.h>
 #include <cusolverDn.h>
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "bqc_internal.h"
 #include "eigh.h"
@@ -121,6 +126,7 @@ constexpr int kClusterMax = 8;
 
 struct RefineStat {
   unsigned long long g, top;  // bits of the largest |off-diagonal| and |diagonal| of H, by round
+  unsigned long long res;     // bits of the largest |X^T X - 1| after it
   int fail;                   // of any round
 };
 
@@ -174,7 +180,7 @@ __global__ void __launch_bounds__(64) k_refine_clusters(int n, const double *__r
   auto diag = [&](int k) { return H[(int64_t)k * n + k]; };
   const double top = __longlong_as_double((long long)st->top);
   const double thr =
-      fmax(128.0 * __longlong_as_double((long long)st->g), 1e-12 * top);
+      fmax(128.0 * __longlong_as_double((long long)st->g), 1e-8 * top);
   if (i > 0 && diag(i) - diag(i - 1) < -thr) st->fail = 1;  // not in order
   if (i > 0 && !(diag(i) - diag(i - 1) > thr)) return;      // not the first of a cluster
   int m = 1;
@@ -273,6 +279,21 @@ __global__ void __launch_bounds__(256) k_refine_m(int n, const double *__restric
   M[e] = v;
 }
 
+// M = (3 - X^T X) / 2, and the largest |X^T X - 1|.
+__global__ void __launch_bounds__(256) k_refine_orth(int n, const double *__restrict__ XX,
+                                                     RefineStat *st, double *__restrict__ M) {
+  const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  unsigned long long r = 0;
+  if (e < (int64_t)n * n) {
+    const double one = e % n == e / n ? 1.0 : 0.0, rt = XX[e] - one;
+    M[e] = fma(-0.5, rt, one);
+    r = (unsigned long long)__double_as_longlong(rt) & 0x7fffffffffffffffULL;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) r = max(r, __shfl_xor_sync(0xffffffffu, r, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(&st->res, r);
+}
+
 int EighRefiner::reserve(Ctx *c, cusolverDnHandle_t sol, int n) {
   nmax = 0;
   if (n < 2 || n > kEighRefineMax) return BQC_OK;
@@ -310,7 +331,7 @@ int EighRefiner::run(cusolverDnHandle_t sol, const SmallGemm &mm, double *A, int
   BQC_LAUNCH_CHECK();
   BQC_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(RefineStat), s));
   for (int round = 0; round < 5; ++round) {
-    if (round) BQC_CUDA_TRY(cudaMemsetAsync(st, 0, 2 * sizeof(unsigned long long), s));
+    if (round) BQC_CUDA_TRY(cudaMemsetAsync(st, 0, 3 * sizeof(unsigned long long), s));
     BQC_TRY(mm.run(true, false, n, n, n, x, n, x, n, xx, n, s));
     BQC_TRY(mm.run(false, false, n, n, n, A, n, x, n, t, n, s));
     BQC_TRY(mm.run(true, false, n, n, n, x, n, t, n, sm, n, s));
@@ -324,6 +345,11 @@ int EighRefiner::run(cusolverDnHandle_t sol, const SmallGemm &mm, double *A, int
     BQC_TRY(mm.run(false, false, n, n, n, x, n, sm, n, t, n, s));
     std::swap(x, t);
     if (round < 2) continue;  // two rounds always; then look before another one
+    BQC_TRY(mm.run(true, false, n, n, n, x, n, x, n, xx, n, s));
+    k_refine_orth<<<gb, 256, 0, s>>>(n, xx, st, sm);
+    BQC_LAUNCH_CHECK();
+    BQC_TRY(mm.run(false, false, n, n, n, x, n, sm, n, t, n, s));
+    std::swap(x, t);
     struct {
       RefineStat st;
       char pad[128 - sizeof(RefineStat)];
@@ -331,11 +357,13 @@ int EighRefiner::run(cusolverDnHandle_t sol, const SmallGemm &mm, double *A, int
     } h;
     BQC_CUDA_TRY(cudaMemcpyAsync(&h, stat.p, sizeof(h), cudaMemcpyDeviceToHost, s));
     BQC_CUDA_TRY(cudaStreamSynchronize(s));
-    double g, top;
-    std::copy_n(reinterpret_cast<const char *>(&h.st.g), 8, reinterpret_cast<char *>(&g));
-    std::copy_n(reinterpret_cast<const char *>(&h.st.top), 8, reinterpret_cast<char *>(&top));
-    if (h.info || h.st.fail || !std::isfinite(g) || !std::isfinite(top)) return BQC_OK;
-    if (g <= 1e-12 * top) {
+    double g, top, res;
+    std::memcpy(&g, &h.st.g, 8);
+    std::memcpy(&top, &h.st.top, 8);
+    std::memcpy(&res, &h.st.res, 8);
+    if (h.info || h.st.fail || !std::isfinite(g) || !std::isfinite(top) || !std::isfinite(res))
+      return BQC_OK;
+    if (g <= 1e-12 * top && res <= 1e-9) {
       BQC_CUDA_TRY(cudaMemcpyAsync(A, x, nn * 8, cudaMemcpyDeviceToDevice, s));
       *done = true;
       return BQC_OK;

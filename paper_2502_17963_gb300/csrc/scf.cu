@@ -803,11 +803,38 @@ int scf_run(Ctx *ctx, Df *df, const bqc_scf_opts &o, cudaStream_t s, bqc_scf_res
   return converged ? BQC_OK : BQC_E_NOT_CONVERGED;
 }
 
+// The decomposition of the FP64 stage: refined from FP32 where that applies.
+static int eigh_fp64(Ctx *ctx, int n, double *A, double *evals, bool *refined, cudaStream_t s) {
+  ScfWork w;
+  BQC_TRY(get_handles(ctx->device, w));
+  BQC_SOLVER_TRY(cusolverDnSetStream(w.sol, s));
+  SmallGemm small;
+  EighRefiner refiner;
+  DBuf work, info;
+  BQC_TRY(small.reserve(ctx, n));
+  BQC_TRY(refiner.reserve(ctx, w.sol, n));
+  StreamGuard guard{s};
+  BQC_TRY(refiner.run(w.sol, small, A, n, evals, refined, s));
+  if (!*refined) BQC_TRY(eigh(w, ctx, A, n, evals, work, info, s));
+  BQC_CUDA_TRY(cudaStreamSynchronize(s));
+  return ctx->check_flag(s);
+}
+
 }  // namespace bqc
 
 using namespace bqc;
 
 extern "C" {
+
+int bqc_eigh(bqc_ctx *ctx, int n, double *A_dev, double *w_dev, int *refined,
+             bqc_stream_t stream) {
+  if (!ctx || n < 1 || n > 32768 || !A_dev || !w_dev) return BQC_E_INVALID;
+  BQC_CUDA_TRY(cudaSetDevice(ctx->device));
+  bool done = false;
+  BQC_TRY(eigh_fp64(ctx, n, A_dev, w_dev, &done, (cudaStream_t)stream));
+  if (refined) *refined = done ? 1 : 0;
+  return BQC_OK;
+}
 
 int bqc_scf_run(bqc_ctx *ctx, bqc_df *df, const bqc_scf_opts *opts, bqc_stream_t stream,
                 bqc_scf_result *out) {
