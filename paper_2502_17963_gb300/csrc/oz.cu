@@ -197,7 +197,7 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr) {
 
 struct OzParams {
   int64_t M;
-  int N, mt, nt;
+  int N, nt;
   int nkb, split_kb, ns;
   int tiles;  // tiles of one split
   int tri;
@@ -216,16 +216,12 @@ __device__ __forceinline__ OzItem oz_item(const OzParams &p, int64_t it) {
   OzItem x;
   x.split = (int)(it / p.tiles);
   const int t = (int)(it - (int64_t)x.split * p.tiles);
-  if (p.tri) {  // row tile tm has column tiles 0 .. 2 tm + 1 (upper: counted from the end)
+  if (p.tri) {  // row tile tm has column tiles 0 .. 2 tm + 1
     int tm = (int)((sqrtf(4.0f * t + 1.0f) - 1.0f) * 0.5f);
     while ((tm + 1) * (tm + 2) <= t) ++tm;
     while (tm * (tm + 1) > t) --tm;
     x.tm = tm;
     x.tn = t - tm * (tm + 1);
-    if (p.tri == kOzUpper) {  // an odd column count leaves tile nt empty
-      x.tm = p.mt - 1 - x.tm;
-      x.tn = 2 * p.mt - 1 - x.tn;
-    }
   } else {
     x.tm = t / p.nt;
     x.tn = t - x.tm * p.nt;
@@ -438,14 +434,12 @@ int oz_gemm(const OzOperand &A, const OzOperand &B, int split_kb, int alpha, int
   OzParams p;
   p.M = A.rows;
   p.N = (int)B.rows;
-  p.mt = (int)((A.rows + kOzM - 1) / kOzM);
   p.nt = (int)((B.rows + kOzN - 1) / kOzN);
   p.nkb = oz_kblocks(A.K);
   p.split_kb = split_kb;
   p.ns = (p.nkb + split_kb - 1) / split_kb;
   p.tri = tri;
-  const int64_t tiles = tri == kOzUpper ? (int64_t)p.mt * (p.mt + 1)
-                                        : oz_tiles(A.rows, B.rows, tri == kOzLower);
+  const int64_t tiles = oz_tiles(A.rows, B.rows, tri == kOzLower);
   if (tiles > (1 << 30)) return BQC_E_INVALID;
   p.tiles = (int)tiles;
   p.eA = A.exps;

@@ -57,12 +57,12 @@ inline int oz_splits(int K, int nsplit) {
 // Slices a source; exponents per row and split of split_kb k-blocks.
 int oz_slice(const OzSrc &src, int split_kb, void *slices, int *exps, cudaStream_t s);
 
-enum OzTri { kOzFull = 0, kOzLower = 1, kOzUpper = 2 };
+enum OzTri { kOzFull = 0, kOzLower = 1 };
 
 // out[split][n * ldo + m] = beta out + alpha sum_k A(m, k) B(n, k), m < A.rows,
 // n < B.rows, alpha = +-1, beta = 0 or 1; split covers split_kb k-blocks and
-// its result goes to out + split * split_stride.  tri (A.rows == B.rows): only
-// tiles that hold an element with n <= m (kOzLower) or n >= m (kOzUpper).
+// its result goes to out + split * split_stride.  kOzLower (A.rows == B.rows):
+// only tiles that hold an element with n <= m.
 int oz_gemm(const OzOperand &A, const OzOperand &B, int split_kb, int alpha, int beta, double *out,
             int64_t ldo, int64_t split_stride, int tri, int *flag, cudaStream_t s);
 
