@@ -302,7 +302,9 @@ int bqc_jk_grouped(int n, bqc_df *const *dfs, const double *const *C_dev, double
  * durations in ms.  Stored mode: [0] X pass (X = B C, with the fused w
  * contraction in FP64 and MIXED_TF32), [1] J (mixed builds: on a side stream,
  * overlapping [0] in MIXED_TF32X3 and [2] in MIXED_TF32), [2] K (SYRK and
- * its FP64 reduction), [3] operand preparation.  Direct mode: [0] first integral pass (integrals, gamma, X),
+ * its FP64 reduction), [3] operand preparation.  An FP64 build of at most 112
+ * functions does X, w and its parts of J and K in one kernel: [0] holds that
+ * kernel, [1] is 0 and [2] the final sums.  Direct mode: [0] first integral pass (integrals, gamma, X),
  * [1] metric solve and K, [2] second integral pass (J), [3] preparation.
  * BQC_E_NOT_READY if no timed call has been made. */
 int bqc_df_timing(bqc_df *df, int enable);

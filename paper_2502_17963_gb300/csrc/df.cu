@@ -706,9 +706,11 @@ static int jk_fp64_oz(Df *df, const OzJkPlan &p, const double *C, double *J, dou
     BQC_LAUNCH_CHECK();
     // K partials; a short last chunk may have fewer splits than the others, and
     // adds to the first ones
+    df->mark_k(s);
     BQC_TRY(oz_rows_of_x(X, n, no, np, ns, scr + p.xs, ints(p.xe), &ox, s));
     const int kb = oz_split_kb(ox.K, ns);
     BQC_TRY(oz_gemm(ox, ox, kb, 1, P0 > 0, kp, n, (int64_t)n * n, 1, df->ctx->flag, s));
+    df->mark_k(s);
   }
   df->mark(2, s);
   BQC_TRY(jpass_fp64(df, J, s));
@@ -1155,6 +1157,12 @@ int bqc_df_phase_ms(bqc_df *df, float *ms, int n) {
   } else {
     BQC_CUDA_TRY(cudaEventElapsedTime(&t[1], df->ev[2], df->ev[3]));
     BQC_CUDA_TRY(cudaEventElapsedTime(&t[2], df->ev[3], df->ev[4]));
+    for (int k = 0; k + 1 < df->kev_used; k += 2) {
+      float x = 0;
+      BQC_CUDA_TRY(cudaEventElapsedTime(&x, df->kev[k], df->kev[k + 1]));
+      t[0] -= x;
+      t[2] += x;
+    }
   }
   for (int i = 0; i < n && i < 4; ++i) ms[i] = t[i];
   return BQC_OK;
@@ -1167,6 +1175,7 @@ int bqc_jk(bqc_df *df, const double *C, int nocc, int prec, double *J, double *K
   NvtxRange nv(prec == BQC_PREC_FP64 ? "bqc_jk fp64" : "bqc_jk mixed");
   cudaStream_t s = (cudaStream_t)stream;
   if (df->timing) df->timed = true;
+  df->kev_used = 0;
   df->last_mixed = prec != BQC_PREC_FP64;
   if (df->mode == BQC_DF_DIRECT) return jk_direct(df, C, prec, J, K, s);
   if (df->mode == BQC_DF_NONE) return jk_4c(df, C, prec, J, K, s);

@@ -1,6 +1,7 @@
 // Internal state of a DF handle (stored or direct mode).
 #pragma once
 #include <memory>
+#include <vector>
 
 #include "bqc_internal.h"
 
@@ -74,6 +75,19 @@ struct Df {
   void mark(int i, cudaStream_t s) {
     if (timing && ev[i]) cudaEventRecord(ev[i], s);
   }
+  // K's part of each chunk of a sliced FP64 build, which alternates with the X
+  // pass: events 2 k and 2 k + 1 around chunk k's, the first kev_used recorded
+  std::vector<cudaEvent_t> kev;
+  int kev_used = 0;
+  void mark_k(cudaStream_t s) {
+    if (!timing) return;
+    if ((size_t)kev_used == kev.size()) {
+      cudaEvent_t e = nullptr;
+      if (cudaEventCreate(&e) != cudaSuccess) return;
+      kev.push_back(e);
+    }
+    cudaEventRecord(kev[kev_used++], s);
+  }
   // side stream of the mixed build: J runs there concurrently with the tensor-core passes
   cudaStream_t side = nullptr;
   cudaStream_t tcs = nullptr;  // tensor-core stream, one priority level above side
@@ -88,6 +102,7 @@ struct Df {
     if (gdone) cudaEventDestroy(gdone);
     for (auto &e : ev)
       if (e) cudaEventDestroy(e);
+    for (auto &e : kev) cudaEventDestroy(e);
     if (fork) cudaEventDestroy(fork);
     if (fork2) cudaEventDestroy(fork2);
     if (prep) cudaEventDestroy(prep);
