@@ -262,8 +262,10 @@ int jpass_fp64(Df *df, double *J, cudaStream_t s, int min_aux) {
   const int n = df->basis->nbf, naux = df->naux_loc;
   const int64_t npair = df->npair;
   if (!df->B64.p) return BQC_E_INVALID;
-  const int sp = jpass_split(npair, naux, min_aux);
-  if (df->Jp.n < (size_t)sp * npair * 8) return BQC_E_INVALID;
+  // as many chunks as there are slices for (AUTO mode may leave fewer)
+  const int sp = (int)std::min<size_t>(jpass_split(npair, naux, min_aux),
+                                       df->Jp.n / ((size_t)npair * 8));
+  if (sp < jpass_split(npair, naux)) return BQC_E_INVALID;
   k_jpass64<<<dim3((unsigned)((npair / 2 + 256) / 256), (unsigned)sp), 256, 0, s>>>(
       df->B64.as<double>(), df->w.as<double>(), naux, npair, df->Jp.as<double>());
   BQC_LAUNCH_CHECK();
@@ -878,8 +880,9 @@ size_t df_stored_bytes(int n, int naux, int nocc, int shadow) {
   const size_t npair = (size_t)n * (n + 1) / 2;
   size_t b = (size_t)naux * naux * 8 + (size_t)naux * npair * 8;  // L, B64
   b += (size_t)naux * n * nocc * 8;                                // X64
-  // (J partials of systems that fill the GPU; the few MB that smaller ones
-  // hold beyond this, and X's scratch, are among the caller's small buffers)
+  // (the X buffer's scratch, at most 32 MiB, and the J partials' further slices,
+  // at most 3 MB, come on top: AUTO mode takes them from what its limit leaves,
+  // serving from its allowance for small buffers)
   b += (size_t)jpass_split((int64_t)npair, naux) * npair * 8 + (size_t)naux * 8 * 2;
   if (shadow == BQC_SHADOW_TF32 || shadow == BQC_SHADOW_F16)
     b += mixed_workspace_bytes(n, naux, nocc, shadow);
@@ -915,7 +918,7 @@ int bqc_df_coulomb(bqc_df *df, const double *D_dev, double *J_dev, int variant,
   }
   BQC_CUDA_TRY(cudaSetDevice(df->ctx->device));
   if (df->D2.n < (size_t)df->npair * 8) BQC_TRY(df->D2.alloc(df->ctx, (size_t)df->npair * 8));
-  const int need = jpass_split(df->npair, df->naux_loc, kFp64JAux);
+  const int need = jpass_split(df->npair, df->naux_loc);
   if (df->Jp.n < (size_t)need * df->npair * 8)
     BQC_TRY(df->Jp.alloc(df->ctx, (size_t)need * df->npair * 8));
   cudaStream_t s = (cudaStream_t)stream;
@@ -942,6 +945,7 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
   const int n = basis->nbf, naux = basis->naux, no = basis->nocc;
   const int64_t npair = (int64_t)n * (n + 1) / 2;
   int mode = o.mode;
+  size_t room = SIZE_MAX;  // for scratch beyond df_stored_bytes
   if (mode == BQC_DF_AUTO) {
     size_t limit = o.hbm_limit;
     if (!limit) {
@@ -949,7 +953,9 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
       BQC_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
       limit = (size_t)(fr * 0.9);
     }
-    mode = df_stored_bytes(n, naux, no, o.keep_fp32) <= limit ? BQC_DF_STORED : BQC_DF_DIRECT;
+    const size_t need = df_stored_bytes(n, naux, no, o.keep_fp32);
+    mode = need <= limit ? BQC_DF_STORED : BQC_DF_DIRECT;
+    room = need <= limit ? limit - need : 0;
   }
   if (mode != BQC_DF_STORED && mode != BQC_DF_DIRECT && mode != BQC_DF_NONE) return BQC_E_INVALID;
   if (o.keep_fp32 < BQC_SHADOW_NONE || o.keep_fp32 > BQC_SHADOW_F16) return BQC_E_INVALID;
@@ -989,20 +995,6 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
     *out = df;
     return BQC_OK;
   }
-  // the FP64 X buffer (stored) or the raw block (direct), first used as the
-  // scratch of the factorisation and of the metric solve
-  DBuf &scr = mode == BQC_DF_STORED ? df->X64 : df->raw;
-  df->aux_block = std::max(1, std::min(o.aux_block, naux));
-  // direct mode: blocks of equal size (in multiples of 32, X's storage blocks;
-  // a block is padded to the largest), so that none is mostly padding and the
-  // one that the second integral pass finds in the buffer is no remainder
-  if (df->aux_block % 32 == 0 && naux > df->aux_block) {
-    const int nblk = (naux + df->aux_block - 1) / df->aux_block;
-    df->aux_block = std::min(df->aux_block, ((naux + nblk - 1) / nblk + 31) / 32 * 32);
-  }
-  if ((st = scr.alloc(ctx, mode == BQC_DF_STORED ? x64_bytes(n, df->naux_loc, no)
-                                                 : (size_t)df->aux_block * npair * 8)) != BQC_OK)
-    return fail(st);
   // metric and its Cholesky factor
   if ((st = df->L.alloc(ctx, (size_t)naux * naux * 8)) != BQC_OK) return fail(st);
   if ((st = launch_int2c(basis, df->L.as<double>(), s)) != BQC_OK) return fail(st);
@@ -1026,9 +1018,13 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
     // (H2O)_12: 4e-9, against 1e-12).  What it costs: set-up of (H2O)_24 with FP16
     // shadows 570 ms, with the sliced solve 77.
     const bool sliced = o.keep_fp32 == BQC_SHADOW_NONE;
-    void *const sp = sliced ? df->X64.p : nullptr;
-    const size_t sn = sliced ? df->X64.n : 0;
+    // the FP64 X buffer, first the scratch of the sliced solve
+    const int nl = df->naux_loc;
+    const size_t x = (size_t)nl * n * no * 8;
+    const size_t xs = x + std::min(room, x64_bytes(n, nl, no) - x);
+    room -= xs - x;
     if (!shard) {
+      if ((st = df->X64.alloc(ctx, xs)) != BQC_OK) return fail(st);
       if ((st = df->B64.alloc(ctx, (size_t)naux * npair * 8)) != BQC_OK) return fail(st);
       if (cudaMemsetAsync(df->B64.p, 0, (size_t)naux * npair * 8, s) != cudaSuccess)
         return fail(BQC_E_CUDA);
@@ -1036,12 +1032,14 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
           BQC_OK)
         return fail(st);
       if ((st = trsm_lower_left(ctx, df->L.as<double>(), naux, df->B64.as<double>(), npair,
-                                npair, sp, sn, s)) != BQC_OK)
+                                npair, sliced ? df->X64.p : nullptr, sliced ? df->X64.n : 0,
+                                s)) != BQC_OK)
         return fail(st);
     } else {
       // B_P for P in [P0, P1) depends on (Q|mu nu) for every Q <= P (the
       // triangular solve couples them): solve rows [0, P1) with the leading
-      // P1 x P1 block of L and keep the shard's rows
+      // P1 x P1 block of L and keep the shard's rows (raw is the largest array
+      // of the build: the scratch beside it is given back before B is allocated)
       DBuf raw, Lb;
       if ((st = raw.alloc(ctx, (size_t)P1 * npair * 8)) != BQC_OK) return fail(st);
       if (cudaMemsetAsync(raw.p, 0, (size_t)P1 * npair * 8, s) != cudaSuccess)
@@ -1052,9 +1050,12 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
       if (cudaMemcpy2DAsync(Lb.p, (size_t)P1 * 8, df->L.p, (size_t)naux * 8, (size_t)P1 * 8, P1,
                             cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return fail(BQC_E_CUDA);
+      if (sliced && df->X64.alloc(ctx, xs) != BQC_OK) df->X64.release();
       if ((st = trsm_lower_left(ctx, Lb.as<double>(), P1, raw.as<double>(), npair, npair,
-                                sp, sn, s)) != BQC_OK)
+                                df->X64.p, df->X64.n, s)) != BQC_OK)
         return fail(st);
+      if (cudaStreamSynchronize(s) != cudaSuccess) return fail(BQC_E_CUDA);
+      df->X64.release();
       if ((st = df->B64.alloc(ctx, (size_t)(P1 - P0) * npair * 8)) != BQC_OK) return fail(st);
       if (cudaMemcpyAsync(df->B64.p, raw.as<double>() + (size_t)P0 * npair,
                           (size_t)(P1 - P0) * npair * 8, cudaMemcpyDeviceToDevice,
@@ -1062,9 +1063,10 @@ int bqc_df_build(bqc_ctx *ctx, const bqc_basis *basis, const bqc_df_opts *opts,
         return fail(BQC_E_CUDA);
       if (cudaStreamSynchronize(s) != cudaSuccess) return fail(BQC_E_CUDA);
     }
-    const int nl = df->naux_loc;
-    if ((st = df->Jp.alloc(ctx, (size_t)jpass_split(npair, nl, kFp64JAux) * npair * 8)) != BQC_OK)
-      return fail(st);
+    if (!df->X64.p && (st = df->X64.alloc(ctx, xs)) != BQC_OK) return fail(st);
+    const int jmin = jpass_split(npair, nl), jmax = jpass_split(npair, nl, kFp64JAux);
+    const int js = jmin + (int)std::min<size_t>(jmax - jmin, room / ((size_t)npair * 8));
+    if ((st = df->Jp.alloc(ctx, (size_t)js * npair * 8)) != BQC_OK) return fail(st);
     if (o.keep_fp32 != BQC_SHADOW_NONE)
       if ((st = mixed_setup(df, o.keep_fp32, s)) != BQC_OK) return fail(st);
   } else {

@@ -115,6 +115,15 @@ int direct_setup(Df *df, cudaStream_t s) {
   BQC_LAUNCH_CHECK();
   BQC_TRY(trsm_lower_left(ctx, df->L.as<double>(), naux, df->Linv.as<double>(), naux, naux,
                           nullptr, 0, s));
+  df->aux_block = std::max(1, std::min(df->opts.aux_block, naux));
+  // blocks of equal size (in multiples of 32, X's storage blocks; a block is
+  // padded to the largest), so that none is mostly padding and the one that the
+  // second integral pass finds in the buffer is no remainder
+  if (df->aux_block % 32 == 0 && naux > df->aux_block) {
+    const int nblk = (naux + df->aux_block - 1) / df->aux_block;
+    df->aux_block = std::min(df->aux_block, ((naux + nblk - 1) / nblk + 31) / 32 * 32);
+  }
+  BQC_TRY(df->raw.alloc(ctx, (size_t)df->aux_block * df->npair * 8));
   BQC_TRY(df->gamma.alloc(ctx, (size_t)naux * 8 * 2));
   BQC_TRY(df->D2.alloc(ctx, (size_t)df->npair * 8));
   BQC_TRY(df->Jp.alloc(ctx, (size_t)df->npair * 8));

@@ -182,7 +182,11 @@ size_t serve_footprint(int n, int naux, int nocc, int shadow) {
   b += (size_t)naux * naux * 8;             // metric copy during the build
   b += (size_t)(16 + 2 * 8) * nn * 8;       // SCF matrices + DIIS history
   b += (size_t)3 * n * n / 2 * 16;          // shell-pair plan (generous)
-  b += (size_t)64 << 20;                    // Boys table, small buffers, alignment
+  // Boys table, alignment and small buffers: X's scratch beyond df_stored_bytes
+  // (at most 32 MiB, and 0 from about 20 waters on), J's further slices (3 MB), the
+  // slices (12 MB at 640 functions) and refined eigenvectors (5 MB at 320) of the
+  // SCF, library workspaces
+  b += (size_t)64 << 20;
   return b;
 }
 

@@ -1923,7 +1923,7 @@ static int mixed_setup_f16(Df *df, MixedState *ms, cudaStream_t s) {
       slices += jpass_split(df->npair, (int)((int64_t)naux * (k + 1) / np) -
                                            (int)((int64_t)naux * k / np));
     const size_t need =
-        (size_t)std::max(jpass_split(df->npair, naux, kFp64JAux), slices) * df->npair * 8;
+        (size_t)std::max(jpass_split(df->npair, naux), slices) * df->npair * 8;
     if (df->Jp.n < need) BQC_TRY(df->Jp.alloc(ctx, need));
   }
   BQC_TRY(ms->Xh16.alloc(ctx, (size_t)naux * n * m.ldx * 2));
