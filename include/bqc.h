@@ -58,7 +58,20 @@ enum {
 };
 
 /* Precision of the Fock build (the X = B C and K contractions, the B.D
- * products).  FP64: all FP64 (DFMA).  MIXED_TF32: tcgen05 kind::tf32 MMAs on
+ * products).  FP64: FP64 throughout.  Up to 112 functions (as far as B_P, C and
+ * X_P fit in shared memory) X and K are DFMA chains; above, they are assembled
+ * from exact FP16 slices on the tensor cores.  A slice set keeps an operand
+ * element to 2^-56 of a power of two that bounds its row's elements (at most
+ * twice the largest): the product of rows a and b over k terms is off by at most
+ * k 2^-53 max|a| max|b|, plus the result's own rounding.  On rows of even size
+ * the norm of a product's error is below DFMA's (6e-17 of the result's norm
+ * against 9e-16), and B, J, K, F and E2 of the (H2O)_n workloads are as near to
+ * 64-bit references as DFMA's.  But the bound does not shrink with the single
+ * terms as DFMA's does: a product of rows that are large where the other is small
+ * (localised orbitals far apart), or whose few large elements do not enter it,
+ * keeps fewer than 53 significant bits (rows spread log-normally over e^(+-3):
+ * 6e-15 of the norm against 7e-16).  bqc_jk_fp64_noalloc is DFMA throughout.
+ * MIXED_TF32: tcgen05 kind::tf32 MMAs on
  * TF32-rounded B and C_occ (one product per term, ~2^-11 relative per
  * product), FP32 accumulation in short chains, FP64 chunk sums; J from the
  * TF32 shadow of B.  MIXED_TF32X3: K the same with every operand split
@@ -320,13 +333,15 @@ int bqc_df_phase_ms(bqc_df *df, float *ms, int n);
  * df: a stored-mode handle.  C_dev: N x nmo row-major canonical orbitals
  * (columns; the first nocc occupied, the rest virtual), eps_dev: their nmo
  * orbital energies (bqc_scf_run's C_dev / eps_dev outputs have this layout).
- * prec: BQC_PREC_FP64 (every GEMM on the DFMA path) or BQC_PREC_MIXED_F16X3
- * (the MO transform in FP64, the (ia|jb) blocks as split-FP16 tensor-core
- * GEMMs with FP32 accumulation in short chains and FP64 blocks, ~2^-22
- * relative per integral); other precisions BQC_E_UNSUPPORTED.
+ * prec: BQC_PREC_FP64 (transform and blocks in FP64: sliced products above 64
+ * functions, with the row-wise bound given at bqc_prec, DFMA up to 64) or
+ * BQC_PREC_MIXED_F16X3 (the MO transform in FP64, the (ia|jb) blocks as
+ * split-FP16 tensor-core GEMMs with FP32 accumulation in short chains and FP64
+ * blocks, ~2^-22 relative per integral); other precisions BQC_E_UNSUPPORTED.
  * Writes *e2 (host).  Allocates its working memory from the context
- * (Naux * nocc * nvir doubles and a block of (ia|jb) of at most 1 GiB) and
- * synchronises the stream; reuses the handle's X buffer, so it must not
+ * (Naux * nocc * nvir doubles, a block of (ia|jb) of at most 1 GiB, and where
+ * sliced products run 14 bytes for each element of the former; without memory
+ * for these the DFMA GEMM) and synchronises the stream; reuses the handle's X buffer, so it must not
  * overlap a bqc_jk on the same handle. */
 int bqc_mp2(bqc_df *df, const double *C_dev, const double *eps_dev, int nmo, int prec,
             double *e2, bqc_stream_t stream);
@@ -426,6 +441,16 @@ enum { BQC_SWITCH_NONE = 0, BQC_SWITCH_STAGE_TOL = 1, BQC_SWITCH_FLOOR = 2 };
  * in *out is written. */
 int bqc_scf_run(bqc_ctx *ctx, bqc_df *df, const bqc_scf_opts *opts, bqc_stream_t stream,
                 bqc_scf_result *out);
+
+/* The FP64 products from exact FP16 slices that FP64 builds, the metric solve
+ * and MP2 use (their error: see bqc_prec), exposed for testing: with A_dev
+ * (m x k) and B_dev (n x k) row-major, slab q < splits of C_dev (splits x n x m)
+ * gets sum A[i][l] B[j][l] at [j][i] over the q-th part of the contraction
+ * (parts are multiples of 32; slabs past the last stay zero); lower != 0 (m = n)
+ * leaves 128 x 64 tiles without an element j <= i out.  Allocates the slices,
+ * synchronises the stream. */
+int bqc_gemm_sliced(bqc_ctx *ctx, int m, int n, int k, const double *A_dev, const double *B_dev,
+                    int splits, int lower, double *C_dev, bqc_stream_t stream);
 
 /* Symmetric eigen-decomposition of the SCF's FP64 stage (up to 320 functions an
  * FP32 decomposition refined to FP64 by products, cuSOLVER's FP64 one above and

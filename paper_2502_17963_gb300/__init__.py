@@ -148,6 +148,7 @@ _SIGS = {
                             ctypes.POINTER(vp), vp]),
     "bqc_df_coulomb": (ip, [vp, vp, vp, ip, vp]),
     "bqc_ctx_multicast": (ip, [vp]),
+    "bqc_gemm_sliced": (ip, [vp, ip, ip, ip, vp, vp, ip, ip, vp, vp]),
     "bqc_eigh": (ip, [vp, ip, vp, vp, ctypes.POINTER(ctypes.c_int), vp]),
     "bqc_wait_selftest": (ip, [vp, ctypes.c_longlong, vp]),
     "bqc_mp2": (ip, [vp, vp, vp, ip, ip, ctypes.POINTER(ctypes.c_double), vp]),
@@ -482,6 +483,17 @@ def scf_run(ctx: Context, df: DF, prec: int = PREC_FP64, diis_tol: float = 1e-8,
     if keep_arrays:
         out.update(C=Cbuf[: n * r.nmo].view(n, r.nmo), eps=eps[: r.nmo], F=F)
     return out
+
+
+def gemm_sliced(ctx: Context, A, B, splits: int = 1, lower: bool = False, stream=None):
+    """(splits, n, m) partial products B A^T of FP64 device matrices A (m x k) and
+    B (n x k), one slab per part of the contraction (bqc_gemm_sliced)."""
+    A, B = A.contiguous(), B.contiguous()
+    C = _empty((splits, B.shape[0], A.shape[0]))
+    check(lib().bqc_gemm_sliced(ctx.h, A.shape[0], B.shape[0], A.shape[1], _ptr(A), _ptr(B),
+                                splits, 1 if lower else 0, _ptr(C), _stream_ptr(stream)),
+          "bqc_gemm_sliced")
+    return C
 
 
 def eigh(ctx: Context, A, stream=None):

@@ -17,8 +17,10 @@
 //    contraction elements: at most 7 * 128 * 2^14 < 2^24, so every FP32
 //    partial sum is an exact integer and the tensor core's truncation has
 //    nothing to truncate.  Levels 8 and up (below 2^-64 of the row bounds'
-//    product times about 5 K) are left out, which keeps the result closer to
-//    the exact one than a DFMA chain is.
+//    product times about 5 K) are left out.  For rows of even size the result is
+//    closer to the exact one than a DFMA chain's; the bound is one of the rows,
+//    not of the terms (rows spread log-normally over e^(+-3): 5.6e-15 of the
+//    norm, DFMA 7.4e-16).
 //  * Chains are drained into two 64-bit integers per element (levels 0-3 and
 //    4-7, one IMAD.WIDE per level), exact for up to 2^15 chains, and turned
 //    into FP64 once per tile with integer arithmetic (the FP64 pipe would
@@ -29,13 +31,14 @@
 // 32: 14 slices of a k-block (84 KB) arrive as two TMA boxes and feed 34 x 2
 // MMAs, so shared-memory reads (6 KB an MMA, 48 clocks where the arithmetic takes
 // 32; measured) and not the load path bound the main loop: multicasting an
-// operand tile to CTA pairs changed nothing.  30000 x 900 x 900: 31.6 TFLOP/s of
-// FP64 product (1075 of FP16 issued, 0.55 of the measured 1942; DFMA 1.2), error
-// 5.9e-17 of the result's norm against DFMA's 9.2e-16; 60000 x 64 x 64, where
-// the drain and the conversion of a tile take as long as its MMAs, about 8.  The accumulators are single-buffered: a level is
-// handed over as soon as its last MMA of the chain is issued, the MMAs of a
-// k-block run level by level, and so the eight epilogue warps drain level d
-// while levels d + 1 ... and the next chain's first levels are computed.
+// operand tile to CTA pairs changed nothing.  30000 x 900 x 900: 30 to 31.6
+// TFLOP/s of FP64 product (1031 to 1075 of FP16 issued, 0.53 to 0.55 of the
+// measured 1942; DFMA 1.2), error of normal deviates 5.9e-17 of the result's norm
+// against DFMA's 9.2e-16; 60000 x 64 x 64, where the drain and the conversion of a
+// tile take as long as its MMAs, about 8.  The accumulators are single-buffered: a
+// level is handed over as soon as its last MMA of the chain is issued, the MMAs of
+// a k-block run level by level, and so the eight epilogue warps drain level d while
+// levels d + 1 ... and the next chain's first levels are computed.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -490,3 +493,37 @@ int oz_sym_reduce(const double *part, int nsplit, int64_t split_stride, int n, i
 }
 
 }  // namespace bqc
+
+using namespace bqc;
+
+extern "C" int bqc_gemm_sliced(bqc_ctx *ctx, int m, int n, int k, const double *A_dev,
+                               const double *B_dev, int splits, int lower, double *C_dev,
+                               bqc_stream_t stream) {
+  if (!ctx || m < 1 || n < 1 || k < 1 || !A_dev || !B_dev || !C_dev || splits < 1 ||
+      splits > 65535 || (lower && m != n))
+    return BQC_E_INVALID;
+  BQC_CUDA_TRY(cudaSetDevice(ctx->device));
+  cudaStream_t s = (cudaStream_t)stream;
+  const int ns = oz_splits(k, splits), kb = oz_split_kb(k, splits);
+  DBuf buf[2];
+  OzOperand o[2];
+  StreamGuard guard{s};
+  BQC_CUDA_TRY(cudaMemsetAsync(C_dev, 0, (size_t)splits * m * n * 8, s));
+  for (int q = 0; q < 2; ++q) {
+    OzSrc x;
+    x.p = q ? B_dev : A_dev;
+    x.rows = q ? n : m;
+    x.K = k;
+    x.ld = k;
+    BQC_TRY(buf[q].alloc(ctx, oz_slice_bytes(x.rows, k) + oz_exp_bytes(x.rows, ns)));
+    o[q].slices = buf[q].p;
+    int *e = reinterpret_cast<int *>(buf[q].as<char>() + oz_slice_bytes(x.rows, k));
+    o[q].exps = e;
+    o[q].rows = x.rows;
+    o[q].K = k;
+    BQC_TRY(oz_slice(x, kb, buf[q].p, e, s));
+  }
+  BQC_TRY(oz_gemm(o[0], o[1], kb, 1, 0, C_dev, m, (int64_t)m * n, lower ? kOzLower : kOzFull,
+                  ctx->flag, s));
+  return ctx->check_flag(s);
+}
