@@ -555,7 +555,7 @@ def run_screen_ablation(args):
 def mp2_roofline(transform_flops, pair_flops, dt, n, fp64, pk, pk_src):
     """Roofline entry of one DF-MP2 energy of dt seconds, transform and pair blocks
     together.  FP64 products are assembled from 34 FP16 ones (the transform in
-    both precisions above 112 functions, the FP64 pair blocks above 64); a
+    FP64 above 64 functions and in split FP16 above 80, the FP64 pair blocks above 64); a
     split-FP16 pair block issues 3.  Up to 64 functions everything in FP64 runs on
     the DFMA pipe."""
     flops = transform_flops + pair_flops
@@ -566,7 +566,7 @@ def mp2_roofline(transform_flops, pair_flops, dt, n, fp64, pk, pk_src):
                 "peak_source": "FP64: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz",
                 "algorithmic_flop": flops}
     sust = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
-    sliced = n > (64 if fp64 else 112)  # the transform; else it is on the DFMA pipe
+    sliced = n > (64 if fp64 else 80)  # the transform; else it is on the DFMA pipe
     issued = (34 if sliced else 0) * transform_flops + (34 if fp64 else 3) * pair_flops
     return {"bound": "tensor",
             "kernel": "k_oz_gemm (34 FP16 products per FP64 product)" if fp64 else

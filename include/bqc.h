@@ -335,8 +335,8 @@ int bqc_df_phase_ms(bqc_df *df, float *ms, int n);
  * orbital energies (bqc_scf_run's C_dev / eps_dev outputs have this layout).
  * prec: BQC_PREC_FP64 (transform and blocks in FP64: sliced products above 64
  * functions, with the row-wise bound given at bqc_prec, DFMA up to 64) or
- * BQC_PREC_MIXED_F16X3 (the MO transform in FP64, the (ia|jb) blocks as
- * split-FP16 tensor-core GEMMs with FP32 accumulation in short chains and FP64
+ * BQC_PREC_MIXED_F16X3 (the MO transform in FP64, sliced above 80 functions, the
+ * (ia|jb) blocks as split-FP16 tensor-core GEMMs with FP32 accumulation in short chains and FP64
  * blocks, ~2^-22 relative per integral); other precisions BQC_E_UNSUPPORTED.
  * Writes *e2 (host).  Allocates its working memory from the context
  * (Naux * nocc * nvir doubles, a block of (ia|jb) of at most 1 GiB, and where

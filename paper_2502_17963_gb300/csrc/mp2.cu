@@ -223,8 +223,12 @@ static int mp2_transform_oz(Df *df, const double *C, int nmo, double *Bt, char *
 // prec FP64: the transform and the pair blocks V = B_ia^T B_jb as sliced
 // FP64-accurate tensor-core products; MIXED_F16X3: the pair blocks as
 // split-FP16 tensor-core GEMMs (FP32 accumulation in short chains, float-float
-// drains, FP64 blocks); the energy in FP64.  Without memory for the slices,
-// or up to 64 functions, where a tile would be mostly padding, the DFMA GEMM.
+// drains, FP64 blocks); the energy in FP64.  Without memory for the slices the
+// DFMA GEMM, and for few functions, where a tile is mostly padding: in FP64 up
+// to 64 (whole energy, N = 75: 614 us sliced, 1000 DFMA; 100: 820 and 2634), in
+// MIXED_F16X3, where only the transform is at stake, up to 80 (75: 672 us with the
+// sliced transform, 585 without; 100: 838 and 1227).
+constexpr int kMp2DfmaMax = 64, kMp2DfmaMaxF16 = 80;
 static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec, double *e2,
                    cudaStream_t s) {
   const Basis *b = df->basis;
@@ -241,7 +245,8 @@ static int mp2_run(Df *df, const double *C, const double *eps, int nmo, int prec
     BQC_TRY(Bt.alloc(ctx, (size_t)naux * Q * 8));
     const int bi = mp2_block(no, nv);
     int pc = 0;
-    if (n > (prec == BQC_PREC_FP64 ? 64 : 112) && Ts.alloc(ctx, oz_slice_bytes(Q, naux) + oz_exp_bytes(Q, 1)) == BQC_OK)
+    if (n > (prec == BQC_PREC_FP64 ? kMp2DfmaMax : kMp2DfmaMaxF16) &&
+        Ts.alloc(ctx, oz_slice_bytes(Q, naux) + oz_exp_bytes(Q, 1)) == BQC_OK)
       pc = mp2_transform_pc(n, naux, no, nv, Ts.n);
     bool oz = prec == BQC_PREC_FP64 && Ts.p;
     if (pc)

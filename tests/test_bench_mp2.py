@@ -27,5 +27,5 @@ def test_mp2_roofline_is_a_share(waters, fp64, seconds, unit):
     assert r["algorithmic_flop"] == transform + pair
     if unit == "tensor":
         assert r["frac"] < r["frac_issued"] < 1
-        issued = (34 if n > 112 else 0) * transform + (34 if fp64 else 3) * pair
+        issued = (34 if n > 80 else 0) * transform + (34 if fp64 else 3) * pair
         assert r["issued_tensor_flop"] == issued
