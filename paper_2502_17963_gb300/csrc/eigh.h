@@ -8,11 +8,11 @@
 namespace bqc {
 
 // Largest orders served.  Products: above 640 the SCF's work matrices are large
-// enough that the slices would count.  The refined decomposition wins at every
-// size measured (600: 6.5 ms of FP32 syevd and about 2 of refinement against
-// 19), but a solve of 400 functions in FP64 would end within the 0.3 s after
-// which tests/test_gpu_serve.py cancels it and expects to find it running, so
-// it stays at the sizes where the library call dominates a solve.
+// enough that the slices would count.  The refined decomposition is tested up to
+// 320 (tests/test_gpu_eigh.py); it also wins above (600: 6.5 ms of FP32 syevd and
+// about 2 of refinement against 19), where the FP64 call stays: with it taken, an
+// FP64 solve of 400 functions ends within the 0.3 s after which
+// tests/test_gpu_serve.py expects to find it running.
 constexpr int kSmallGemmMax = 640;
 constexpr int kEighRefineMax = 320;
 

@@ -4,10 +4,11 @@
 // Sec. 2.2.
 //
 // On GB300 FP64 runs at ~1.2 TFLOP/s (about 2 DFMA per clock per SM, a quarter
-// of that for a lone warp), so the products of both run as sliced FP16 products
-// on the tensor cores (oz.cu) when the caller has scratch for the slices; the
-// 64x64 register-blocked DFMA GEMM (gemm64.cuh) serves without it.  Set-up of
-// (H2O)_24 (Naux = 1800): 575 ms on the DFMA pipe, about 60 ms so.
+// of that for a lone warp).  The factorisation (Naux^3 / 3) runs there; the
+// solve's products run as sliced FP16 products on the tensor cores (oz.cu) where
+// the caller gives scratch for the slices, which a handle without split shadows
+// does, and on the 64x64 register-blocked DFMA GEMM (gemm64.cuh) elsewhere.
+// Set-up of (H2O)_24 (Naux = 1800): 73 ms sliced, 570 on the DFMA pipe.
 #include <cuda_runtime.h>
 
 #include <algorithm>
